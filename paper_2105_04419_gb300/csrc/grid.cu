@@ -1384,6 +1384,7 @@ __global__ void __launch_bounds__(256) k_items_nodes(VS vs, int rx, int ry, int 
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
   if (vs.skip(g)) return;
+  if (bid == 0 && threadIdx.x == 0) g.counters[C_FORM] = g.half ? kFormHalf : kFormInt;  // what the passes will store
   __shared__ int wsum[8];
   __shared__ int base_sh, count_sh;
   __shared__ int nbr_sh[2];

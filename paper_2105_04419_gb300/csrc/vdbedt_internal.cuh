@@ -63,13 +63,15 @@ enum Counter : int {
   C_OBST = 12,
   C_NB_START = 13,  // stored bricks when the running update began (its global-vs-incremental choice)
   C_EPOCH = 14,  // incremental update epoch (run and brick dedupe marks)
-  C_SPARE = 15,  // unused
+  C_FORM = 15,  // encoding of the g1 / g2 fields as stored (kForm*; 0: none yet), written by each global form
   C_XB = 16,  // stored bricks in the update's dirty runs per axis (x, y, z: three consecutive words)
   C_YB = 17,
   C_ZB = 18,
   C_BIG = 19,  // this update's edits reach so far that it takes the global form after applying them
   C_NUM = 20
 };
+
+constexpr int kFormHalf = 1, kFormInt = 2;  // fp16 bit patterns; 16-bit integers
 
 // brick flags
 constexpr uint32_t F_OBST = 1u;    // holds an occupied voxel
