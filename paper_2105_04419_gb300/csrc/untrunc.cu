@@ -5,8 +5,10 @@
 // over whole lines of the grid, one axis after the other (Eq. 1's minimum taken per axis):
 //   x: per row, the distance to the nearest occupied voxel on either side (a forward sweep that
 //      keeps one carry per brick, and a backward sweep that writes g1 = dx^2);
-//   y, z: per line, the lower envelope of the parabolas f(i) + (t - i)^2 rooted at the line's
-//      finite values (g1, then g2): built on a stack in one sweep, read back in a second.  Two
+//   y, z: per line, the minimum over i of f(i) + (t - i)^2 (f: g1, then g2).  Lines of up to kLineMax
+//      positions are staged whole in shared memory (k_ut_line, by the bracketed minima of
+//      line_min.cuh).  Longer ones: the lower envelope of the parabolas rooted at the line's
+//      finite values, built on a stack in one sweep, read back in a second.  Two
 //      parabolas are compared through their intersection with the denominators multiplied out,
 //      exactly: the grid's size limit keeps every f(p) + p^2 below 2^31, so the differences are
 //      int32 and each product one widening multiply (below 2^48).
@@ -14,6 +16,7 @@
 // written; g1 and g2 hold int32 here (their arrays are allocated twice as large).
 #include <algorithm>
 
+#include "line_min.cuh"
 #include "vdbedt_internal.cuh"
 
 namespace vdbedt {
@@ -26,6 +29,8 @@ __device__ __forceinline__ int ut_slot(const GridView& g, int bx, int by, int bz
 }
 
 __device__ __forceinline__ int ut_vox(int x, int y, int z) { return (x & 7) + 8 * (y & 7) + 64 * (z & 7); }
+// g1 is stored y-major, so that the y pass reads planes
+__device__ __forceinline__ int ut_vox_g1(int x, int y, int z) { return (x & 7) + 8 * (z & 7) + 64 * (y & 7); }
 
 // A line's stack in the scratch, interleaved with the other 31 lines of its group of 32 (entry m
 // of line t at ((t >> 5) n + m) 32 + (t & 31)): lanes of a warp that push or pop at similar depths
@@ -145,7 +150,7 @@ __global__ void k_ut_x(GridView g, int32_t* __restrict__ carry) {
     const int y = 8 * by + (q & 7), z = 8 * bz + (q >> 3);
     if (y >= g.ny || z >= g.nz) continue;
     const int shift = 8 * (y & 7);
-    const size_t row = (size_t)(8 * (y & 7) + 64 * (z & 7));
+    const size_t row = (size_t)ut_vox_g1(0, y, z);
     int last = -1;
     for (int bx = 0; bx < g.BX; ++bx) {
       carry[(size_t)bx * nrows + t] = last;
@@ -193,17 +198,18 @@ __global__ void k_ut_x(GridView g, int32_t* __restrict__ carry) {
 }
 
 // Voxel i of line (x, c) along AXIS (1: y, c = z; 2: z, c = y) in a pool of bricks at fixed slots:
-// base + (i >> 3) * brick stride + (i & 7) * voxel stride.
-template <int AXIS>
+// base + (i >> 3) * brick stride + (i & 7) * voxel stride.  IN: of the pass's input field (planes along
+// the axis), else of its output.
+template <int AXIS, bool IN>
 struct LineAt {
   size_t base, bstride;
   __device__ __forceinline__ LineAt(const GridView& g, int x, int c) {
-    base = AXIS == 1 ? (size_t)ut_slot(g, x >> 3, 0, c >> 3) * kBrickVox + ut_vox(x, 0, c)
+    base = AXIS == 1 ? (size_t)ut_slot(g, x >> 3, 0, c >> 3) * kBrickVox + (IN ? ut_vox_g1(x, 0, c) : ut_vox(x, 0, c))
                      : (size_t)ut_slot(g, x >> 3, c >> 3, 0) * kBrickVox + ut_vox(x, c, 0);
     bstride = (size_t)kBrickVox * (AXIS == 1 ? g.BX : (size_t)g.BX * g.BY);
   }
   __device__ __forceinline__ size_t operator()(int i) const {
-    return base + (size_t)(i >> 3) * bstride + (size_t)((i & 7) * (AXIS == 1 ? 8 : 64));
+    return base + (size_t)(i >> 3) * bstride + (size_t)((i & 7) * (AXIS == 1 && !IN ? 8 : 64));
   }
 };
 
@@ -213,7 +219,7 @@ struct LineAt {
 // widening 32 x 32 -> 64-bit products exactly.  The inputs are loaded a brick (8 positions) at a
 // time, all eight before any is used.  Returns the entry count.
 template <int AXIS>
-__device__ __forceinline__ int env_build(const LineStack& st, const LineAt<AXIS>& at, const int32_t* __restrict__ in,
+__device__ __forceinline__ int env_build(const LineStack& st, const LineAt<AXIS, true>& at, const int32_t* __restrict__ in,
                                          int n) {
   int m = 0, p0 = 0, F0 = 0, p1 = 0, F1 = 0;
   for (int i0 = 0; i0 < n; i0 += 8) {
@@ -287,10 +293,11 @@ __global__ void k_ut_env(GridView g, const int32_t* __restrict__ in, int32_t* __
   const int64_t nlines = (int64_t)g.nx * (AXIS == 1 ? g.nz : g.ny);
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nlines; t += (int64_t)gridDim.x * blockDim.x) {
     const int x = (int)(t % g.nx), c = (int)(t / g.nx);  // c: z (AXIS 1) or y (AXIS 2)
-    const LineAt<AXIS> at(g, x, c);
+    const LineAt<AXIS, true> at(g, x, c);
+    const LineAt<AXIS, false> to(g, x, c);
     const LineStack st(stack, t, n);
     EnvRead env(st, env_build<AXIS>(st, at, in, n));
-    for (int i = 0; i < n; ++i) out[at(i)] = env.at(i);
+    for (int i = 0; i < n; ++i) out[to(i)] = env.at(i);
   }
 }
 
@@ -318,12 +325,13 @@ __global__ void k_ut_env_upd(GridView g, const int32_t* __restrict__ in, int32_t
     const bool dirty = (w >> lane) & 1u;  // set only for x < nx
     if (!dirty) continue;
     const int x = (int)(t % nxp), c = (int)(t / nxp);  // c: z (AXIS 1) or y (AXIS 2)
-    const LineAt<AXIS> at(g, x, c);
+    const LineAt<AXIS, true> at(g, x, c);
+    const LineAt<AXIS, false> to(g, x, c);
     const LineStack st(stack, t, n);
     EnvRead env(st, env_build<AXIS>(st, at, in, n));
     for (int i = 0; i < n; ++i) {
       const int val = env.at(i);
-      const size_t a = at(i);
+      const size_t a = to(i);
       if (AXIS == 1) {
         if (out[a] != val) {
           out[a] = val;
@@ -350,6 +358,127 @@ __global__ void k_ut_flags(GridView g) {
   }
 }
 
+// y (AXIS 1: g1 -> g2) or z (AXIS 2: g2 -> D) pass of lines that fit shared memory: a block per tile of
+// 32 lines (8 along x times 4 across; half of a brick column), staged whole as planes of 32 words, then
+// the bracketed minima of line_min.cuh, each warp on its own bricks.  Missing inputs (kNone, and the
+// ragged end of the line) stay the largest candidates: kNone + d^2 is at least kNone and fits 32 bits.
+// UPD (an update): only the lines of the tile whose dirty byte is set (cleared once read); the y pass
+// writes the g2 values that changed and sets the z-line byte of each.
+// Bound by issue (searches and candidates, about 40 instructions a voxel) with 8 B of memory traffic a
+// voxel under it.  512 x 512 x 256 tunnel scene: y 0.24 ms, z 0.21 ms (the stack kernels 0.58 and 0.66;
+// memory alone would take 0.08); dirty lines of its first lidar frames 0.19 and 0.18 ms (0.42 and 0.26).
+// kLineMax is what shared memory holds: 152 B a position with minima and arguments, of 227 KB.
+constexpr int kLineMax = 1496;
+__host__ __device__ inline int line_bricks(int n) { return (n + 7) >> 3; }
+__host__ __device__ inline size_t line_smem(int n) {
+  const size_t nb = (size_t)line_bricks(n);
+  return nb * 8 * 128 + nb * 128 + (nb + 1) * 64;
+}
+
+template <int AXIS, bool UPD>
+__global__ void k_ut_line(GridView g, const int32_t* __restrict__ in, int32_t* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int n = AXIS == 1 ? g.ny : g.nz, nb = line_bricks(n), nc = AXIS == 1 ? g.nz : g.ny;
+  uint32_t* val = reinterpret_cast<uint32_t*>(smem);               // [8 nb][32]
+  uint32_t* bmin = val + (size_t)nb * 256;                         // [nb][32]
+  uint16_t* args = reinterpret_cast<uint16_t*>(bmin + nb * 32);    // [nb + 1][32]
+  __shared__ uint32_t lmin[32];                                    // the lines' minima
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  // tile: brick column (bx, bc), lines c = 8 bc + 4 h + (lane >> 3)
+  const int h = (int)(blockIdx.x & 1), bx = (int)((blockIdx.x >> 1) % g.BX), bc = (int)((blockIdx.x >> 1) / g.BX);
+  const int x = 8 * bx + (lane & 7), c = 8 * bc + 4 * h + (lane >> 3);
+  bool live = x < g.nx && c < nc;
+  if (UPD) {
+    uint8_t* flag = reinterpret_cast<uint8_t*>(g.ut_bits + ut_row_words(g) + (AXIS == 1 ? 0 : ut_yline_words(g)));
+    const size_t fi = (size_t)ut_nxp(g) * c + x;
+    live = live && flag[fi] != 0;
+    const unsigned dirty = __ballot_sync(0xffffffffu, live);
+    if (!dirty) return;  // block-uniform: every warp read the same 32 bytes
+    __syncthreads();     // all of them, before they are cleared
+    if (warp == 0) {
+      if (live) flag[fi] = 0;
+      if (lane == 0) atomicAdd(&g.items_ctr[AXIS], __popc(dirty));
+    }
+  }
+  const size_t bstride = (size_t)kBrickVox * (AXIS == 1 ? (size_t)g.BX : (size_t)g.BX * g.BY);
+  const size_t base = (size_t)(AXIS == 1 ? ut_slot(g, bx, 0, bc) : ut_slot(g, bx, bc, 0)) * kBrickVox;
+  if (warp == 0) lmin[lane] = (uint32_t)kNone;
+  // stage: 16 bytes per copy, eight to a plane; positions past the line's end are kNone
+  for (int i = threadIdx.x; i < nb * 64; i += blockDim.x) {
+    const int pos = i >> 3;
+    if (pos < n) {
+      const int32_t* src = in + base + (size_t)(pos >> 3) * bstride + 64 * (pos & 7) + 32 * h + 4 * (i & 7);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(val + 4 * i)),
+                   "l"(src)
+                   : "memory");
+    } else {
+      reinterpret_cast<int4*>(val)[i] = make_int4(kNone, kNone, kNone, kNone);
+    }
+  }
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  for (int b = warp; b < nb; b += nw) {
+    const uint32_t m = line_brick_min<uint32_t, 32>(val + b * 256 + lane);
+    bmin[b * 32 + lane] = m;
+    atomicMin(&lmin[lane], m);
+  }
+  __syncthreads();
+  const uint32_t least = lmin[lane];
+  const bool some = live && least != (uint32_t)kNone;  // a line without a finite input is kNone throughout
+  // arguments at the brick boundaries 8 b (the last one at n - 1): every eighth first, then the rest
+  for (int q = warp; 8 * q < nb + 8; q += nw) {
+    const int b = min(8 * q, nb), p = min(8 * b, n - 1);
+    uint32_t best = some ? ~0u : 0u;
+    int arg = 0;
+    line_argmin<uint32_t, 32>(val + lane, bmin + lane, least, p, 0, nb - 1, best, arg);
+    args[b * 32 + lane] = (uint16_t)arg;
+  }
+  __syncthreads();
+  for (int b = warp; b < nb; b += nw) {
+    if ((b & 7) == 0) continue;
+    const int p = 8 * b, a0 = args[(b & ~7) * 32 + lane], a1 = args[min((b & ~7) + 8, nb) * 32 + lane];
+    const uint32_t c0 = val[a0 * 32 + lane] + (uint32_t)((p - a0) * (p - a0));
+    const uint32_t c1 = val[a1 * 32 + lane] + (uint32_t)((p - a1) * (p - a1));
+    uint32_t best = some ? min(c0, c1) : 0u;
+    int arg = c0 <= c1 ? a0 : a1;
+    line_argmin<uint32_t, 32>(val + lane, bmin + lane, least, p, min(a0, a1) >> 3, max(a0, a1) >> 3, best, arg);
+    args[b * 32 + lane] = (uint16_t)arg;
+  }
+  __syncthreads();
+  for (int b = warp; b < nb; b += nw) {
+    if (!live) continue;
+    const int a0 = args[b * 32 + lane], a1 = args[b * 32 + 32 + lane];
+    uint32_t r[8];
+    line_outputs<uint32_t, 32>(val + lane, 8 * b, min(a0, a1), some ? max(a0, a1) : -1, r);
+    int32_t* dst = out + base + (size_t)b * bstride + (AXIS == 1 ? ut_vox(x, 0, c) : 32 * h + lane);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int o = (int)min(r[k], (uint32_t)kNone), at = k * (AXIS == 1 ? 8 : 64);
+      if (8 * b + k >= n) break;
+      if (UPD && AXIS == 1) {
+        if (dst[at] != o) {
+          dst[at] = o;
+          reinterpret_cast<uint8_t*>(g.ut_bits + ut_row_words(g) + ut_yline_words(g))[(size_t)ut_nxp(g) * (8 * b + k) + x] = 1;
+        }
+      } else {
+        dst[at] = o;
+      }
+    }
+  }
+}
+
+template <int AXIS, bool UPD>
+cudaError_t launch_line(const GridView& g, const int32_t* in, int32_t* out, cudaStream_t st) {
+  const int n = AXIS == 1 ? g.ny : g.nz;
+  const int64_t tiles = 2ll * g.BX * (AXIS == 1 ? g.BZ : g.BY);
+  const cudaError_t e = cudaFuncSetAttribute(k_ut_line<AXIS, UPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)line_smem(kLineMax));
+  if (e != cudaSuccess) return e;
+  const int threads = n <= 64 ? 128 : (n <= 128 ? 256 : (n <= 768 ? 512 : 1024));
+  VDB_LAUNCH((k_ut_line<AXIS, UPD>), (unsigned)tiles, threads, line_smem(n), st, g, in, out);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_ut_init(const GridView& g, cudaStream_t st) {
@@ -368,10 +497,11 @@ cudaError_t launch_ut_dense(const GridView& g, const uint8_t* grid, cudaStream_t
   return cudaGetLastError();
 }
 
-// The line stacks (8 bytes per voxel of lines padded along x to a multiple of 32), or the x pass's
-// carries (4 bytes per row and brick), whichever is larger.
+// The x pass's carries (4 bytes per row and brick) or, where lines are too long to be staged, the line
+// stacks (8 bytes per voxel of lines padded along x to a multiple of 32), whichever is larger.
 size_t ut_scratch_bytes(const GridView& g) {
-  return std::max((size_t)ut_nxp(g) * g.ny * g.nz * sizeof(int2), (size_t)g.BX * g.BY * g.BZ * 64 * sizeof(int32_t));
+  const size_t stacks = g.ny > kLineMax || g.nz > kLineMax ? (size_t)ut_nxp(g) * g.ny * g.nz * sizeof(int2) : 0;
+  return std::max(stacks, (size_t)g.BX * g.BY * g.BZ * 64 * sizeof(int32_t));
 }
 
 cudaError_t launch_ut_pass(const GridView& g, int axis, void* scratch, cudaStream_t st) {
@@ -380,10 +510,17 @@ cudaError_t launch_ut_pass(const GridView& g, int axis, void* scratch, cudaStrea
   int2* stack = static_cast<int2*>(scratch);
   if (axis == 0) {
     VDB_LAUNCH(k_ut_x<false>, ut_blocks((int64_t)g.BY * g.BZ * 64), kUT, 0, st, g, static_cast<int32_t*>(scratch));
+  } else if (axis == 1 && g.ny <= kLineMax) {
+    return launch_line<1, false>(g, g1, g2, st);
   } else if (axis == 1) {
     VDB_LAUNCH(k_ut_env<1>, ut_blocks((int64_t)g.nx * g.nz), kUT, 0, st, g, g1, g2, stack);
   } else {
-    VDB_LAUNCH(k_ut_env<2>, ut_blocks((int64_t)g.nx * g.ny), kUT, 0, st, g, g2, g.dist, stack);
+    if (g.nz <= kLineMax) {
+      const cudaError_t e = launch_line<2, false>(g, g2, g.dist, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      VDB_LAUNCH(k_ut_env<2>, ut_blocks((int64_t)g.nx * g.ny), kUT, 0, st, g, g2, g.dist, stack);
+    }
     VDB_LAUNCH(k_ut_flags, ut_blocks((int64_t)g.BX * g.BY * g.BZ), kUT, 0, st, g);
   }
   return cudaGetLastError();
@@ -394,11 +531,18 @@ cudaError_t launch_ut_update_pass(const GridView& g, int axis, void* scratch, cu
   int32_t* g2 = reinterpret_cast<int32_t*>(g.g2);
   if (axis == 0) {
     VDB_LAUNCH(k_ut_x<true>, ut_blocks((int64_t)g.BY * g.BZ * 64), kUT, 0, st, g, static_cast<int32_t*>(scratch));
+  } else if (axis == 1 && g.ny <= kLineMax) {
+    return launch_line<1, true>(g, g1, g2, st);
   } else if (axis == 1) {
     VDB_LAUNCH(k_ut_env_upd<1>, ut_blocks((int64_t)ut_nxp(g) * g.nz), kUT, 0, st, g, g1, g2, static_cast<int2*>(scratch));
   } else {
-    VDB_LAUNCH(k_ut_env_upd<2>, ut_blocks((int64_t)ut_nxp(g) * g.ny), kUT, 0, st, g, g2, g.dist,
-               static_cast<int2*>(scratch));
+    if (g.nz <= kLineMax) {
+      const cudaError_t e = launch_line<2, true>(g, g2, g.dist, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      VDB_LAUNCH(k_ut_env_upd<2>, ut_blocks((int64_t)ut_nxp(g) * g.ny), kUT, 0, st, g, g2, g.dist,
+                 static_cast<int2*>(scratch));
+    }
     VDB_LAUNCH(k_ut_flags, ut_blocks((int64_t)g.BX * g.BY * g.BZ), kUT, 0, st, g);
   }
   return cudaGetLastError();
