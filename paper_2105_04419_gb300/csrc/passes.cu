@@ -38,10 +38,11 @@
 // reaches every output's current minimum in the warp, and skips windows whose input bricks hold no
 // value below dmax^2.
 //
-// Grids with dmax above 45 (up to 181), and any grid tuned to variant 8, take the lower-envelope
-// kernels at the end of the file: O(1) amortised work per voxel, whatever the window.
+// Grids with dmax above 45 (up to 181), and any grid tuned to variant 8, take the envelope kernels at
+// the end of the file, whose work per voxel hardly grows with the window.
 #include <cuda_fp16.h>
 
+#include "line_min.cuh"
 #include "vdbedt_internal.cuh"
 
 namespace vdbedt {
@@ -497,7 +498,7 @@ __global__ void __launch_bounds__(256) k_x_direct(GridView g, const int32_t* __r
 }
 
 // ------------------------------------------------------------------------------------------------
-// Lower-envelope kernels (any dmax up to 181; the only form above 45, variant 8 below it).
+// Envelope kernels (any dmax up to 181; the only form above 45, variant 8 below it).
 //
 // Fields hold plain 16-bit integers (g1 y-major, g2 z-major, as in the windowed kernels).  A work
 // item is a run of kEnvRun bricks along the pass axis (a node's length); each kernel finds the
@@ -507,23 +508,11 @@ __global__ void __launch_bounds__(256) k_x_direct(GridView g, const int32_t* __r
 //      the neighbouring bricks' bytes outward until one holds a set bit (a warp per output brick,
 //      a lane per two x-rows).
 //   y, z: for one line f(0 .. n-1) along the axis (the run and its halo, n = 8 (kEnvRun + 2R)),
-//      every output x needs min over q of (x - q)^2 + f(q), the lower envelope of the parabolas
-//      rooted at (q, f(q)) evaluated at x (the separable exact transform of Felzenszwalb and
-//      Huttenlocher, "Distance Transforms of Sampled Functions", 2012, restated here for integers
-//      and a streaming deque).  A thread owns a line.  Input q enters as the parabola with
-//      h = f(q) + q^2 (inputs at dmax^2 are left out: they cannot bring an output below dmax^2);
-//      the back of the deque is dropped while it is nowhere strictly below both its predecessor and
-//      the new parabola -- (h_q - h_b)(v_b - v_a) <= (h_b - h_a)(q - v_b), the intersection test
-//      with the denominators multiplied out (no division, exact in int32).  Once q = x + W, output x
-//      has seen every input within W (any farther one costs at least (W + 1)^2 >= dmax^2):
-//      parabolas rooted more than W before x are dropped from the front, the front is dropped while
-//      its successor is at least as low at x (h_b - h_a <= 2x (v_b - v_a)), and the front gives
-//      min(dmax^2, h - 2xv + x^2).  Queries advance monotonically, so every parabola enters and
-//      leaves once: O(1) amortised per voxel, independent of the window.  The deque holds at most
-//      2W + 2 entries (a ring in the thread's local memory, one packed word h << 9 | v each).
+//      every output i needs min over j of (i - j)^2 + f(j) (any input farther than the halo costs at
+//      least (W + 1)^2 >= dmax^2): the bracketed minima of line_min.cuh.  Work per voxel hardly grows
+//      with the window.
 // ------------------------------------------------------------------------------------------------
 constexpr int kEnvRun = 16;
-constexpr int kEnvThreads = 64;  // y, z: one line of an item per thread (8 x 8 lines)
 
 __device__ __forceinline__ int occ_byte(const GridView& g, int slot, int row) {
   return slot >= 0 ? (int)reinterpret_cast<const uint8_t*>(g.occ)[(size_t)slot * 64 + row] : 0;
@@ -593,88 +582,121 @@ __global__ void __launch_bounds__(256) k_env_x(GridView g, const unsigned long l
   }
 }
 
-// y (AXIS 1: g1 -> g2) or z (AXIS 2: g2 -> D) pass by the lower envelope.  Block = one item at a
-// time, thread t = the line (t & 7, t >> 3) across the axis.  RING >= 2W + 2.
-template <int AXIS, int RING>
-__global__ void __launch_bounds__(kEnvThreads) k_env_yz(GridView g, const unsigned long long* __restrict__ items,
+// y (AXIS 1: g1 -> g2) or z (AXIS 2: g2 -> D) pass: a block per item at a time, its run and halo staged
+// whole in shared memory as planes of 64 lines (16-bit values; bricks that are absent or hold nothing
+// below dmax^2 are filled with it), then the bracketed minima of line_min.cuh, a lane per line and each
+// warp on its own (brick, half of the lines).  Positions count from the first halo brick.
+// Bound by issue; R halo bricks each side make the staged bytes (kEnvRun + 2R) / kEnvRun times the run's.
+// 512 x 512 x 256 tunnel scene, dmax 64: y 0.26 ms, z 0.22 ms (a thread per line with its envelope in a
+// local-memory deque: 0.72 and 0.66).
+constexpr int kEnvBlock = 256;
+constexpr int kEnvMaxNB = kEnvRun + 2 * 23;
+size_t env_smem(int R) { return (size_t)(kEnvRun + 2 * R) * (kBrickVox * 2 + 128); }
+
+template <int AXIS>
+__global__ void __launch_bounds__(kEnvBlock) k_env_line(GridView g, const unsigned long long* __restrict__ items,
                                                         int max_items) {
-  __shared__ int slots[kEnvRun + 2 * 23];  // stored bricks of the run and its halo (-1: none)
-  __shared__ int inslot[kEnvRun + 2 * 23];  // the same, -1 also where the brick's input is all dmax^2
-  __shared__ __align__(16) uint16_t tile[kBrickVox];  // y pass: one output brick, transposed to z-major
-  const int R = g.R, W = 8 * R, NB = kEnvRun + 2 * R, n = 8 * NB, INF = g.INF;
+  extern __shared__ __align__(16) uint16_t smem16[];
+  __shared__ int slots[kEnvMaxNB];   // stored bricks of the run and its halo (-1: none)
+  __shared__ int inslot[kEnvMaxNB];  // the same, -1 also where the brick's input is all dmax^2
+  __shared__ uint32_t lmin[64];      // the lines' minima
+  __shared__ uint16_t args[(kEnvRun + 1) * 64];
+  __shared__ uint32_t fin[kEnvRun];
+  __shared__ __align__(16) uint16_t rows[kEnvBlock / 32][256];  // y pass: a warp's 8 outputs x 32 lines, by row
+  const int R = g.R, NB = kEnvRun + 2 * R, INF = g.INF;
+  uint16_t* val = smem16;                  // [8 NB][64]
+  uint16_t* bmin = val + NB * kBrickVox;   // [NB][64]
   const int nitems = min(g.items_ctr[AXIS], max_items);
-  const int t = threadIdx.x;
-  const int c0 = t & 7, c1 = t >> 3;  // y pass: (x, z); z pass: (x, y)
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  constexpr int nw = kEnvBlock / 32;
   const uint16_t* __restrict__ src = AXIS == 1 ? g.g1 : g.g2;
   const uint32_t in_fin = AXIS == 1 ? F_G1FIN : F_G2FIN;
-  int ring[RING];
+  const uint32_t inf2 = (uint32_t)INF | ((uint32_t)INF << 16);
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     int bx, by, bz;
     unpack_brick(items[it], bx, by, bz);
-    __syncthreads();  // the previous item's slots are no longer read
-    for (int i = t; i < NB; i += blockDim.x) {
-      const int s = AXIS == 1 ? find_brick(g, bx, by - R + i, bz) : find_brick(g, bx, by, bz - R + i);
-      slots[i] = s;
-      inslot[i] = (s >= 0 && (g.bflags[s] & in_fin)) ? s : -1;
+    __syncthreads();  // the previous item's shared memory is no longer read
+    if (t < NB) {
+      const int s = AXIS == 1 ? find_brick(g, bx, by - R + t, bz) : find_brick(g, bx, by, bz - R + t);
+      slots[t] = s;
+      inslot[t] = (s >= 0 && (g.bflags[s] & in_fin)) ? s : -1;
+    }
+    if (t < 64) lmin[t] = (uint32_t)INF;
+    if (t < kEnvRun) fin[t] = 0u;
+    const bool some = __syncthreads_or(t < NB && inslot[t] >= 0);
+    if (some) {
+      for (int i = t; i < NB * 64; i += kEnvBlock) {  // 16 bytes each, 64 to a brick
+        const int s = inslot[i >> 6];
+        if (s >= 0)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(val + 8 * i)),
+                       "l"(src + (size_t)s * kBrickVox + 8 * (i & 63))
+                       : "memory");
+        else
+          reinterpret_cast<uint4*>(val)[i] = make_uint4(inf2, inf2, inf2, inf2);
+      }
+      asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      for (int u = warp; u < 2 * NB; u += nw) {
+        const int b = u >> 1, line = 32 * (u & 1) + lane;
+        const uint32_t m = line_brick_min<uint16_t, 64>(val + b * kBrickVox + line);
+        bmin[b * 64 + line] = (uint16_t)m;
+        if (inslot[b] >= 0) atomicMin(&lmin[line], m);
+      }
+      __syncthreads();
+      // arguments at the run's brick boundaries 8 (R + b), b = 0 .. kEnvRun: every eighth, then the rest
+      for (int u = warp; u < 2 * (kEnvRun / 8 + 1); u += nw) {
+        const int b = 8 * (u >> 1), line = 32 * (u & 1) + lane;
+        const uint32_t least = lmin[line];
+        uint32_t best = least < (uint32_t)INF ? ~0u : 0u;
+        int arg = 0;
+        line_argmin<uint16_t, 64>(val + line, bmin + line, least, 8 * (R + b), 0, NB - 1, best, arg);
+        args[b * 64 + line] = (uint16_t)arg;
+      }
+      __syncthreads();
+      for (int u = warp; u < 2 * kEnvRun; u += nw) {
+        const int b = u >> 1, line = 32 * (u & 1) + lane;
+        if ((b & 7) == 0) continue;
+        const int p = 8 * (R + b), a0 = args[(b & ~7) * 64 + line], a1 = args[((b & ~7) + 8) * 64 + line];
+        const uint32_t c0 = val[a0 * 64 + line] + (uint32_t)((p - a0) * (p - a0));
+        const uint32_t c1 = val[a1 * 64 + line] + (uint32_t)((p - a1) * (p - a1));
+        const uint32_t least = lmin[line];
+        uint32_t best = least < (uint32_t)INF ? min(c0, c1) : 0u;
+        int arg = c0 <= c1 ? a0 : a1;
+        line_argmin<uint16_t, 64>(val + line, bmin + line, least, p, min(a0, a1) >> 3, max(a0, a1) >> 3, best, arg);
+        args[b * 64 + line] = (uint16_t)arg;
+      }
+      __syncthreads();
+    }
+    for (int u = warp; u < 2 * kEnvRun; u += nw) {
+      const int b = u >> 1, h = u & 1, line = 32 * h + lane, slot = slots[R + b];
+      if (slot < 0) continue;  // warp-uniform
+      const int a0 = args[b * 64 + line], a1 = args[(b + 1) * 64 + line];
+      const bool any = some && lmin[line] < (uint32_t)INF;  // (a line without an input below dmax^2 is dmax^2)
+      uint32_t r[8];
+      line_outputs<uint16_t, 64>(val + line, 8 * (R + b), min(a0, a1), any ? max(a0, a1) : -1, r);
+      bool f = false;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        r[k] = min(r[k], (uint32_t)INF);
+        f |= r[k] < (uint32_t)INF;
+      }
+      if (AXIS == 1) {
+        // g2 is z-major: the warp's 4 planes z (lane >> 3) of 8 rows, gathered so that a lane stores a row
+        uint16_t* w = rows[warp];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) w[64 * (lane >> 3) + 8 * k + (lane & 7)] = (uint16_t)r[k];
+        __syncwarp();
+        reinterpret_cast<uint4*>(g.g2 + (size_t)slot * kBrickVox + 256 * h)[lane] = reinterpret_cast<const uint4*>(w)[lane];
+      } else {
+        int32_t* dst = g.dist + (size_t)slot * kBrickVox + line;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) dst[64 * k] = (int)r[k];
+      }
+      if (__any_sync(0xffffffffu, f) && lane == 0) atomicOr(&fin[b], 1u);
     }
     __syncthreads();
-    int head = 0, tail = 0, cnt = 0;
-    bool fin = false;
-    for (int q = 0; q < n; ++q) {
-      const int sq = inslot[q >> 3];
-      // input (c0, c1) at position q & 7 along the axis: g1 y-major x + 8z + 64y, g2 z-major x + 8y + 64z
-      const int f = sq >= 0 ? (int)src[(size_t)sq * kBrickVox + 64 * (q & 7) + 8 * c1 + c0] : INF;
-      if (f < INF) {
-        const int hq = f + q * q;
-        while (cnt >= 2) {
-          const int ib = tail == 0 ? RING - 1 : tail - 1, ia = ib == 0 ? RING - 1 : ib - 1;
-          const int b = ring[ib], a = ring[ia];
-          const int vb = b & 511, hb = b >> 9, va = a & 511, ha = a >> 9;
-          if ((hq - hb) * (vb - va) > (hb - ha) * (q - vb)) break;
-          tail = ib;
-          --cnt;
-        }
-        ring[tail] = (hq << 9) | q;
-        tail = tail + 1 == RING ? 0 : tail + 1;
-        ++cnt;
-      }
-      const int x = q - W;  // output position, once every input within W of it is in
-      if (x < W) continue;  // block-uniform
-      while (cnt > 0 && (ring[head] & 511) < x - W) {
-        head = head + 1 == RING ? 0 : head + 1;
-        --cnt;
-      }
-      while (cnt >= 2) {
-        const int ib = head + 1 == RING ? 0 : head + 1;
-        const int a = ring[head], b = ring[ib];
-        if ((b >> 9) - (a >> 9) > 2 * x * ((b & 511) - (a & 511))) break;
-        head = ib;
-        --cnt;
-      }
-      int res = INF;
-      if (cnt > 0) {
-        const int a = ring[head];
-        res = min(INF, (a >> 9) - 2 * x * (a & 511) + x * x);
-      }
-      fin |= res < INF;
-      const int oslot = slots[x >> 3];  // block-uniform
-      const int k = x & 7;
-      if (AXIS == 1)
-        tile[c0 + 8 * k + 64 * c1] = (uint16_t)res;  // g2 z-major: x + 8 y + 64 z
-      else if (oslot >= 0)
-        g.dist[(size_t)oslot * kBrickVox + 64 * k + 8 * c1 + c0] = res;  // D z-major: x + 8 y + 64 z
-      if (k == 7) {  // block-uniform: the output brick is complete
-        const int any = __syncthreads_or(fin);
-        fin = false;
-        if (oslot >= 0) {
-          if (AXIS == 1)
-            for (int i = t; i < kBrickVox / 8; i += blockDim.x)
-              reinterpret_cast<uint4*>(g.g2 + (size_t)oslot * kBrickVox)[i] = reinterpret_cast<const uint4*>(tile)[i];
-          if (t == 0) set_flag_bit(g, oslot, AXIS == 1 ? F_G2FIN : F_FINITE, any != 0);
-        }
-        if (AXIS == 1) __syncthreads();  // the tile is read before the next brick overwrites it
-      }
-    }
+    if (t < kEnvRun && slots[R + t] >= 0) set_flag_bit(g, slots[R + t], AXIS == 1 ? F_G2FIN : F_FINITE, fin[t] != 0u);
   }
 }
 
@@ -692,31 +714,27 @@ int num_sms() {
 // Persistent launch of an envelope kernel: as many blocks as fit on the GPU at once (items are
 // taken grid-stride; blocks beyond the queued count exit at once).
 template <typename K>
-cudaError_t launch_env_kernel(K kernel, int threads, const GridView& g, const unsigned long long* items,
+cudaError_t launch_env_kernel(K kernel, int threads, size_t smem, const GridView& g, const unsigned long long* items,
                               cudaStream_t st) {
   if (g.item_cap <= 0) return cudaSuccess;
+  // the largest radius's shared memory, whatever this grid's: concurrent callers set the same value
+  cudaError_t e = smem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)env_smem(23)) : cudaSuccess;
+  if (e != cudaSuccess) return e;
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
   int grid = num_sms() * per_sm;
   if (grid > g.item_cap) grid = g.item_cap;
-  VDB_LAUNCH(kernel, grid, threads, 0, st, g, items, g.item_cap);
+  VDB_LAUNCH(kernel, grid, threads, smem, st, g, items, g.item_cap);
   return cudaGetLastError();
 }
 
-// Envelope pass along `axis`; the deque ring is sized for the grid's window (2W + 2 entries).
+// Envelope pass along `axis`.
 cudaError_t launch_env(const GridView& g, int axis, const Items& it, cudaStream_t st) {
-  if (axis == 0) return launch_env_kernel(k_env_x, 256, g, it.run[0], st);
-  const int need = 2 * 8 * g.R + 2;
-  if (axis == 1) {
-    if (need <= 130) return launch_env_kernel(k_env_yz<1, 130>, kEnvThreads, g, it.run[1], st);
-    if (need <= 258) return launch_env_kernel(k_env_yz<1, 258>, kEnvThreads, g, it.run[1], st);
-    return launch_env_kernel(k_env_yz<1, 370>, kEnvThreads, g, it.run[1], st);
-  }
-  if (need <= 130) return launch_env_kernel(k_env_yz<2, 130>, kEnvThreads, g, it.run[2], st);
-  if (need <= 258) return launch_env_kernel(k_env_yz<2, 258>, kEnvThreads, g, it.run[2], st);
-  return launch_env_kernel(k_env_yz<2, 370>, kEnvThreads, g, it.run[2], st);
+  if (axis == 0) return launch_env_kernel(k_env_x, 256, 0, g, it.run[0], st);
+  if (axis == 1) return launch_env_kernel(k_env_line<1>, kEnvBlock, env_smem(g.R), g, it.run[1], st);
+  return launch_env_kernel(k_env_line<2>, kEnvBlock, env_smem(g.R), g, it.run[2], st);
 }
 
 template <int R, int RUN, int AXIS>
