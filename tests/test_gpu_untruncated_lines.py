@@ -1,6 +1,6 @@
 """Whole-line passes of untruncated grids against the oracle where the staged tiles can go wrong: lines
 around one brick, one group of eight bricks and the longest staged line (1,496 positions; longer ones keep
-the stack kernels), ragged across, with one far obstacle, few and many, then updates of a few voxels."""
+the stack kernels), x rows around one and several steps of 32 bricks, ragged across, with one far obstacle, few and many, then updates of a few voxels."""
 import numpy as np
 import pytest
 
@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("shape_xyz", [(3, 7, 9), (9, 8, 64), (17, 63, 65), (33, 66, 8), (5, 520, 71), (6, 5, 513),
-                                       (9, 1496, 3), (9, 1497, 3), (5, 3, 1495), (4, 2, 1505)])
+                                       (9, 1496, 3), (9, 1497, 3), (5, 3, 1495), (4, 2, 1505), (256, 5, 9),
+                                       (257, 9, 2), (523, 3, 17), (2100, 2, 3)])
 @pytest.mark.parametrize("count", [1, 3, 400])
 def test_lines(shape_xyz, count):
     import paper_2105_04419_gb300 as V
