@@ -39,7 +39,7 @@
 // value below dmax^2.
 //
 // Grids with dmax above 45 (up to 181), and any grid tuned to variant 8, take the envelope kernels at
-// the end of the file, whose work per voxel hardly grows with the window.
+// the end of the file, whose work per voxel follows the distances, not the window.
 #include <cuda_fp16.h>
 
 #include "line_min.cuh"
@@ -506,8 +506,8 @@ __global__ void __launch_bounds__(256) k_x_direct(GridView g, const int32_t* __r
 //   x: the distance to the nearest occupied voxel of an x-line, from the line's bits.
 //   y, z: for one line f(0 .. n-1) along the axis (the run and its halo, n = 8 (kEnvRun + 2R)),
 //      every output i needs min over j of (i - j)^2 + f(j) (any input farther than the halo costs at
-//      least (W + 1)^2 >= dmax^2): the bracketed minima of line_min.cuh.  Work per voxel hardly grows
-//      with the window.
+//      least (W + 1)^2 >= dmax^2): the walk of line_min.cuh.  Work per voxel follows the distances, not the
+//      window.
 // ------------------------------------------------------------------------------------------------
 constexpr int kEnvRun = 16;
 
@@ -594,50 +594,52 @@ __global__ void __launch_bounds__(256) k_env_x(GridView g, const unsigned long l
 
 // y (AXIS 1: g1 -> g2) or z (AXIS 2: g2 -> D) pass: a block per item at a time, its run and halo staged
 // whole in shared memory as planes of 64 lines (16-bit values; bricks that are absent or hold nothing
-// below dmax^2 are filled with it), then the bracketed minima of line_min.cuh, a lane per line and each
-// warp on its own (brick, half of the lines).  Positions count from the first halo brick.
+// below dmax^2 are filled with it), then line_min.cuh's walk, a lane per two lines and each warp on its own
+// bricks.  Positions count from the first halo brick.
 // Bound by issue; R halo bricks each side make the staged bytes (kEnvRun + 2R) / kEnvRun times the run's.
-// 512 x 512 x 256 tunnel scene, dmax 64: y 0.26 ms, z 0.22 ms (a thread per line with its envelope in a
-// local-memory deque: 0.72 and 0.66).
+// 512 x 512 x 256 tunnel scene, dmax 64 / 128 / 181: y 0.16 / 0.23 / 0.31 ms, z 0.15 / 0.19 / 0.25 (a
+// thread per line with its envelope in a local-memory deque: y 0.73 / 1.00 / 1.15, z 0.67 / 0.85 / 0.84; brackets
+// over single lines: 0.26 and 0.22 at 64).  With isolated obstacles far apart the walk passes more bricks: at
+// 2e-5 of the voxels and dmax 181 y takes 0.50 (0.40), z 0.23 (0.64), x 0.07 (0.37).
 constexpr int kEnvBlock = 256;
-size_t env_smem(int R) { return (size_t)(kEnvRun + 2 * R) * (kBrickVox * 2 + 128); }
+// values, minima, squares of -8 NB .. 8 NB + 15
+size_t env_smem(int R) { return (size_t)(kEnvRun + 2 * R) * (kBrickVox * 2 + 128 + 64) + 64; }
 
 template <int AXIS>
 __global__ void __launch_bounds__(kEnvBlock) k_env_line(GridView g, const unsigned long long* __restrict__ items,
                                                         int max_items) {
-  extern __shared__ __align__(16) uint16_t smem16[];
+  extern __shared__ __align__(16) uint32_t smem32[];
   __shared__ int slots[kEnvMaxNB];   // stored bricks of the run and its halo (-1: none)
   __shared__ int inslot[kEnvMaxNB];  // the same, -1 also where the brick's input is all dmax^2
-  __shared__ uint32_t lmin[64];      // the lines' minima
-  __shared__ uint16_t args[(kEnvRun + 1) * 64];
-  __shared__ uint32_t fin[kEnvRun];
-  __shared__ __align__(16) uint16_t rows[kEnvBlock / 32][256];  // y pass: a warp's 8 outputs x 32 lines, by row
+  __shared__ uint32_t gmin[(kEnvMaxNB + 7) / 8 * 32];  // minima over eight bricks
+  __shared__ __align__(16) uint32_t rows[kEnvBlock / 32][256];  // y pass: a warp's output brick, by row
   const int R = g.R, NB = kEnvRun + 2 * R, INF = g.INF;
-  uint16_t* val = smem16;                  // [8 NB][64]
-  uint16_t* bmin = val + NB * kBrickVox;   // [NB][64]
+  uint32_t* val = smem32;                  // [8 NB][32]
+  uint32_t* bmin = val + NB * kBrickWords;  // [NB][32]
+  uint32_t* sq = bmin + NB * 32 + 8 * NB;
   const int nitems = min(g.items_ctr[AXIS], max_items);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   constexpr int nw = kEnvBlock / 32;
   const uint16_t* __restrict__ src = AXIS == 1 ? g.g1 : g.g2;
   const uint32_t in_fin = AXIS == 1 ? F_G1FIN : F_G2FIN;
   const uint32_t inf2 = (uint32_t)INF | ((uint32_t)INF << 16);
+  for (int u = t - 8 * NB; u < 8 * NB + 16; u += kEnvBlock) sq[u] = line16_square(u);
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     int bx, by, bz;
     unpack_brick(items[it], bx, by, bz);
     __syncthreads();  // the previous item's shared memory is no longer read
-    if (t < NB) {
+    if (t < NB) {  // at most 62
       const int s = AXIS == 1 ? find_brick(g, bx, by - R + t, bz) : find_brick(g, bx, by, bz - R + t);
       slots[t] = s;
       inslot[t] = (s >= 0 && (g.bflags[s] & in_fin)) ? s : -1;
     }
-    if (t < 64) lmin[t] = (uint32_t)INF;
-    if (t < kEnvRun) fin[t] = 0u;
     const bool some = __syncthreads_or(t < NB && inslot[t] >= 0);
+    uint32_t least = inf2;
     if (some) {
       for (int i = t; i < NB * 64; i += kEnvBlock) {  // 16 bytes each, 64 to a brick
         const int s = inslot[i >> 6];
         if (s >= 0)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(val + 8 * i)),
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(val + 4 * i)),
                        "l"(src + (size_t)s * kBrickVox + 8 * (i & 63))
                        : "memory");
         else
@@ -645,67 +647,52 @@ __global__ void __launch_bounds__(kEnvBlock) k_env_line(GridView g, const unsign
       }
       asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
       __syncthreads();
-      for (int u = warp; u < 2 * NB; u += nw) {
-        const int b = u >> 1, line = 32 * (u & 1) + lane;
-        const uint32_t m = line_brick_min<uint16_t, 64>(val + b * kBrickVox + line);
-        bmin[b * 64 + line] = (uint16_t)m;
-        if (inslot[b] >= 0) atomicMin(&lmin[line], m);
+      for (int q = warp; 8 * q < NB; q += nw) {
+        uint32_t m8 = ~0u;
+        for (int b = 8 * q; b < min(8 * q + 8, NB); ++b) {
+          const uint32_t m = inslot[b] >= 0 ? line16_min8(val + b * kBrickWords + lane) : inf2;
+          bmin[b * 32 + lane] = m;
+          m8 = __vminu2(m8, m);
+        }
+        gmin[q * 32 + lane] = m8;
       }
       __syncthreads();
-      // arguments at the run's brick boundaries 8 (R + b), b = 0 .. kEnvRun: every eighth, then the rest
-      for (int u = warp; u < 2 * (kEnvRun / 8 + 1); u += nw) {
-        const int b = 8 * (u >> 1), line = 32 * (u & 1) + lane;
-        const uint32_t least = lmin[line];
-        uint32_t best = least < (uint32_t)INF ? ~0u : 0u;
-        int arg = 0;
-        line_argmin<uint16_t, 64>(val + line, bmin + line, least, 8 * (R + b), 0, NB - 1, best, arg);
-        args[b * 64 + line] = (uint16_t)arg;
-      }
-      __syncthreads();
-      for (int u = warp; u < 2 * kEnvRun; u += nw) {
-        const int b = u >> 1, line = 32 * (u & 1) + lane;
-        if ((b & 7) == 0) continue;
-        const int p = 8 * (R + b), a0 = args[(b & ~7) * 64 + line], a1 = args[((b & ~7) + 8) * 64 + line];
-        const uint32_t c0 = val[a0 * 64 + line] + (uint32_t)((p - a0) * (p - a0));
-        const uint32_t c1 = val[a1 * 64 + line] + (uint32_t)((p - a1) * (p - a1));
-        const uint32_t least = lmin[line];
-        uint32_t best = least < (uint32_t)INF ? min(c0, c1) : 0u;
-        int arg = c0 <= c1 ? a0 : a1;
-        line_argmin<uint16_t, 64>(val + line, bmin + line, least, p, min(a0, a1) >> 3, max(a0, a1) >> 3, best, arg);
-        args[b * 64 + line] = (uint16_t)arg;
-      }
-      __syncthreads();
+      for (int q = 0; 8 * q < NB; ++q) least = __vminu2(least, gmin[q * 32 + lane]);
     }
-    for (int u = warp; u < 2 * kEnvRun; u += nw) {
-      const int b = u >> 1, h = u & 1, line = 32 * h + lane, slot = slots[R + b];
+    const bool live = least != inf2;  // (lines without an input below dmax^2 are dmax^2)
+    for (int b = warp; b < kEnvRun; b += nw) {
+      const int slot = slots[R + b];
       if (slot < 0) continue;  // warp-uniform
-      const int a0 = args[b * 64 + line], a1 = args[(b + 1) * 64 + line];
-      const bool any = some && lmin[line] < (uint32_t)INF;  // (a line without an input below dmax^2 is dmax^2)
       uint32_t r[8];
-      line_outputs<uint16_t, 64>(val + line, 8 * (R + b), min(a0, a1), any ? max(a0, a1) : -1, r);
-      bool f = false;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) r[k] = inf2;
+      if (__any_sync(0xffffffffu, live))
+        line16_outputs(val + lane, bmin + lane, gmin + lane, sq, least, NB, R + b, live, r);
+      uint32_t least_out = inf2;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        r[k] = min(r[k], (uint32_t)INF);
-        f |= r[k] < (uint32_t)INF;
+        r[k] = __vminu2(r[k], inf2);
+        least_out = __vminu2(least_out, r[k]);
       }
       if (AXIS == 1) {
-        // g2 is z-major: the warp's 4 planes z (lane >> 3) of 8 rows, gathered so that a lane stores a row
-        uint16_t* w = rows[warp];
+        // g2 is z-major: a lane's word of eight rows of plane z = lane >> 2, gathered so that a lane
+        // stores rows
+        uint32_t* w = rows[warp];
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < 8; ++k) w[64 * (lane >> 3) + 8 * k + (lane & 7)] = (uint16_t)r[k];
+        for (int k = 0; k < 8; ++k) w[32 * (lane >> 2) + 4 * k + (lane & 3)] = r[k];
         __syncwarp();
-        reinterpret_cast<uint4*>(g.g2 + (size_t)slot * kBrickVox + 256 * h)[lane] = reinterpret_cast<const uint4*>(w)[lane];
+        uint4* dst = reinterpret_cast<uint4*>(g.g2 + (size_t)slot * kBrickVox);
+        dst[lane] = reinterpret_cast<const uint4*>(w)[lane];
+        dst[lane + 32] = reinterpret_cast<const uint4*>(w)[lane + 32];
       } else {
-        int32_t* dst = g.dist + (size_t)slot * kBrickVox + line;
+        int2* dst = reinterpret_cast<int2*>(g.dist + (size_t)slot * kBrickVox) + lane;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) dst[64 * k] = (int)r[k];
+        for (int k = 0; k < 8; ++k) dst[32 * k] = make_int2((int)(r[k] & 0xFFFFu), (int)(r[k] >> 16));
       }
-      if (__any_sync(0xffffffffu, f) && lane == 0) atomicOr(&fin[b], 1u);
+      const bool f = __any_sync(0xffffffffu, least_out != inf2);
+      if (lane == 0) set_flag_bit(g, slot, AXIS == 1 ? F_G2FIN : F_FINITE, f);
     }
-    __syncthreads();
-    if (t < kEnvRun && slots[R + t] >= 0) set_flag_bit(g, slots[R + t], AXIS == 1 ? F_G2FIN : F_FINITE, fin[t] != 0u);
   }
 }
 

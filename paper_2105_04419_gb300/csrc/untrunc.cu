@@ -403,7 +403,8 @@ __global__ void k_ut_flags(GridView g) {
 // writes the g2 values that changed and sets the z-line byte of each.
 // Bound by issue (searches and candidates, about 40 instructions a voxel) with 8 B of memory traffic a
 // voxel under it.  512 x 512 x 256 tunnel scene: y 0.24 ms, z 0.21 ms (the stack kernels 0.58 and 0.66;
-// memory alone would take 0.08); dirty lines of its first lidar frames 0.19 and 0.18 ms (0.42 and 0.26).
+// memory alone would take 0.08); dirty lines of its first lidar frames 0.18 and 0.17 ms (0.42 and 0.26).
+// Isolated obstacles far apart (2e-5 of the voxels) take y 0.31, z 0.22 (0.19 and 0.34).
 // kLineMax is what shared memory holds: 152 B a position with minima and arguments, of 227 KB.
 constexpr int kLineMax = 1496;
 __host__ __device__ inline int line_bricks(int n) { return (n + 7) >> 3; }
@@ -455,7 +456,7 @@ __global__ void k_ut_line(GridView g, const int32_t* __restrict__ in, int32_t* _
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   for (int b = warp; b < nb; b += nw) {
-    const uint32_t m = line_brick_min<uint32_t, 32>(val + b * 256 + lane);
+    const uint32_t m = line_brick_min(val + b * 256 + lane);
     bmin[b * 32 + lane] = m;
     atomicMin(&lmin[lane], m);
   }
@@ -467,7 +468,7 @@ __global__ void k_ut_line(GridView g, const int32_t* __restrict__ in, int32_t* _
     const int b = min(8 * q, nb), p = min(8 * b, n - 1);
     uint32_t best = some ? ~0u : 0u;
     int arg = 0;
-    line_argmin<uint32_t, 32>(val + lane, bmin + lane, least, p, 0, nb - 1, best, arg);
+    line_argmin(val + lane, bmin + lane, least, p, 0, nb - 1, best, arg);
     args[b * 32 + lane] = (uint16_t)arg;
   }
   __syncthreads();
@@ -478,7 +479,7 @@ __global__ void k_ut_line(GridView g, const int32_t* __restrict__ in, int32_t* _
     const uint32_t c1 = val[a1 * 32 + lane] + (uint32_t)((p - a1) * (p - a1));
     uint32_t best = some ? min(c0, c1) : 0u;
     int arg = c0 <= c1 ? a0 : a1;
-    line_argmin<uint32_t, 32>(val + lane, bmin + lane, least, p, min(a0, a1) >> 3, max(a0, a1) >> 3, best, arg);
+    line_argmin(val + lane, bmin + lane, least, p, min(a0, a1) >> 3, max(a0, a1) >> 3, best, arg);
     args[b * 32 + lane] = (uint16_t)arg;
   }
   __syncthreads();
@@ -486,7 +487,7 @@ __global__ void k_ut_line(GridView g, const int32_t* __restrict__ in, int32_t* _
     if (!live) continue;
     const int a0 = args[b * 32 + lane], a1 = args[b * 32 + 32 + lane];
     uint32_t r[8];
-    line_outputs<uint32_t, 32>(val + lane, 8 * b, min(a0, a1), some ? max(a0, a1) : -1, r);
+    line_outputs(val + lane, bmin + lane, 8 * b, min(a0, a1), some ? max(a0, a1) : -1, r);
     int32_t* dst = out + base + (size_t)b * bstride + (AXIS == 1 ? ut_vox(x, 0, c) : 32 * h + lane);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
