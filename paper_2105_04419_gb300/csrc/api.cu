@@ -212,7 +212,7 @@ Tuning effective_tuning(const vdbedt_map* h) {
 }
 
 vdbedt_status run_passes(vdbedt_map* h, const Tuning& t, bool need_slots) {
-  if (need_slots && half_path(h->g)) CK(h, launch_item_slots(h->g, t, h->items, h->st), "item slots");
+  if (need_slots && windowed_form(h->g)) CK(h, launch_item_slots(h->g, t, h->items, h->st), "item slots");
   mark(h, 3);
   CK(h, launch_pass(h->g, t, 0, h->items, h->st), "x pass");
   mark(h, 4);
@@ -262,7 +262,7 @@ vdbedt_status do_global(vdbedt_map* h) {
   mark(h, 1);
   CK(h, launch_activation_full(h->g, h->st), "activation");
   mark(h, 2);
-  CK(h, launch_build_items_full(h->g, t, h->items, half_path(h->g), h->st), "items");
+  CK(h, launch_build_items_full(h->g, t, h->items, windowed_form(h->g), h->st), "items");
   vdbedt_status s = run_passes(h, t, false);
   if (s) return s;
   h->computed = true;
@@ -349,7 +349,7 @@ vdbedt_status create_impl(const vdbedt_config* cfg, const PoolSlice* slice, vdbe
   g.dmax = cfg->dmax;
   g.R = (cfg->dmax + 6) / 8;
   g.INF = untrunc ? kNone : cfg->dmax * cfg->dmax;
-  g.half = (!untrunc && cfg->dmax <= 45 && g.R >= 1 && g.R <= 6) ? 1 : 0;  // fp16 fields unless the envelope form is chosen
+  g.windowed = (!untrunc && cfg->dmax <= 45 && g.R >= 1 && g.R <= 6) ? 1 : 0;  // unless the envelope form is chosen
   g.untrunc = untrunc ? 1 : 0;
   uint32_t hcap = 64;
   while ((int64_t)hcap < 2 * node_cap) hcap <<= 1;
@@ -721,11 +721,11 @@ vdbedt_status vdbedt_update(vdbedt_handle h, vdbedt_update_stats* stats) {
     mark(h, 2);
     // slot lists of the dirty runs (an update that switched to the global form got them with its
     // work lists), then the side stream's branch joins before the passes
-    if (half_path(h->g)) CK(h, launch_item_slots(h->g, t, h->items, h->st), "item slots");
+    if (windowed_form(h->g)) CK(h, launch_item_slots(h->g, t, h->items, h->st), "item slots");
     CK(h, cudaStreamWaitEvent(h->st, h->fork.join, 0), "join");
     s = run_passes(h, t, false);
     if (s) return s;
-    if (stats && half_path(h->g))
+    if (stats && windowed_form(h->g))
       CK(h, launch_count_run_bricks(nullptr, h->g, h->g.items_ctr, h->g.item_cap, t, h->items, h->st), "count");
   }
   if (stats) {
@@ -898,11 +898,10 @@ vdbedt_status vdbedt_set_tuning(vdbedt_handle h, const vdbedt_tuning* t) {
   h->tune.run[1] = t->y_run ? t->y_run : d.run[1];
   h->tune.run[2] = t->z_run ? t->z_run : d.run[2];
   h->tune.variant = v ? v : d.variant;
-  // the windowed kernels keep fp16 fields, the envelope kernels 16-bit integers: a change of form
-  // makes the stored intermediates unusable, so the next update recomputes the whole field
-  const int half = (h->cfg.dmax <= 45 && h->g.R >= 1 && h->g.R <= 6 && h->tune.variant != kVariantEnvelope) ? 1 : 0;
-  if (half != h->g.half) {
-    h->g.half = half;
+  // after a change of form the next update recomputes the whole field
+  const int windowed = (h->cfg.dmax <= 45 && h->g.R >= 1 && h->g.R <= 6 && h->tune.variant != kVariantEnvelope) ? 1 : 0;
+  if (windowed != h->g.windowed) {
+    h->g.windowed = windowed;
     h->computed = false;
   }
   return VDBEDT_OK;
@@ -1065,7 +1064,7 @@ vdbedt_status batch_global(vdbedt_batch* b) {
   if (s) return s;
   DeviceGuard guard(b->device);
   const GridView& g0 = b->maps[0]->g;
-  if (!half_path(g0)) {
+  if (!windowed_form(g0)) {
     // the envelope kernels find bricks through each grid's own tables: grid by grid (the phase
     // events then put the whole transform in the last phase)
     for (int i = 0; i < 5; ++i) bmark(b, i);
@@ -1128,7 +1127,7 @@ vdbedt_status batch_update(vdbedt_batch* b, vdbedt_update_stats* stats) {
     // a grid without a field yet: the global transform of the whole batch (applies the records)
     s = batch_global(b);
     if (s) return s;
-  } else if (!half_path(g0)) {
+  } else if (!windowed_form(g0)) {
     // the envelope form: grid by grid
     for (vdbedt_map* m : b->maps) {
       s = vdbedt_update(m, nullptr);
@@ -1140,7 +1139,7 @@ vdbedt_status batch_update(vdbedt_batch* b, vdbedt_update_stats* stats) {
     // The grids' arguments in device memory stay fixed while staging does not reallocate (every
     // grid reads its record count from its device count word), so a captured update replays with
     // the same arguments; they are uploaded again only when they change, outside a capture.
-    BatchUpdShape shape{b->k, 0, 0, g0.R, half_path(g0)};
+    BatchUpdShape shape{b->k, 0, 0, g0.R, windowed_form(g0)};
     BatchCounts counts{};
     std::vector<UpdArgs> args((size_t)b->k);
     for (int i = 0; i < b->k; ++i) {
@@ -1461,7 +1460,7 @@ vdbedt_status vdbedt_batch_set_tuning(vdbedt_batch_handle b, const vdbedt_tuning
     if (s) return bfail(b, s, m->err);
   }
   b->tune = b->maps[0]->tune;
-  if (b->pool.half != b->maps[0]->g.half) {
+  if (b->pool.windowed != b->maps[0]->g.windowed) {
     // the field form changed: the device copy of the grids' views follows
     DeviceGuard guard(b->device);
     std::vector<GridView> views;
@@ -1469,7 +1468,7 @@ vdbedt_status vdbedt_batch_set_tuning(vdbedt_batch_handle b, const vdbedt_tuning
     BCK(b, cudaMemcpyAsync(b->d_views, views.data(), sizeof(GridView) * views.size(), cudaMemcpyHostToDevice, b->st),
         "views");
     BCK(b, cudaStreamSynchronize(b->st), "views");
-    b->pool.half = b->maps[0]->g.half;
+    b->pool.windowed = b->maps[0]->g.windowed;
   }
   return VDBEDT_OK;
 }

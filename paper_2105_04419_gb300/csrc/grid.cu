@@ -22,8 +22,6 @@
 //            runs: x within R along x, in-plane within R in x and y, z within R in x, y and z.
 //   batches  the per-grid kernels take a view source: one grid, or every grid of a batch with
 //            block shares of one launch.
-#include <cuda_fp16.h>
-
 #include "vdbedt_internal.cuh"
 
 namespace vdbedt {
@@ -210,17 +208,8 @@ __device__ __forceinline__ void init_brick_meta(const GridView& g, int slot, int
   g.bepoch[slot] = 0;
 }
 
-// dmax^2 twice in the 16-bit encoding of g1 / g2 (fp16 bits in the windowed form, integers else)
-__device__ __forceinline__ uint32_t field_inf2(const GridView& g) {
-  uint16_t inf;
-  if (g.half) {
-    __half h = __int2half_rn(g.INF);
-    inf = *reinterpret_cast<uint16_t*>(&h);
-  } else {
-    inf = (uint16_t)g.INF;
-  }
-  return (uint32_t)inf | ((uint32_t)inf << 16);
-}
+// dmax^2 twice, as g1 and g2 hold it
+__device__ __forceinline__ uint32_t field_inf2(const GridView& g) { return (uint32_t)g.INF * 0x10001u; }
 
 // g1, g2 and D of `slot` at dmax^2, written by a whole warp (every lane passes the same slot): each
 // store instruction covers 512 contiguous bytes.
@@ -1384,7 +1373,6 @@ __global__ void __launch_bounds__(256) k_items_nodes(VS vs, int rx, int ry, int 
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
   if (vs.skip(g)) return;
-  if (bid == 0 && threadIdx.x == 0) g.counters[C_FORM] = g.half ? kFormHalf : kFormInt;  // what the passes will store
   __shared__ int wsum[8];
   __shared__ int base_sh, count_sh;
   __shared__ int nbr_sh[2];
@@ -2208,7 +2196,7 @@ cudaError_t launch_incremental_mark(const GridView& g, const Tuning& t, const in
   UpdArgs a{};
   a.g = g;
   a.changed = const_cast<int32_t*>(changed);
-  return update_mark_kernels(UpdOne{a}, GatedOne{g}, 1, g.node_cap, g.R, half_path(g), t, it, fk, st);
+  return update_mark_kernels(UpdOne{a}, GatedOne{g}, 1, g.node_cap, g.R, windowed_form(g), t, it, fk, st);
 }
 
 // Batched update: begin + tracked ingest of every grid, then the marking (one launch per step).
@@ -2224,7 +2212,7 @@ cudaError_t launch_update_batch_ingest(const UpdArgs* d_args, const BatchUpdShap
 cudaError_t launch_update_batch_mark(const UpdArgs* d_args, const BatchUpdShape& s, const Tuning& t, const Items& it,
                                      const Fork& fk, cudaStream_t st) {
   if (s.k <= 0) return cudaSuccess;
-  return update_mark_kernels(UpdBatch{d_args}, GatedBatch{d_args}, s.k, (int)s.max_node_cap, s.R, s.half, t, it, fk,
+  return update_mark_kernels(UpdBatch{d_args}, GatedBatch{d_args}, s.k, (int)s.max_node_cap, s.R, s.windowed, t, it, fk,
                              st);
 }
 

@@ -26,22 +26,15 @@
 //     pass axis is 32 words (two voxels per word) and a lane's line is one word per plane, so the
 //     32 lanes of a consumer read 32 consecutive words.
 //
-// Arithmetic of the windowed minimum: packed half2, two voxels per 32-bit lane.  Every operand is
-// an integer in [0, 2048] (values are saturated at dmax^2 <= 2025 for dmax <= 45 before they enter
-// a window, and offsets whose square exceeds 2048 are represented by 2048): fp16 represents each
-// such integer exactly, the sum of two is exact whenever it is below 2048 and rounds to a value
-// >= 2048 otherwise, and min is exact, so every minimum below dmax^2 is computed exactly and every
-// candidate at or above it stays at or above it.  Each lane owns 8 consecutive outputs of two
-// neighbouring lines, pairing offsets +d and -d: acc = min(acc, v[k-d] + d^2, v[k+d] + d^2), two
-// fp16 adds and one three-input minimum taken on the bit patterns as unsigned 16-bit integers
-// (non-negative fp16 values order like their bit patterns).  The pruned form stops when (d + 1)^2
+// Arithmetic of the windowed minimum: 16-bit integers, two voxels per 32-bit lane.  Every value is
+// saturated at dmax^2 <= 2025 before it enters a window and a squared offset is at most 48^2, so a plain
+// 32-bit add sums both halves (no carry between them).  Each lane owns 8 consecutive outputs of two
+// neighbouring lines, pairing offsets +d and -d (window_min8).  The pruned form stops when (d + 1)^2
 // reaches every output's current minimum in the warp, and skips windows whose input bricks hold no
 // value below dmax^2.
 //
 // Grids with dmax above 45 (up to 181), and any grid tuned to variant 8, take the envelope kernels at
 // the end of the file, whose work per voxel follows the distances, not the window.
-#include <cuda_fp16.h>
-
 #include "line_min.cuh"
 #include "vdbedt_internal.cuh"
 
@@ -49,20 +42,8 @@ namespace vdbedt {
 
 namespace {
 
-__device__ __forceinline__ uint32_t h2u(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
-__device__ __forceinline__ __half2 u2h(uint32_t u) { return *reinterpret_cast<__half2*>(&u); }
-
-// fp16 bit pattern of a non-negative integer n (exact for n <= 2048; larger n map to 2048, which
-// is above every saturation value the half kernels use, so such offsets stay irrelevant).
-__host__ __device__ constexpr uint32_t half_bits(int n) {
-  if (n > 2048) n = 2048;
-  if (n == 0) return 0u;
-  int e = 0;
-  while ((1 << (e + 1)) <= n) ++e;
-  uint32_t mant = e <= 10 ? ((uint32_t)(n << (10 - e)) & 0x3FFu) : ((uint32_t)(n >> (e - 10)) & 0x3FFu);
-  return ((uint32_t)(e + 15) << 10) | mant;
-}
-__host__ __device__ constexpr uint32_t half2_bits(int n) { return half_bits(n) | (half_bits(n) << 16); }
+// n in both halves of a word
+__host__ __device__ constexpr uint32_t twice(uint32_t n) { return n * 0x10001u; }
 
 // Sets or clears one bit of a brick's flags with a reduction (no value returned, so the warp does
 // not wait for the word's round trip); each pass owns the bit it writes.
@@ -115,7 +96,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(const GridView& g, uint64_t* b
   return false;
 }
 
-// One 8-output window minimum on packed half2 registers:
+// One 8-output window minimum on packed registers:
 //   out[k] = min over |d| <= W of v[k + W + d] + d^2, pairing +d and -d,
 // where v[j] is plane j of the lane's staged column (c[j * 32]).  Planes are loaded when first
 // needed: the 8 centre planes, then at offset d the two planes that enter the window (W - d and
@@ -123,11 +104,15 @@ __device__ __forceinline__ bool mbar_wait_bounded(const GridView& g, uint64_t* b
 // With `prune`, the offsets stop once (d + 1)^2 is at least every output's current minimum in the
 // warp (a farther candidate costs at least (d + 1)^2, so none can lower any output); the test runs
 // every 4 offsets and is warp-uniform.
+// The eight candidates of four offsets go in as three pairs of adds with a three-way minimum and two fused
+// add-minima: the adds issue beside the minima, so the mix takes 1.4 cycles a candidate where fused
+// add-minima alone take 2.0, adds with three-way minima 1.6 and fp16 adds with them 1.8 (fp16 fields
+// before: y 0.330 and z 0.354 ms, now 0.313 and 0.332; 1024 x 1024 x 256 tunnel scene, dmax 32, runs of 4).
 template <int W>
 __device__ __forceinline__ void window_min8(const uint32_t* __restrict__ c, uint32_t (&out)[8], bool prune) {
   static_assert(W % 4 == 0, "window is a multiple of 4 offsets");
   uint32_t v[8 + 2 * W];
-  uint32_t acc[8];  // fp16x2 bits: non-negative halves order as unsigned 16-bit integers
+  uint32_t acc[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     v[k + W] = c[(k + W) * 32];
@@ -137,24 +122,28 @@ __device__ __forceinline__ void window_min8(const uint32_t* __restrict__ c, uint
 #pragma unroll
   for (int ch = 0; ch < W / 4; ++ch) {
     if (live) {
+      const int d = 4 * ch + 1;  // offsets d .. d + 3
 #pragma unroll
-      for (int dd = 1; dd <= 4; ++dd) {
-        const int d = 4 * ch + dd;
-        v[W - d] = c[(W - d) * 32];
-        v[W + 7 + d] = c[(W + 7 + d) * 32];
-        const __half2 sq = u2h(half2_bits(d * d));
+      for (int dd = 0; dd < 4; ++dd) {
+        v[W - d - dd] = c[(W - d - dd) * 32];
+        v[W + 7 + d + dd] = c[(W + 7 + d + dd) * 32];
+      }
+      constexpr auto sq = [](int n) { return twice((uint32_t)(n * n)); };
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {  // two fp16 adds, one three-way minimum of the bit patterns
-          const uint32_t lo = h2u(__hadd2(u2h(v[k + W - d]), sq)), hi = h2u(__hadd2(u2h(v[k + W + d]), sq));
-          acc[k] = __vimin3_u16x2(acc[k], lo, hi);
-        }
+      for (int k = 0; k < 8; ++k) {
+        uint32_t r = acc[k];
+        r = __vimin3_u16x2(r, v[k + W - d] + sq(d), v[k + W + d] + sq(d));
+        r = __viaddmin_u16x2(v[k + W - d - 1], sq(d + 1), r);
+        r = __vimin3_u16x2(r, v[k + W + d + 1] + sq(d + 1), v[k + W - d - 2] + sq(d + 2));
+        r = __viaddmin_u16x2(v[k + W + d + 2], sq(d + 2), r);
+        r = __vimin3_u16x2(r, v[k + W - d - 3] + sq(d + 3), v[k + W + d + 3] + sq(d + 3));
+        acc[k] = r;
       }
       if (prune && ch + 1 < W / 4) {
-        const int d1 = 4 * ch + 5;  // the next offset
         const uint32_t mx = __vimax3_u16x2(__vimax3_u16x2(acc[0], acc[1], acc[2]), __vimax3_u16x2(acc[3], acc[4], acc[5]),
                                            __vmaxu2(acc[6], acc[7]));
-        const bool done = __hbge2(u2h(half2_bits(d1 * d1)), u2h(mx));
-        live = !__all_sync(0xffffffffu, done);
+        const uint32_t next = sq(d + 4);  // the next offset's square
+        live = !__all_sync(0xffffffffu, __vmaxu2(mx, next) == next);
       }
     }
   }
@@ -175,7 +164,7 @@ struct ColShape {
   static constexpr int THREADS = 32 * (RUN + 1);
   static constexpr size_t DATA_BYTES = (size_t)NS * STAGE_BYTES;
   static constexpr size_t META_BYTES = (size_t)NS * META * 4;
-  static constexpr size_t LUT_BYTES = 80;  // x pass: fp16 bits of min(d^2, dmax^2), d = 0..32
+  static constexpr size_t LUT_BYTES = 80;  // x pass: min(d^2, dmax^2), d = 0..32
   static constexpr size_t SMEM = DATA_BYTES + ((META_BYTES + 15) & ~(size_t)15) + 2 * NS * 8 + LUT_BYTES + 16;
 };
 
@@ -243,7 +232,7 @@ __device__ __forceinline__ void x_compute_rows(const GridView& g, const uint32_t
           const uint32_t Rw = __funnelshift_r(E[r][P >> 5], E[r][(P >> 5) + 1], P & 31);      // bit 0 = P
           const int d = min(__clz(Lw), __clz(__brev(Rw)));  // 32 when the side is empty
           fin |= d < g.dmax;                                  // d^2 < dmax^2
-          hv[x] = lut[d];                                     // fp16 bits of min(d^2, dmax^2)
+          hv[x] = lut[d];                                     // min(d^2, dmax^2)
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) w[r][q] = hv[2 * q] | (hv[2 * q + 1] << 16);
@@ -270,7 +259,7 @@ __device__ __forceinline__ void x_compute_rows(const GridView& g, const uint32_t
       if ((lo[r] | hi[r]) == 0ull) {
         w[r][0] = w[r][1] = w[r][2] = w[r][3] = inf2;
       } else {
-        __half hv[8];
+        uint32_t hv[8];
 #pragma unroll
         for (int x = 0; x < 8; ++x) {
           const int p = 8 * R + x;  // position of voxel x in the line (8 <= p < 64 for 1 <= R <= 6)
@@ -286,10 +275,10 @@ __device__ __forceinline__ void x_compute_rows(const GridView& g, const uint32_t
             best = min(best, dr * dr);
           }
           fin |= best < g.INF;
-          hv[x] = __int2half_rn(best);
+          hv[x] = (uint32_t)best;
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) w[r][q] = h2u(__halves2half2(hv[2 * q], hv[2 * q + 1]));
+        for (int q = 0; q < 4; ++q) w[r][q] = hv[2 * q] | (hv[2 * q + 1] << 16);
       }
     }
   }
@@ -310,7 +299,6 @@ __device__ __forceinline__ void window_compute(const GridView& g, const uint32_t
   constexpr int W = 8 * R;
   const int lane = threadIdx.x & 31;
   const int xp = lane & 3, a = lane >> 2;
-  const __half2 hinf2 = u2h(inf2);
   bool any_fin = !prune;
 #pragma unroll
   for (int b = 0; b <= 2 * R; ++b) any_fin |= fin_flags[w + b] != 0;
@@ -329,17 +317,15 @@ __device__ __forceinline__ void window_compute(const GridView& g, const uint32_t
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       dst[q * 4] = out[q];
-      fin |= !__hbge2(u2h(out[q]), hinf2);
+      fin |= out[q] != inf2;  // every value is at most dmax^2
     }
   } else {
     // D, z-major int32: pair index z * 32 + y * 4 + xpair, here y = a and z = q
     int2* dst = reinterpret_cast<int2*>(g.dist + (size_t)slot * kBrickVox) + a * 4 + xp;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const __half2 h = u2h(out[q]);
-      const int lo = __half2int_rn(__low2half(h)), hi = __half2int_rn(__high2half(h));
-      fin |= (lo < g.INF) | (hi < g.INF);
-      dst[q * 32] = make_int2(lo, hi);
+      fin |= out[q] != inf2;
+      dst[q * 32] = make_int2((int)(out[q] & 0xFFFFu), (int)(out[q] >> 16));
     }
   }
   const unsigned anyfin = __any_sync(0xffffffffu, fin);
@@ -374,18 +360,14 @@ __global__ void __launch_bounds__(32 * (RUN + 1), pass_min_blocks(RUN, AXIS))
   uint16_t* lut = reinterpret_cast<uint16_t*>(empty + NS);
   const int nitems = min(g.items_ctr[AXIS], max_items);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const __half hinf = __int2half_rn(g.INF);
-  const uint32_t inf2 = h2u(__halves2half2(hinf, hinf));
+  const uint32_t inf2 = twice((uint32_t)g.INF);
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], RUN);
     }
   }
-  if (AXIS == 0 && threadIdx.x <= 32) {
-    const __half h = __int2half_rn(min((int)(threadIdx.x * threadIdx.x), g.INF));
-    lut[threadIdx.x] = *reinterpret_cast<const uint16_t*>(&h);
-  }
+  if (AXIS == 0 && threadIdx.x <= 32) lut[threadIdx.x] = (uint16_t)min((int)(threadIdx.x * threadIdx.x), g.INF);
   __syncthreads();
 
   if (warp == 0) {
@@ -470,16 +452,12 @@ __global__ void __launch_bounds__(256) k_x_direct(GridView g, const int32_t* __r
   const int nitems = min(g.items_ctr[0], max_items);
   const int lane = threadIdx.x & 31;
   const int z = lane & 7, y0 = (lane >> 3) * 2;
-  const __half hinf = __int2half_rn(g.INF);
-  const uint32_t inf2 = h2u(__halves2half2(hinf, hinf));
+  const uint32_t inf2 = twice((uint32_t)g.INF);
   const int64_t total = (int64_t)nitems * run;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const unsigned char* occ = reinterpret_cast<const unsigned char*>(g.occ);
   __shared__ uint16_t lut[33];
-  if (threadIdx.x <= 32) {
-    const __half h = __int2half_rn(min((int)(threadIdx.x * threadIdx.x), g.INF));
-    lut[threadIdx.x] = *reinterpret_cast<const uint16_t*>(&h);
-  }
+  if (threadIdx.x <= 32) lut[threadIdx.x] = (uint16_t)min((int)(threadIdx.x * threadIdx.x), g.INF);
   __syncthreads();
   for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += nw) {
     const int item = (int)(w / run), j = (int)(w % run);
@@ -500,7 +478,7 @@ __global__ void __launch_bounds__(256) k_x_direct(GridView g, const int32_t* __r
 // ------------------------------------------------------------------------------------------------
 // Envelope kernels (any dmax up to 181; the only form above 45, variant 8 below it).
 //
-// Fields hold plain 16-bit integers (g1 y-major, g2 z-major, as in the windowed kernels).  A work
+// Fields as in the windowed kernels (16-bit integers, g1 y-major, g2 z-major).  A work
 // item is a run of kEnvRun bricks along the pass axis (a node's length); each kernel finds the
 // run's bricks and their R bricks of halo on each side through the node tables.
 //   x: the distance to the nearest occupied voxel of an x-line, from the line's bits.
@@ -622,7 +600,7 @@ __global__ void __launch_bounds__(kEnvBlock) k_env_line(GridView g, const unsign
   constexpr int nw = kEnvBlock / 32;
   const uint16_t* __restrict__ src = AXIS == 1 ? g.g1 : g.g2;
   const uint32_t in_fin = AXIS == 1 ? F_G1FIN : F_G2FIN;
-  const uint32_t inf2 = (uint32_t)INF | ((uint32_t)INF << 16);
+  const uint32_t inf2 = twice((uint32_t)INF);
   for (int u = t - 8 * NB; u < 8 * NB + 16; u += kEnvBlock) sq[u] = line16_square(u);
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     int bx, by, bz;
@@ -734,7 +712,7 @@ cudaError_t launch_env(const GridView& g, int axis, const Items& it, cudaStream_
 }
 
 template <int R, int RUN, int AXIS>
-cudaError_t pass_half(const GridView& g, const int32_t* islots, int max_items, cudaStream_t st, bool prune) {
+cudaError_t pass_window(const GridView& g, const int32_t* islots, int max_items, cudaStream_t st, bool prune) {
   using S = ColShape<R, RUN, AXIS>;
   auto kernel = k_pass<R, RUN, AXIS>;
   if (max_items <= 0) return cudaSuccess;
@@ -765,25 +743,25 @@ cudaError_t pass_half(const GridView& g, const int32_t* islots, int max_items, c
 }
 
 template <int RUN, int AXIS>
-cudaError_t pass_half_r(const GridView& g, const int32_t* islots, int max_items, cudaStream_t st, bool prune) {
+cudaError_t pass_window_r(const GridView& g, const int32_t* islots, int max_items, cudaStream_t st, bool prune) {
   switch (g.R) {
-    case 1: return pass_half<1, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 2: return pass_half<2, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 3: return pass_half<3, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 4: return pass_half<4, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 5: return pass_half<5, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 6: return pass_half<6, RUN, AXIS>(g, islots, max_items, st, prune);
+    case 1: return pass_window<1, RUN, AXIS>(g, islots, max_items, st, prune);
+    case 2: return pass_window<2, RUN, AXIS>(g, islots, max_items, st, prune);
+    case 3: return pass_window<3, RUN, AXIS>(g, islots, max_items, st, prune);
+    case 4: return pass_window<4, RUN, AXIS>(g, islots, max_items, st, prune);
+    case 5: return pass_window<5, RUN, AXIS>(g, islots, max_items, st, prune);
+    case 6: return pass_window<6, RUN, AXIS>(g, islots, max_items, st, prune);
   }
   return cudaErrorInvalidValue;
 }
 
 template <int AXIS>
-cudaError_t pass_half_run(const GridView& g, int run, const int32_t* islots, int max_items, cudaStream_t st,
+cudaError_t pass_window_run(const GridView& g, int run, const int32_t* islots, int max_items, cudaStream_t st,
                           bool prune) {
   switch (run) {
-    case 4: return pass_half_r<4, AXIS>(g, islots, max_items, st, prune);
-    case 8: return pass_half_r<8, AXIS>(g, islots, max_items, st, prune);
-    case 16: return pass_half_r<16, AXIS>(g, islots, max_items, st, prune);
+    case 4: return pass_window_r<4, AXIS>(g, islots, max_items, st, prune);
+    case 8: return pass_window_r<8, AXIS>(g, islots, max_items, st, prune);
+    case 16: return pass_window_r<16, AXIS>(g, islots, max_items, st, prune);
   }
   return cudaErrorInvalidValue;
 }
@@ -836,11 +814,11 @@ cudaError_t launch_wait_selftest(const GridView& g, int which, cudaStream_t st) 
   return cudaGetLastError();
 }
 
-bool half_path(const GridView& g) { return g.half != 0; }
+bool windowed_form(const GridView& g) { return g.windowed != 0; }
 
-int effective_run(const GridView& g, const Tuning& t, int axis) { return half_path(g) ? t.run[axis] : kEnvRun; }
+int effective_run(const GridView& g, const Tuning& t, int axis) { return windowed_form(g) ? t.run[axis] : kEnvRun; }
 
-// The half kernels address bricks by pool slot (the slot lists hold local slot + slot_base):
+// The windowed kernels address bricks by pool slot (the slot lists hold local slot + slot_base):
 // their view has the per-brick pointers moved back to the first slot of the pool.
 GridView pool_view(const GridView& g) {
   GridView p = g;
@@ -858,12 +836,12 @@ GridView pool_view(const GridView& g) {
 
 cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, cudaStream_t st) {
   const bool prune = (t.variant & 3) != 1;
-  if (half_path(g)) {
+  if (windowed_form(g)) {
     const GridView p = pool_view(g);
     if (axis == 0 && (t.variant & kVariantXDirect)) return x_direct(p, it.slots[0], g.item_cap, t.run[0], st);
-    if (axis == 0) return pass_half_run<0>(p, t.run[0], it.slots[0], g.item_cap, st, prune);
-    if (axis == 1) return pass_half_run<1>(p, t.run[1], it.slots[1], g.item_cap, st, prune);
-    return pass_half_run<2>(p, t.run[2], it.slots[2], g.item_cap, st, prune);
+    if (axis == 0) return pass_window_run<0>(p, t.run[0], it.slots[0], g.item_cap, st, prune);
+    if (axis == 1) return pass_window_run<1>(p, t.run[1], it.slots[1], g.item_cap, st, prune);
+    return pass_window_run<2>(p, t.run[2], it.slots[2], g.item_cap, st, prune);
   }
   // the envelope kernels find bricks through the grid's own tables (local slots)
   return launch_env(g, axis, it, st);

@@ -12,8 +12,6 @@
 // Backward: dc/dp = -2 max(0, tau - d) (1 / vs) grad_t(trilinear), scaled by the upstream
 // gradient of the trajectory's cost.  One warp per trajectory, points strided over the lanes,
 // a warp shuffle sum for the forward.
-#include <cuda_fp16.h>
-
 #include "vdbedt_internal.cuh"
 
 namespace vdbedt {
@@ -121,7 +119,7 @@ __device__ __forceinline__ int isqrt_floor(int v) {
 // field g2) through (x, y, z) with field(o) = want - (o - c)^2, its value in `rest`; -1: none.  A
 // brick's eight values are loaded together (planes 128 B apart: a sector each).
 template <int AXIS>
-__device__ __forceinline__ int line_match(const GridView& g, int x, int y, int z, int want, bool half, NodeCache& nc,
+__device__ __forceinline__ int line_match(const GridView& g, int x, int y, int z, int want, NodeCache& nc,
                                           int& rest) {
   const int c = AXIS == 1 ? y : z, n = AXIS == 1 ? g.ny : g.nz, r = isqrt_floor(want);
   const int b1 = min(c + r, n - 1) >> 3;
@@ -136,7 +134,7 @@ __device__ __forceinline__ int line_match(const GridView& g, int x, int y, int z
     int at = -1;
 #pragma unroll
     for (int q = 7; q >= 0; --q) {
-      const int d = 8 * b + q - c, f = half ? __half2int_rn(__ushort_as_half(v[q])) : (int)v[q];
+      const int d = 8 * b + q - c, f = (int)v[q];
       if (f == want - d * d) {
         at = 8 * b + q;
         rest = f;
@@ -157,7 +155,6 @@ __device__ __forceinline__ int line_match(const GridView& g, int x, int y, int z
 // the sphere in (z, y, x) order and testing occupancy bits: 3.7 ms).
 __global__ void __launch_bounds__(128) k_query_nearest(GridView g, const int32_t* __restrict__ xyz, int64_t n,
                                                        int32_t* __restrict__ out) {
-  const bool half = g.counters[C_FORM] == kFormHalf;  // of the fields as stored
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int x = xyz[3 * i] + g.off, y = xyz[3 * i + 1] + g.off, z = xyz[3 * i + 2] + g.off;
     int rx = -1 + g.off, ry = -1 + g.off, rz = -1 + g.off;
@@ -167,8 +164,8 @@ __global__ void __launch_bounds__(128) k_query_nearest(GridView g, const int32_t
       const int D = s >= 0 ? g.dist[(size_t)s * kBrickVox + (x & 7) + 8 * (y & 7) + 64 * (z & 7)] : g.INF;
       if ((unsigned)D < (unsigned)g.INF) {
         int plane = 0, dx2 = 0, oy = -1;
-        const int oz = line_match<2>(g, x, y, z, D, half, nc, plane);
-        if (oz >= 0) oy = line_match<1>(g, x, y, oz, plane, half, nc, dx2);
+        const int oz = line_match<2>(g, x, y, z, D, nc, plane);
+        if (oz >= 0) oy = line_match<1>(g, x, y, oz, plane, nc, dx2);
         bool found = false;
         if (oy >= 0) {
           const int dx = isqrt_floor(dx2);

@@ -63,15 +63,13 @@ enum Counter : int {
   C_OBST = 12,
   C_NB_START = 13,  // stored bricks when the running update began (its global-vs-incremental choice)
   C_EPOCH = 14,  // incremental update epoch (run and brick dedupe marks)
-  C_FORM = 15,  // encoding of the g1 / g2 fields as stored (kForm*; 0: none yet), written by each global form
+  C_SPARE = 15,  // unused
   C_XB = 16,  // stored bricks in the update's dirty runs per axis (x, y, z: three consecutive words)
   C_YB = 17,
   C_ZB = 18,
   C_BIG = 19,  // this update's edits reach so far that it takes the global form after applying them
   C_NUM = 20
 };
-
-constexpr int kFormHalf = 1, kFormInt = 2;  // fp16 bit patterns; 16-bit integers
 
 // brick flags
 constexpr uint32_t F_OBST = 1u;    // holds an occupied voxel
@@ -84,8 +82,7 @@ struct GridView {
   int BX, BY, BZ;     // bricks per axis
   int NX, NY, NZ;     // nodes per axis
   int dmax, R, INF;   // truncation, brick radius of influence, dmax^2
-  int half;           // 1: g1 / g2 hold fp16 bit patterns (windowed kernels, dmax <= 45); 0: 16-bit
-                      // integers (lower-envelope kernels)
+  int windowed;       // 1: windowed kernels (dmax <= 45, runs with slot lists); 0: envelope kernels
   int off;            // added to caller coordinates (0; kUnboundedOffset for an unbounded grid)
   int unbounded;      // 1: no per-node-key arrays (nodes are created where records fall)
   int untrunc;        // 1: no truncation; every brick stored at slot bx + BX (by + BY bz), g1 / g2 hold
@@ -311,7 +308,7 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     ::vdbedt::launch_pdl(kernel, dim3(grid), dim3(block), (smem), (stream), __VA_ARGS__); \
   } while (0)
 
-constexpr int kItemSlots = 32;  // slot list entries per work item (run + 2R <= 28 on the half path)
+constexpr int kItemSlots = 32;  // slot list entries per work item (run + 2R <= 28 in the windowed form)
 constexpr int kBatchMax = 1024;  // grids per batch (the dense-ingest source table is a kernel parameter)
 
 // Tuning.variant: low bits 1 = full windowed minimum, 3 = windowed minimum with early exit and
@@ -327,7 +324,7 @@ struct Tuning {
   int variant = 3;
 };
 
-// Work lists of the passes: runs of bricks along each axis, and (half path) the slots of each
+// Work lists of the passes: runs of bricks along each axis, and (windowed form) the slots of each
 // run's bricks with their halo of R bricks on both sides.
 struct Items {
   unsigned long long* run[3];  // packed brick coordinates of the first brick of each run
@@ -394,7 +391,7 @@ cudaError_t launch_begin_update(const GridView& g, cudaStream_t st);
 size_t dense_scratch_bytes(const GridView& g);
 cudaError_t launch_ingest_dense(const GridView& g, const uint8_t* grid, Scratch& scr, cudaStream_t st);
 cudaError_t launch_activation_full(const GridView& g, cudaStream_t st);
-// every run holding a stored brick, with slot lists when with_slots (half path)
+// every run holding a stored brick, with slot lists when with_slots (windowed form)
 cudaError_t launch_build_items_full(const GridView& g, const Tuning& t, const Items& it, bool with_slots,
                                     cudaStream_t st);
 // A side stream for the update's two alternative branches: the global form's activation and work
@@ -416,7 +413,7 @@ struct BatchUpdShape {
   int k;
   int64_t max_n, max_node_cap;
   int R;      // common to the batch
-  bool half;  // the windowed form (work lists carry slot lists)
+  bool windowed;  // the windowed form (work lists carry slot lists)
 };
 // record counts of the grids staged without a device count (-1: the grid's count word is already
 // written), passed by value to the first kernel
@@ -445,7 +442,7 @@ cudaError_t launch_ut_pass(const GridView& g, int axis, void* scratch, cudaStrea
 // voxel; y, z: lines whose input changed), marking the next axis's lines where its output changed;
 // lines recomputed are counted in items_ctr[axis].  The z pass also refreshes the brick flags.
 cudaError_t launch_ut_update_pass(const GridView& g, int axis, void* scratch, cudaStream_t st);
-// slot lists of every queued run (half path)
+// slot lists of every queued run (windowed form)
 cudaError_t launch_item_slots(const GridView& g, const Tuning& t, const Items& it, cudaStream_t st);
 
 // The same steps for every grid of a batch at once: one launch per step (views: device array of
@@ -475,7 +472,7 @@ cudaError_t launch_build_items_batch(const GridView* views, const BatchShape& b,
                                      int32_t* items_ctr, cudaStream_t st);
 
 // passes (passes.cu)
-bool half_path(const GridView& g);
+bool windowed_form(const GridView& g);
 // pass along `axis` (0 x, 1 y, 2 z) over the queued runs
 cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, cudaStream_t st);
 int effective_run(const GridView& g, const Tuning& t, int axis);
