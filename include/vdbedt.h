@@ -393,6 +393,14 @@ vdbedt_status vdbedt_get_info(vdbedt_handle h, vdbedt_info* info);
 /* The handle's stream (cudaStream_t). */
 void* vdbedt_stream(vdbedt_handle h);
 
+/* Ordering against another stream of the handle's device (cudaStream_t, null: the default stream), without
+ * waiting on the host: vdbedt_wait_stream makes the handle's later work wait for what is queued on
+ * `stream` now (inputs produced there); vdbedt_join_stream makes later work on `stream` wait for what is
+ * queued on the handle's stream now (results used there).  Any thread; works under stream capture as an
+ * event recorded on one stream and waited for on the other does. */
+vdbedt_status vdbedt_wait_stream(vdbedt_handle h, void* stream);
+vdbedt_status vdbedt_join_stream(vdbedt_handle h, void* stream);
+
 /* Last error message for the handle (or for handle-less failures when h is NULL); never NULL. */
 const char* vdbedt_last_error(vdbedt_handle h);
 

@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -70,6 +71,8 @@ struct vdbedt_map {
   cudaEvent_t ev[7] = {};
   bool ev_recorded = false;
   Fork fork;  // side stream of the update's global-form branch
+  cudaEvent_t order = nullptr;  // vdbedt_wait_stream / vdbedt_join_stream
+  std::mutex order_lock;        // an event is waited for as it was last recorded: the pair is one step
 };
 
 namespace {
@@ -365,6 +368,7 @@ vdbedt_status create_impl(const vdbedt_config* cfg, const PoolSlice* slice, vdbe
     if (h->fork.side) cudaStreamDestroy(h->fork.side);
     if (h->fork.fork) cudaEventDestroy(h->fork.fork);
     if (h->fork.join) cudaEventDestroy(h->fork.join);
+    if (h->order) cudaEventDestroy(h->order);
     if (h->own_stream && h->st) cudaStreamDestroy(h->st);
     delete h;
     return s;
@@ -380,6 +384,7 @@ vdbedt_status create_impl(const vdbedt_config* cfg, const PoolSlice* slice, vdbe
   e = cudaStreamCreateWithFlags(&h->fork.side, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->fork.fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->fork.join, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->order, cudaEventDisableTiming);
   if (e != cudaSuccess) return bail(e, "side stream");
 #define AL(ptr, count)                                   \
   do {                                                   \
@@ -481,6 +486,7 @@ void destroy_impl(vdbedt_map* h) {
   if (h->fork.side) cudaStreamDestroy(h->fork.side);
   if (h->fork.fork) cudaEventDestroy(h->fork.fork);
   if (h->fork.join) cudaEventDestroy(h->fork.join);
+  if (h->order) cudaEventDestroy(h->order);
   if (h->own_stream) cudaStreamDestroy(h->st);
   delete h;
 }
@@ -938,6 +944,26 @@ vdbedt_status vdbedt_get_info(vdbedt_handle h, vdbedt_info* info) {
 }
 
 void* vdbedt_stream(vdbedt_handle h) { return h ? (void*)h->st : nullptr; }
+
+vdbedt_status vdbedt_wait_stream(vdbedt_handle h, void* stream) {
+  vdbedt_status s = check_handle(h);
+  if (s) return s;
+  DeviceGuard guard(h->device);
+  std::lock_guard<std::mutex> one(h->order_lock);
+  CK(h, cudaEventRecord(h->order, (cudaStream_t)stream), "wait stream");
+  CK(h, cudaStreamWaitEvent(h->st, h->order, 0), "wait stream");
+  return VDBEDT_OK;
+}
+
+vdbedt_status vdbedt_join_stream(vdbedt_handle h, void* stream) {
+  vdbedt_status s = check_handle(h);
+  if (s) return s;
+  DeviceGuard guard(h->device);
+  std::lock_guard<std::mutex> one(h->order_lock);
+  CK(h, cudaEventRecord(h->order, h->st), "join stream");
+  CK(h, cudaStreamWaitEvent((cudaStream_t)stream, h->order, 0), "join stream");
+  return VDBEDT_OK;
+}
 
 vdbedt_status vdbedt_set_profiling(vdbedt_handle h, int on) {
   vdbedt_status s = check_handle(h);

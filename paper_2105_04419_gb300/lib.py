@@ -90,6 +90,8 @@ SIGNATURES = {
     "vdbedt_synchronize": (ctypes.c_int, [_H]),
     "vdbedt_get_info": (ctypes.c_int, [_H, ctypes.POINTER(Info)]),
     "vdbedt_stream": (ctypes.c_void_p, [_H]),
+    "vdbedt_wait_stream": (ctypes.c_int, [_H, ctypes.c_void_p]),
+    "vdbedt_join_stream": (ctypes.c_int, [_H, ctypes.c_void_p]),
     "vdbedt_set_profiling": (ctypes.c_int, [_H, ctypes.c_int]),
     "vdbedt_get_phase_times": (ctypes.c_int, [_H, ctypes.POINTER(PhaseTimes)]),
     "vdbedt_kernel_launches": (ctypes.c_int64, []),
@@ -106,6 +108,8 @@ def library_path() -> str:
 def load():
     """Load libvdbedt.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(_SO):
@@ -128,6 +132,13 @@ def _check(status, where, handle=None):
 def _torch():
     import torch
     return torch
+
+
+def _flat(t, dtype, cols: int = 0):
+    """t as a contiguous tensor of `dtype`, [n, cols] (cols 0: [n]); t itself when it is one already."""
+    if t.dtype is dtype and t.is_contiguous() and (t.dim() == 1 if not cols else t.dim() == 2 and t.shape[1] == cols):
+        return t
+    return t.to(dtype).contiguous().view(-1, cols) if cols else t.to(dtype).contiguous().view(-1)
 
 
 def _ptr_host(a: np.ndarray) -> int:
@@ -192,6 +203,7 @@ class Map:
         if _borrow is not None:
             # a grid of a Batch: the batch owns the handle and the stream
             self._h, self.stream, self._owned = _borrow, stream, False
+            self._raw_stream = stream.cuda_stream
             self.device, self.shape_xyz, self.dmax, self.voxel_size = device, (nx, ny, nz), dmax, voxel_size
             return
         self._owned = True
@@ -201,6 +213,7 @@ class Map:
             stream = torch.cuda.Stream(device)
         self.device = device
         self.stream = stream
+        self._raw_stream = stream.cuda_stream
         flags = (FLAG_UNBOUNDED if unbounded else 0) | (FLAG_UNTRUNCATED if untruncated else 0)
         cfg = Config(nx, ny, nz, 0 if untruncated else dmax, voxel_size, device, ctypes.c_void_p(stream.cuda_stream),
                      flags, max_bricks, max_nodes)
@@ -234,20 +247,19 @@ class Map:
     def _enter(self, *tensors):
         torch = _torch()
         for t in tensors:  # device pointers go to the library: CPU tensors or another GPU's are refused
-            if not isinstance(t, torch.Tensor) or not t.is_cuda or t.device.index != self.device:
+            if not isinstance(t, torch.Tensor) or not t.is_cuda or t.get_device() != self.device:
                 where = t.device if isinstance(t, torch.Tensor) else type(t).__name__
                 raise ValueError(f"expected a CUDA tensor on cuda:{self.device}, got {where}")
-        cur = torch.cuda.current_stream(self.device)
-        if cur.cuda_stream != self.stream.cuda_stream:
-            self.stream.wait_stream(cur)
+        cur = torch._C._cuda_getCurrentRawStream(self.device)
+        if cur != self._raw_stream:
+            _check(_lib.vdbedt_wait_stream(self._h, cur), "vdbedt_wait_stream", self._h)
         for t in tensors:
             t.record_stream(self.stream)
 
     def _leave(self):
-        torch = _torch()
-        cur = torch.cuda.current_stream(self.device)
-        if cur.cuda_stream != self.stream.cuda_stream:
-            cur.wait_stream(self.stream)
+        cur = _torch()._C._cuda_getCurrentRawStream(self.device)
+        if cur != self._raw_stream:
+            _check(_lib.vdbedt_join_stream(self._h, cur), "vdbedt_join_stream", self._h)
 
     # -- occupancy --
     def set_occupancy(self, xyz, occ):
@@ -262,8 +274,8 @@ class Map:
                    "vdbedt_set_occupancy", self._h)
         else:
             torch = _torch()
-            x = xyz.to(torch.int32).contiguous().view(-1, 3)
-            o = occ.to(torch.uint8).contiguous().view(-1)
+            x = _flat(xyz, torch.int32, 3)
+            o = _flat(occ, torch.uint8)
             if x.shape[0] != o.shape[0]:
                 raise ValueError(f"{x.shape[0]} coordinates but {o.shape[0]} occupancy values")
             self._enter(x, o)
@@ -374,7 +386,7 @@ class Map:
             _check(lib.vdbedt_query(self._h, _ptr_host(x), x.shape[0], _ptr_host(out), 0), "vdbedt_query", self._h)
             return out
         torch = _torch()
-        x = xyz.to(torch.int32).contiguous().view(-1, 3)
+        x = _flat(xyz, torch.int32, 3)
         out = torch.empty(x.shape[0], dtype=torch.int32, device=x.device)
         self._enter(x, out)
         _check(lib.vdbedt_query(self._h, x.data_ptr(), x.shape[0], out.data_ptr(), 1), "vdbedt_query", self._h)
@@ -392,7 +404,7 @@ class Map:
                    "vdbedt_query_nearest", self._h)
             return out
         torch = _torch()
-        x = xyz.to(torch.int32).contiguous().view(-1, 3)
+        x = _flat(xyz, torch.int32, 3)
         out = torch.empty_like(x)
         self._enter(x, out)
         _check(lib.vdbedt_query_nearest(self._h, x.data_ptr(), x.shape[0], out.data_ptr(), 1), "vdbedt_query_nearest",

@@ -1,0 +1,51 @@
+"""Ordering between the caller's current torch stream and the map's own: inputs still being produced when the
+call is made, and results used right after it, from a side stream, the default stream and two threads."""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+def session(V, torch, seed, out):
+    rs = np.random.default_rng(seed)
+    side = torch.cuda.Stream()
+    m = V.Map(40, 33, 27, 9)
+    occ = np.zeros((27, 33, 40), np.uint8)
+    ok = True
+    for frame in range(6):
+        xyz = np.stack([rs.integers(0, n, 30) for n in (40, 33, 27)], 1).astype(np.int32)
+        val = rs.integers(0, 2, 30).astype(np.uint8)
+        for (x, y, z), v in zip(xyz, val):
+            occ[z, y, x] = v
+        host = torch.from_numpy(xyz).pin_memory(), torch.from_numpy(val).pin_memory()
+        with torch.cuda.stream(side if frame % 2 else torch.cuda.default_stream()):
+            a, b = torch.zeros((30, 3), dtype=torch.int32, device="cuda"), torch.zeros(30, dtype=torch.uint8, device="cuda")
+            torch.cuda._sleep(2_000_000)  # about a millisecond: the call below is made before the inputs are there
+            a.copy_(host[0], non_blocking=True)
+            b.copy_(host[1], non_blocking=True)
+            m.set_occupancy(a, b)
+            m.update()
+            d = m.export_dense(on_device=True)
+            total = d.sum()  # ordered behind the export by the call itself
+            torch.cuda.current_stream().synchronize()
+            ref = O.edt_factorised(occ, 9)
+            ok &= bool(np.array_equal(d.cpu().numpy(), ref)) and int(total) == int(ref.sum())
+    m.close()
+    out.append(ok)
+
+
+def test_caller_streams():
+    import torch
+    import paper_2105_04419_gb300 as V
+    out = []
+    threads = [threading.Thread(target=session, args=(V, torch, s, out)) for s in (1, 2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    session(V, torch, 3, out)
+    assert out == [True, True, True]
