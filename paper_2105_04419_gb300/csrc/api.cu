@@ -214,14 +214,14 @@ Tuning effective_tuning(const vdbedt_map* h) {
   return t;
 }
 
-vdbedt_status run_passes(vdbedt_map* h, const Tuning& t, bool need_slots) {
-  if (need_slots && windowed_form(h->g)) CK(h, launch_item_slots(h->g, t, h->items, h->st), "item slots");
+// joined: another stream's work joined just before (the x pass then waits for both as a whole)
+vdbedt_status run_passes(vdbedt_map* h, const Tuning& t, bool joined) {
   mark(h, 3);
-  CK(h, launch_pass(h->g, t, 0, h->items, h->st), "x pass");
+  CK(h, launch_pass(h->g, t, 0, h->items, !joined, h->st), "x pass");
   mark(h, 4);
-  CK(h, launch_pass(h->g, t, 1, h->items, h->st), "y pass");
+  CK(h, launch_pass(h->g, t, 1, h->items, true, h->st), "y pass");
   mark(h, 5);
-  CK(h, launch_pass(h->g, t, 2, h->items, h->st), "z pass");
+  CK(h, launch_pass(h->g, t, 2, h->items, true, h->st), "z pass");
   mark(h, 6);
   h->ev_recorded = h->profiling && !capturing(h);
   return VDBEDT_OK;
@@ -237,8 +237,8 @@ void clear_stage(vdbedt_map* h) {
 vdbedt_status do_global(vdbedt_map* h) {
   const Tuning t = effective_tuning(h);
   mark(h, 0);
-  CK(h, cudaMemsetAsync(h->g.counters + C_HAS_ZERO, 0, sizeof(int32_t), h->st), "memset");
   if (h->stage_n > 0) {
+    CK(h, cudaMemsetAsync(h->g.counters + C_UNIQUE, 0, 2 * sizeof(int32_t), h->st), "memset");  // and C_HAS_ZERO
     CK(h,
        launch_ingest_records(h->g, h->stage, h->stage_n, stage_count(h), false, h->changed, h->stage_slot, h->scr,
                              h->vlast, h->st),
@@ -643,12 +643,18 @@ vdbedt_status vdbedt_set_occupancy_dense(vdbedt_handle h, const uint8_t* grid, i
   if (!grid) return fail(h, VDBEDT_EINVAL, "null grid");
   if (h->g.unbounded) return fail(h, VDBEDT_EINVAL, "an unbounded grid has no dense form");
   DeviceGuard guard(h->device);
-  s = vdbedt_reset(h);
-  if (s) return s;
+  const size_t bytes = (size_t)h->g.nx * h->g.ny * h->g.nz;
+  cudaError_t e = on_device ? cudaSuccess : ensure_scratch(h->io, bytes);
+  if (e == cudaSuccess && !h->g.untrunc) e = ensure_scratch(h->scr, dense_scratch_bytes(h->g));
+  if (e != cudaSuccess || h->g.untrunc) {  // (the sparse form's ingest resets the grid itself)
+    s = vdbedt_reset(h);
+    if (s) return s;
+    if (e != cudaSuccess) return cuda_fail(h, e, "io alloc");
+  }
+  clear_stage(h);
+  h->computed = false;
   const uint8_t* src = grid;
   if (!on_device) {
-    size_t bytes = (size_t)h->g.nx * h->g.ny * h->g.nz;
-    CK(h, ensure_scratch(h->io, bytes), "io alloc");
     CK(h, cudaMemcpyAsync(h->io.buf, grid, bytes, cudaMemcpyHostToDevice, h->st), "h2d");
     src = (const uint8_t*)h->io.buf;
   }
@@ -729,7 +735,7 @@ vdbedt_status vdbedt_update(vdbedt_handle h, vdbedt_update_stats* stats) {
     // work lists), then the side stream's branch joins before the passes
     if (windowed_form(h->g)) CK(h, launch_item_slots(h->g, t, h->items, h->st), "item slots");
     CK(h, cudaStreamWaitEvent(h->st, h->fork.join, 0), "join");
-    s = run_passes(h, t, false);
+    s = run_passes(h, t, true);
     if (s) return s;
     if (stats && windowed_form(h->g))
       CK(h, launch_count_run_bricks(nullptr, h->g, h->g.items_ctr, h->g.item_cap, t, h->items, h->st), "count");
@@ -1108,7 +1114,7 @@ vdbedt_status batch_global(vdbedt_batch* b) {
   // staged records: applied grid by grid (the sort-based ingest keeps per-grid scratch)
   for (vdbedt_map* m : b->maps) {
     if (m->stage_n <= 0) continue;
-    BCK(b, cudaMemsetAsync(m->g.counters + C_HAS_ZERO, 0, sizeof(int32_t), b->st), "memset");
+    BCK(b, cudaMemsetAsync(m->g.counters + C_UNIQUE, 0, 2 * sizeof(int32_t), b->st), "memset");  // and C_HAS_ZERO
     BCK(b,
         launch_ingest_records(m->g, m->stage, m->stage_n, stage_count(m), false, nullptr, m->stage_slot, m->scr,
                               m->vlast, b->st),
@@ -1118,12 +1124,12 @@ vdbedt_status batch_global(vdbedt_batch* b) {
   bmark(b, 1);
   BCK(b, launch_activation_batch(b->d_views, b->shape, b->st), "activation");
   bmark(b, 2);
-  BCK(b, launch_build_items_batch(b->d_views, b->shape, t, b->items, b->pool.items_ctr, b->st), "items");
+  BCK(b, launch_build_items_batch(b->d_views, b->shape, t, b->items, b->st), "items");
   bmark(b, 3);
-  BCK(b, launch_pass(b->pool, t, 0, b->items, b->st), "x pass");
+  BCK(b, launch_pass(b->pool, t, 0, b->items, true, b->st), "x pass");
   bmark(b, 4);
-  BCK(b, launch_pass(b->pool, t, 1, b->items, b->st), "y pass");
-  BCK(b, launch_pass(b->pool, t, 2, b->items, b->st), "z pass");
+  BCK(b, launch_pass(b->pool, t, 1, b->items, true, b->st), "y pass");
+  BCK(b, launch_pass(b->pool, t, 2, b->items, true, b->st), "z pass");
   bmark(b, 5);
   b->ev_recorded = b->profiling;
   for (vdbedt_map* m : b->maps) {
@@ -1201,10 +1207,10 @@ vdbedt_status batch_update(vdbedt_batch* b, vdbedt_update_stats* stats) {
     bmark(b, 2);
     BCK(b, launch_item_slots_batch(b->d_views, t, b->items, b->pool.items_ctr, b->pool.item_cap, b->st), "item slots");
     bmark(b, 3);
-    BCK(b, launch_pass(b->pool, t, 0, b->items, b->st), "x pass");
+    BCK(b, launch_pass(b->pool, t, 0, b->items, false, b->st), "x pass");
     bmark(b, 4);
-    BCK(b, launch_pass(b->pool, t, 1, b->items, b->st), "y pass");
-    BCK(b, launch_pass(b->pool, t, 2, b->items, b->st), "z pass");
+    BCK(b, launch_pass(b->pool, t, 1, b->items, true, b->st), "y pass");
+    BCK(b, launch_pass(b->pool, t, 2, b->items, true, b->st), "z pass");
     bmark(b, 5);
     b->ev_recorded = b->profiling;
     if (stats)
@@ -1579,6 +1585,7 @@ namespace {
 __global__ void k_pack_records(const int32_t* __restrict__ xyz, const uint8_t* __restrict__ occ, int64_t n_max,
                                const int32_t* n_dev, int32_t* count_out, int nx, int ny, int nz, int off,
                                rec_t* __restrict__ dst, int32_t* invalid, int32_t* counters) {
+  pdl_enter();
   int64_t n = n_max;
   if (n_dev) {
     const int64_t c = *n_dev;
@@ -1739,7 +1746,7 @@ cudaError_t launch_pack_records(const int32_t* xyz, const uint8_t* occ, int64_t 
   int64_t b = (n + 255) / 256;
   if (b > 152 * 16) b = 152 * 16;
   if (b < 1) b = 1;
-  VDB_LAUNCH(k_pack_records, (unsigned)b, 256, 0, st, xyz, occ, n, n_dev, count_out, nx, ny, nz, off, dst, invalid,
+  VDB_LAUNCH_PDL(k_pack_records, (unsigned)b, 256, 0, st, xyz, occ, n, n_dev, count_out, nx, ny, nz, off, dst, invalid,
              counters);
   return cudaGetLastError();
 }

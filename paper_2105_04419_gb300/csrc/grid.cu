@@ -129,8 +129,9 @@ struct UpdBatch {
 };
 
 // ---- reset ----
+// clear, clear_words: more words to set to zero (a dense ingest's node flags)
 template <class VS>
-__global__ void k_reset_nodes(VS vs) {
+__global__ void k_reset_nodes(VS vs, int32_t* __restrict__ clear, int64_t clear_words) {
   pdl_enter();
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
@@ -146,6 +147,7 @@ __global__ void k_reset_nodes(VS vs) {
   for (int64_t i = t0; i < nn * (384 / 4); i += stride) reinterpret_cast<int4*>(g.mwork)[i] = zero;
   for (int64_t i = t0; i < nn * (128 / 4); i += stride) reinterpret_cast<int4*>(g.nclaim)[i] = zero;
   for (int64_t i = t0; i <= (int64_t)g.hmask; i += stride) g.hslots[i] = ~0ull;
+  for (int64_t i = t0; i < clear_words; i += stride) clear[i] = 0;
 }
 
 // Start of an incremental update: clear the per-update counters and advance the update epoch
@@ -852,9 +854,11 @@ struct DenseScratch {
 constexpr int kDenseX = 64;
 
 template <class VS, class SRC>
-__global__ void __launch_bounds__(256, 4) k_dense_masks(VS vs, SRC src, DenseScratch ds) {
+__global__ void __launch_bounds__(256, 4) k_dense_masks(VS vs, SRC src, DenseScratch ds, bool zero_counters) {
+  pdl_enter();
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
+  if (zero_counters && bid == 0 && (int)threadIdx.x < C_NUM) g.counters[threadIdx.x] = 0;
   const uint8_t* __restrict__ grid = src.get(gi);
   unsigned long long* dbits;
   int32_t* flag;
@@ -939,6 +943,7 @@ __global__ void __launch_bounds__(256, 4) k_dense_masks(VS vs, SRC src, DenseScr
 // from one atomic per block): no insertion ever waits on another.
 template <class VS>
 __global__ void __launch_bounds__(256) k_dense_nodes(VS vs, DenseScratch ds) {
+  pdl_enter();
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
   unsigned long long* dbits;
@@ -960,6 +965,7 @@ __global__ void __launch_bounds__(256) k_dense_nodes(VS vs, DenseScratch ds) {
 
 template <class VS>
 __global__ void __launch_bounds__(256) k_dense_alloc(VS vs, DenseScratch ds) {
+  pdl_enter();
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
   unsigned long long* dbits;
@@ -999,24 +1005,6 @@ __global__ void __launch_bounds__(256) k_dense_alloc(VS vs, DenseScratch ds) {
 // 4096-bit masks, obstacle bits first, then a separable dilation (x, then y, then z), each stage a
 // pure gather over neighbouring nodes' rows (no atomics).  A mask word holds two 16-brick x-rows:
 // word (y >> 1) + 8 z, bits 16 (y & 1) + x.
-
-template <class VS>
-__global__ void k_clear_masks(VS vs) {
-  pdl_enter();
-  int bid, nblk, gi;
-  const GridView g = vs.get(bid, nblk, gi);
-  if (vs.skip(g)) return;
-  (void)gi;
-  const int nn = min(g.counters[C_NNODES], g.node_cap);
-  for (int64_t i = (int64_t)bid * blockDim.x + threadIdx.x; i < (int64_t)nn * 128;
-       i += (int64_t)nblk * blockDim.x) {
-    g.amask[i] = 0u;
-    int64_t node = i >> 7, w = i & 127;
-    g.mwork[node * 384 + w] = 0u;
-    g.mwork[node * 384 + 128 + w] = 0u;
-    g.mwork[node * 384 + 256 + w] = 0u;
-  }
-}
 
 template <class VS>
 __global__ void k_obstacle_flags(VS vs) {
@@ -1285,17 +1273,21 @@ __device__ void alloc_new_bits(const GridView& g, int node, int word, uint32_t b
 }
 
 // Allocate every marked brick without storage: a block per (node, 256-brick chunk), a brick per
-// thread, one atomic per block for the slot range (block scan of the flags).
+// thread, one atomic per block for the slot range (block scan of the flags).  It is the last to run before
+// the work lists and after the dilation, so it also puts the obstacle masks back to zero (they are zero
+// whenever an activation begins) and, in the global form, the work lists' counters.
 template <class VS>
-__global__ void __launch_bounds__(256) k_alloc_marked(VS vs, bool init_fields) {
+__global__ void __launch_bounds__(256) k_alloc_marked(VS vs, bool zero_items) {
   pdl_enter();
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
   if (vs.skip(g)) return;
   (void)gi;
   const int nn = min(g.counters[C_NNODES], g.node_cap);
+  if (zero_items && bid == 0 && threadIdx.x < 3) g.items_ctr[threadIdx.x] = 0;
   for (int b = bid; b < nn * 16; b += nblk) {
     const int node = b >> 4, l = (b & 15) * 256 + threadIdx.x;
+    if (threadIdx.x < 8) g.mwork[(size_t)node * 384 + (b & 15) * 8 + threadIdx.x] = 0u;
     const bool need = ((g.amask[(size_t)node * 128 + (l >> 5)] >> (l & 31)) & 1u) &&
                       g.child[(size_t)node * kNodeBricks + l] == kNoSlot;
     int total = 0;
@@ -1307,7 +1299,7 @@ __global__ void __launch_bounds__(256) k_alloc_marked(VS vs, bool init_fields) {
       } else {
         int nxn, nyn, nzn;
         node_coords(g, (unsigned long long)g.node_key[node], nxn, nyn, nzn);
-        init_brick(g, slot, node, nxn * 16 + (l & 15), nyn * 16 + ((l >> 4) & 15), nzn * 16 + (l >> 8), init_fields);
+        init_brick(g, slot, node, nxn * 16 + (l & 15), nyn * 16 + ((l >> 4) & 15), nzn * 16 + (l >> 8), false);
         g.child[(size_t)node * kNodeBricks + l] = slot;
       }
     }
@@ -1850,8 +1842,7 @@ cudaError_t update_mark_kernels(US us, GV gv, int k, int node_cap, int R, bool w
   // blocks per SM keeps that cheap), on the side stream from the end of the ingest on, beside the
   // incremental marking
   auto gated = [&](unsigned single) { return share(single < 304u ? single : 304u); };
-  VDB_LAUNCH(k_clear_masks<GV>, dim3(gated(256), k), kT, 0, gs, gv);
-  VDB_LAUNCH_PDL(k_obstacle_flags<GV>, dim3(gated(1024), k), kT, 0, gs, gv);
+  VDB_LAUNCH(k_obstacle_flags<GV>, dim3(gated(1024), k), kT, 0, gs, gv);
   VDB_LAUNCH_PDL(k_node_halo<GV>, dim3(gated(64), k), kT, 0, gs, gv);
   if (R <= 16) {
     VDB_LAUNCH_PDL(k_dilate_nodes<GV>, dim3(gated(nc < 1024 ? nc : 1024u), k), 256, 0, gs, gv);
@@ -1891,7 +1882,7 @@ cudaError_t ensure_scratch(Scratch& s, size_t bytes) {
 }
 
 cudaError_t launch_reset(const GridView& g, cudaStream_t st) {
-  VDB_LAUNCH(k_reset_nodes<OneView>, 1024, kT, 0, st, OneView{g});
+  VDB_LAUNCH_PDL(k_reset_nodes<OneView>, 1024, kT, 0, st, OneView{g}, (int32_t*)nullptr, (int64_t)0);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return cudaMemsetAsync(g.counters, 0, sizeof(int32_t) * C_NUM, st);
@@ -1991,28 +1982,24 @@ cudaError_t launch_ingest_records(const GridView& g, const rec_t* rec, int64_t n
   int32_t* nflag = (int32_t*)p;
   int32_t* flag = nflag + nkeys_al;
   p += align_up(((size_t)m + (size_t)nkeys_al) * 4);
+  // the dense mask follows the flags, so that one memset clears both
+  unsigned long long* dbits = dense_bits ? (unsigned long long*)p : nullptr;
+  if (dbits) p += align_up((size_t)nbr_all * 64);
   int32_t* pos = (int32_t*)p;
   p += nb4;
   void* rtemp = p;
   p += align_up(radix_temp_bytes(n));
   void* stemp = p;
-  p += align_up(scan_temp_bytes(m));
-  unsigned long long* dbits = dense_bits ? (unsigned long long*)p : nullptr;
 
   const unsigned nbk = blocks_for(n);
   const uint64_t nbr = (uint64_t)nbr_all;
   if (counting) {
     // one flag per brick of the grid, then compaction
-    e = cudaMemsetAsync(nflag, 0, sizeof(int32_t) * (size_t)(nkeys_al + (int64_t)nbr), st);
+    const size_t clear = dbits ? (size_t)((char*)(dbits + nbr * 8) - (char*)nflag) : sizeof(int32_t) * ((size_t)nkeys_al + nbr);
+    e = cudaMemsetAsync(nflag, 0, clear, st);
     if (e != cudaSuccess) return e;
-    if (dbits) {
-      e = cudaMemsetAsync(dbits, 0, (size_t)nbr * 64, st);
-      if (e != cudaSuccess) return e;
-    }
     VDB_LAUNCH(k_mark_record_bricks, nbk, kT, 0, st, g, rec, n, n_dev, flag, dbits);
-    e = cudaMemsetAsync(g.counters + C_UNIQUE, 0, sizeof(int32_t), st);
-    if (e != cudaSuccess) return e;
-    VDB_LAUNCH(k_compact_flag_index, blocks_for((int64_t)nbr), kT, 0, st, g, flag, (int64_t)nbr, ka, nflag);
+    VDB_LAUNCH_PDL(k_compact_flag_index, blocks_for((int64_t)nbr), kT, 0, st, g, flag, (int64_t)nbr, ka, nflag);
     VDB_LAUNCH_PDL(k_create_flagged_nodes, blocks_for(nkeys), kT, 0, st, g, nflag, nkeys);
     VDB_LAUNCH_PDL(k_alloc_obstacle_bricks, blocks_for((int64_t)nbr), kT, 0, st, g, ka, (int64_t)nbr, track, dbits);
     if (!track && !dbits) VDB_LAUNCH_PDL(k_apply_set_only, nbk, kT, 0, st, g, rec, n, n_dev);
@@ -2048,24 +2035,22 @@ size_t dense_scratch_bytes(const GridView& g) {
 }
 
 cudaError_t launch_ingest_dense(const GridView& g, const uint8_t* grid, Scratch& scr, cudaStream_t st) {
-  cudaError_t e = ensure_scratch(scr, dense_scratch_bytes(g));
-  if (e != cudaSuccess) return e;
   const size_t nbr = (size_t)g.BX * g.BY * g.BZ, nkeys = (size_t)g.NX * g.NY * g.NZ;
   char* p = (char*)scr.buf;
   DenseScratch ds{(unsigned long long*)p, (int32_t*)(p + align_up(nbr * 64)),
                   (int32_t*)(p + align_up(nbr * 64) + align_up(nbr * 4)), nullptr};
-  e = cudaMemsetAsync(ds.nflag, 0, nkeys * 4, st);
-  if (e != cudaSuccess) return e;
   const OneView v{g};
-  VDB_LAUNCH((k_dense_masks<OneView, OneSrc>), batch_blocks(g, BK_DENSE), kT, 0, st, v, OneSrc{grid}, ds);
-  VDB_LAUNCH(k_dense_nodes<OneView>, batch_blocks(g, BK_DNODES), kT, 0, st, v, ds);
-  VDB_LAUNCH(k_dense_alloc<OneView>, batch_blocks(g, BK_DALLOC), kT, 0, st, v, ds);
+  // the reset that a dense ingest starts with also clears the node flags; the counters, which its blocks
+  // read, are cleared by the next kernel
+  VDB_LAUNCH_PDL(k_reset_nodes<OneView>, 1024, kT, 0, st, v, ds.nflag, (int64_t)nkeys);
+  VDB_LAUNCH_PDL((k_dense_masks<OneView, OneSrc>), batch_blocks(g, BK_DENSE), kT, 0, st, v, OneSrc{grid}, ds, true);
+  VDB_LAUNCH_PDL(k_dense_nodes<OneView>, batch_blocks(g, BK_DNODES), kT, 0, st, v, ds);
+  VDB_LAUNCH_PDL(k_dense_alloc<OneView>, batch_blocks(g, BK_DALLOC), kT, 0, st, v, ds);
   return cudaGetLastError();
 }
 
 cudaError_t launch_activation_full(const GridView& g, cudaStream_t st) {
   const OneView v{g};
-  VDB_LAUNCH_PDL(k_clear_masks<OneView>, 256, kT, 0, st, v);
   VDB_LAUNCH_PDL(k_obstacle_flags<OneView>, 1024, kT, 0, st, v);
   VDB_LAUNCH_PDL(k_node_halo<OneView>, 64, kT, 0, st, v);
   if (g.R <= 16) {
@@ -2075,25 +2060,19 @@ cudaError_t launch_activation_full(const GridView& g, cudaStream_t st) {
     VDB_LAUNCH_PDL((k_dilate_stage<1, OneView>), 256, kT, 0, st, v);
     VDB_LAUNCH_PDL((k_dilate_stage<2, OneView>), 256, kT, 0, st, v);
   }
-  VDB_LAUNCH_PDL(k_alloc_marked<OneView>, g.node_cap * 16 < 8192 ? g.node_cap * 16 : 8192, kT, 0, st, v, false);
+  VDB_LAUNCH_PDL(k_alloc_marked<OneView>, g.node_cap * 16 < 8192 ? g.node_cap * 16 : 8192, kT, 0, st, v, true);
   return cudaGetLastError();
-}
-
-static cudaError_t clear_item_counters(const GridView& g, cudaStream_t st) {
-  return cudaMemsetAsync(g.items_ctr, 0, 3 * sizeof(int32_t), st);
 }
 
 cudaError_t launch_build_items_full(const GridView& g, const Tuning& t, const Items& it, bool with_slots,
                                     cudaStream_t st) {
-  cudaError_t e = clear_item_counters(g, st);
-  if (e != cudaSuccess) return e;
-  VDB_LAUNCH(k_items_nodes<OneView>, g.node_cap * 12 < 8192 ? g.node_cap * 12 : 8192, kT, 0, st, OneView{g}, t.run[0],
+  VDB_LAUNCH_PDL(k_items_nodes<OneView>, g.node_cap * 12 < 8192 ? g.node_cap * 12 : 8192, kT, 0, st, OneView{g}, t.run[0],
              t.run[1], t.run[2], it, with_slots);
   return cudaGetLastError();
 }
 
 cudaError_t launch_item_slots(const GridView& g, const Tuning& t, const Items& it, cudaStream_t st) {
-  VDB_LAUNCH(k_item_slots, dim3(405, 3), kT, 0, st, g, t.run[0], t.run[1], t.run[2], it);
+  VDB_LAUNCH_PDL(k_item_slots, dim3(405, 3), kT, 0, st, g, t.run[0], t.run[1], t.run[2], it);
   return cudaGetLastError();
 }
 
@@ -2124,7 +2103,6 @@ int batch_blocks(const GridView& g, int kind) {
     }
     case BK_DNODES: return clamp_blocks(((int64_t)g.NX * g.NY * g.NZ + t - 1) / t, 1024);
     case BK_DALLOC: return clamp_blocks(((int64_t)g.BX * g.BY * g.BZ + t - 1) / t, 152 * 64);
-    case BK_CLEAR: return clamp_blocks(((int64_t)g.node_cap * 128 + t - 1) / t, 256);
     case BK_OBST: return clamp_blocks(((int64_t)g.cap + t - 1) / t, 1024);
     case BK_HALO: return clamp_blocks(((int64_t)g.node_cap * 32 + t - 1) / t, 64);
     case BK_DILATE: return clamp_blocks(g.node_cap, 1024);
@@ -2137,7 +2115,8 @@ int batch_blocks(const GridView& g, int kind) {
 cudaError_t launch_reset_batch(const GridView* views, const BatchShape& b, int32_t* counters_all, size_t n_counters,
                                cudaStream_t st) {
   if (b.k <= 0) return cudaSuccess;
-  VDB_LAUNCH(k_reset_nodes<BatchViews>, b.total[BK_RESET], kT, 0, st, BatchViews{views, b.first[BK_RESET], b.k});
+  VDB_LAUNCH_PDL(k_reset_nodes<BatchViews>, b.total[BK_RESET], kT, 0, st, BatchViews{views, b.first[BK_RESET], b.k},
+                 (int32_t*)nullptr, (int64_t)0);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return cudaMemsetAsync(counters_all, 0, sizeof(int32_t) * n_counters, st);
@@ -2155,36 +2134,33 @@ cudaError_t launch_ingest_dense_batch(const GridView* views, const BatchShape& b
   char* p = (char*)scratch;
   DenseScratch ds{(unsigned long long*)p, (int32_t*)p, (int32_t*)p, offsets};
   VDB_LAUNCH((k_dense_masks<BatchViews, BatchSrc>), b.total[BK_DENSE], kT, 0, st,
-             BatchViews{views, b.first[BK_DENSE], b.k}, src, ds);
-  VDB_LAUNCH(k_dense_nodes<BatchViews>, b.total[BK_DNODES], kT, 0, st, BatchViews{views, b.first[BK_DNODES], b.k}, ds);
-  VDB_LAUNCH(k_dense_alloc<BatchViews>, b.total[BK_DALLOC], kT, 0, st, BatchViews{views, b.first[BK_DALLOC], b.k}, ds);
+             BatchViews{views, b.first[BK_DENSE], b.k}, src, ds, false);
+  VDB_LAUNCH_PDL(k_dense_nodes<BatchViews>, b.total[BK_DNODES], kT, 0, st, BatchViews{views, b.first[BK_DNODES], b.k}, ds);
+  VDB_LAUNCH_PDL(k_dense_alloc<BatchViews>, b.total[BK_DALLOC], kT, 0, st, BatchViews{views, b.first[BK_DALLOC], b.k}, ds);
   return cudaGetLastError();
 }
 
 cudaError_t launch_activation_batch(const GridView* views, const BatchShape& b, cudaStream_t st) {
   if (b.k <= 0) return cudaSuccess;
-  VDB_LAUNCH(k_clear_masks<BatchViews>, b.total[BK_CLEAR], kT, 0, st, BatchViews{views, b.first[BK_CLEAR], b.k});
-  VDB_LAUNCH(k_obstacle_flags<BatchViews>, b.total[BK_OBST], kT, 0, st, BatchViews{views, b.first[BK_OBST], b.k});
-  VDB_LAUNCH(k_node_halo<BatchViews>, b.total[BK_HALO], kT, 0, st, BatchViews{views, b.first[BK_HALO], b.k});
+  VDB_LAUNCH_PDL(k_obstacle_flags<BatchViews>, b.total[BK_OBST], kT, 0, st, BatchViews{views, b.first[BK_OBST], b.k});
+  VDB_LAUNCH_PDL(k_node_halo<BatchViews>, b.total[BK_HALO], kT, 0, st, BatchViews{views, b.first[BK_HALO], b.k});
   const BatchViews dv{views, b.first[BK_DILATE], b.k};
   if (b.R <= 16) {
-    VDB_LAUNCH(k_dilate_nodes<BatchViews>, b.total[BK_DILATE], 256, 0, st, dv);
+    VDB_LAUNCH_PDL(k_dilate_nodes<BatchViews>, b.total[BK_DILATE], 256, 0, st, dv);
   } else {
     VDB_LAUNCH((k_dilate_stage<0, BatchViews>), b.total[BK_DILATE], kT, 0, st, dv);
     VDB_LAUNCH((k_dilate_stage<1, BatchViews>), b.total[BK_DILATE], kT, 0, st, dv);
     VDB_LAUNCH((k_dilate_stage<2, BatchViews>), b.total[BK_DILATE], kT, 0, st, dv);
   }
-  VDB_LAUNCH(k_alloc_marked<BatchViews>, b.total[BK_ALLOC], kT, 0, st, BatchViews{views, b.first[BK_ALLOC], b.k},
-             false);
+  VDB_LAUNCH_PDL(k_alloc_marked<BatchViews>, b.total[BK_ALLOC], kT, 0, st, BatchViews{views, b.first[BK_ALLOC], b.k},
+                 true);
   return cudaGetLastError();
 }
 
 cudaError_t launch_build_items_batch(const GridView* views, const BatchShape& b, const Tuning& t, const Items& it,
-                                     int32_t* items_ctr, cudaStream_t st) {
+                                     cudaStream_t st) {
   if (b.k <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(items_ctr, 0, 3 * sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
-  VDB_LAUNCH(k_items_nodes<BatchViews>, b.total[BK_ITEMS], kT, 0, st, BatchViews{views, b.first[BK_ITEMS], b.k},
+  VDB_LAUNCH_PDL(k_items_nodes<BatchViews>, b.total[BK_ITEMS], kT, 0, st, BatchViews{views, b.first[BK_ITEMS], b.k},
              t.run[0], t.run[1], t.run[2], it, true);
   return cudaGetLastError();
 }

@@ -498,6 +498,7 @@ constexpr int kEnvRun = 16;
 // 512 x 512 x 256 tunnel scene, dmax 64: 0.075 ms (scanning the neighbours' bytes outward: 0.149).
 constexpr int kEnvMaxNB = kEnvRun + 2 * 23;
 __global__ void __launch_bounds__(256) k_env_x(GridView g, const unsigned long long* __restrict__ items, int max_items) {
+  pdl_enter();
   __shared__ int slots[kEnvMaxNB];
   __shared__ uint32_t masks[64 * 17];  // bricks past the halo stay empty
   __shared__ uint32_t fin[kEnvRun];
@@ -586,6 +587,7 @@ size_t env_smem(int R) { return (size_t)(kEnvRun + 2 * R) * (kBrickVox * 2 + 128
 template <int AXIS>
 __global__ void __launch_bounds__(kEnvBlock) k_env_line(GridView g, const unsigned long long* __restrict__ items,
                                                         int max_items) {
+  pdl_enter();
   extern __shared__ __align__(16) uint32_t smem32[];
   __shared__ int slots[kEnvMaxNB];   // stored bricks of the run and its halo (-1: none)
   __shared__ int inslot[kEnvMaxNB];  // the same, -1 also where the brick's input is all dmax^2
@@ -689,7 +691,7 @@ int num_sms() {
 // taken grid-stride; blocks beyond the queued count exit at once).
 template <typename K>
 cudaError_t launch_env_kernel(K kernel, int threads, size_t smem, const GridView& g, const unsigned long long* items,
-                              cudaStream_t st) {
+                              bool chained, cudaStream_t st) {
   if (g.item_cap <= 0) return cudaSuccess;
   // the largest radius's shared memory, whatever this grid's: concurrent callers set the same value
   cudaError_t e = smem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)env_smem(23)) : cudaSuccess;
@@ -700,19 +702,23 @@ cudaError_t launch_env_kernel(K kernel, int threads, size_t smem, const GridView
   if (per_sm < 1) per_sm = 1;
   int grid = num_sms() * per_sm;
   if (grid > g.item_cap) grid = g.item_cap;
-  VDB_LAUNCH(kernel, grid, threads, smem, st, g, items, g.item_cap);
+  if (chained)
+    VDB_LAUNCH_PDL(kernel, grid, threads, smem, st, g, items, (int)g.item_cap);
+  else
+    VDB_LAUNCH(kernel, grid, threads, smem, st, g, items, g.item_cap);
   return cudaGetLastError();
 }
 
 // Envelope pass along `axis`.
-cudaError_t launch_env(const GridView& g, int axis, const Items& it, cudaStream_t st) {
-  if (axis == 0) return launch_env_kernel(k_env_x, 256, 0, g, it.run[0], st);
-  if (axis == 1) return launch_env_kernel(k_env_line<1>, kEnvBlock, env_smem(g.R), g, it.run[1], st);
-  return launch_env_kernel(k_env_line<2>, kEnvBlock, env_smem(g.R), g, it.run[2], st);
+cudaError_t launch_env(const GridView& g, int axis, const Items& it, bool chained, cudaStream_t st) {
+  if (axis == 0) return launch_env_kernel(k_env_x, 256, 0, g, it.run[0], chained, st);
+  if (axis == 1) return launch_env_kernel(k_env_line<1>, kEnvBlock, env_smem(g.R), g, it.run[1], chained, st);
+  return launch_env_kernel(k_env_line<2>, kEnvBlock, env_smem(g.R), g, it.run[2], chained, st);
 }
 
 template <int R, int RUN, int AXIS>
-cudaError_t pass_window(const GridView& g, const int32_t* islots, int max_items, cudaStream_t st, bool prune) {
+cudaError_t pass_window(const GridView& g, const int32_t* islots, int max_items, bool chained, cudaStream_t st,
+                        bool prune) {
   using S = ColShape<R, RUN, AXIS>;
   auto kernel = k_pass<R, RUN, AXIS>;
   if (max_items <= 0) return cudaSuccess;
@@ -734,8 +740,7 @@ cudaError_t pass_window(const GridView& g, const int32_t* islots, int max_items,
   }
   int grid = num_sms() * per_sm;
   if (grid > max_items) grid = max_items;
-  // the y and z passes follow the previous pass directly: their launch overlaps its tail
-  if (AXIS > 0)
+  if (chained)
     VDB_LAUNCH_PDL(kernel, grid, S::THREADS, S::SMEM, st, g, islots, max_items, prune);
   else
     VDB_LAUNCH(kernel, grid, S::THREADS, S::SMEM, st, g, islots, max_items, prune);
@@ -743,25 +748,26 @@ cudaError_t pass_window(const GridView& g, const int32_t* islots, int max_items,
 }
 
 template <int RUN, int AXIS>
-cudaError_t pass_window_r(const GridView& g, const int32_t* islots, int max_items, cudaStream_t st, bool prune) {
+cudaError_t pass_window_r(const GridView& g, const int32_t* islots, int max_items, bool chained, cudaStream_t st,
+                          bool prune) {
   switch (g.R) {
-    case 1: return pass_window<1, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 2: return pass_window<2, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 3: return pass_window<3, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 4: return pass_window<4, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 5: return pass_window<5, RUN, AXIS>(g, islots, max_items, st, prune);
-    case 6: return pass_window<6, RUN, AXIS>(g, islots, max_items, st, prune);
+    case 1: return pass_window<1, RUN, AXIS>(g, islots, max_items, chained, st, prune);
+    case 2: return pass_window<2, RUN, AXIS>(g, islots, max_items, chained, st, prune);
+    case 3: return pass_window<3, RUN, AXIS>(g, islots, max_items, chained, st, prune);
+    case 4: return pass_window<4, RUN, AXIS>(g, islots, max_items, chained, st, prune);
+    case 5: return pass_window<5, RUN, AXIS>(g, islots, max_items, chained, st, prune);
+    case 6: return pass_window<6, RUN, AXIS>(g, islots, max_items, chained, st, prune);
   }
   return cudaErrorInvalidValue;
 }
 
 template <int AXIS>
-cudaError_t pass_window_run(const GridView& g, int run, const int32_t* islots, int max_items, cudaStream_t st,
-                          bool prune) {
+cudaError_t pass_window_run(const GridView& g, int run, const int32_t* islots, int max_items, bool chained,
+                            cudaStream_t st, bool prune) {
   switch (run) {
-    case 4: return pass_window_r<4, AXIS>(g, islots, max_items, st, prune);
-    case 8: return pass_window_r<8, AXIS>(g, islots, max_items, st, prune);
-    case 16: return pass_window_r<16, AXIS>(g, islots, max_items, st, prune);
+    case 4: return pass_window_r<4, AXIS>(g, islots, max_items, chained, st, prune);
+    case 8: return pass_window_r<8, AXIS>(g, islots, max_items, chained, st, prune);
+    case 16: return pass_window_r<16, AXIS>(g, islots, max_items, chained, st, prune);
   }
   return cudaErrorInvalidValue;
 }
@@ -834,17 +840,17 @@ GridView pool_view(const GridView& g) {
   return p;
 }
 
-cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, cudaStream_t st) {
+cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, bool chained, cudaStream_t st) {
   const bool prune = (t.variant & 3) != 1;
   if (windowed_form(g)) {
     const GridView p = pool_view(g);
     if (axis == 0 && (t.variant & kVariantXDirect)) return x_direct(p, it.slots[0], g.item_cap, t.run[0], st);
-    if (axis == 0) return pass_window_run<0>(p, t.run[0], it.slots[0], g.item_cap, st, prune);
-    if (axis == 1) return pass_window_run<1>(p, t.run[1], it.slots[1], g.item_cap, st, prune);
-    return pass_window_run<2>(p, t.run[2], it.slots[2], g.item_cap, st, prune);
+    if (axis == 0) return pass_window_run<0>(p, t.run[0], it.slots[0], g.item_cap, chained, st, prune);
+    if (axis == 1) return pass_window_run<1>(p, t.run[1], it.slots[1], g.item_cap, chained, st, prune);
+    return pass_window_run<2>(p, t.run[2], it.slots[2], g.item_cap, chained, st, prune);
   }
   // the envelope kernels find bricks through the grid's own tables (local slots)
-  return launch_env(g, axis, it, st);
+  return launch_env(g, axis, it, chained, st);
 }
 
 }  // namespace vdbedt

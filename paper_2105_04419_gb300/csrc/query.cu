@@ -27,6 +27,7 @@ __device__ __forceinline__ int sqdist_at(const GridView& g, int x, int y, int z)
 
 // caller coordinates are stored shifted by g.off (an unbounded grid's signed coordinates)
 __global__ void k_query(GridView g, const int32_t* __restrict__ xyz, int64_t n, int32_t* __restrict__ out) {
+  pdl_enter();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = sqdist_at(g, xyz[3 * i] + g.off, xyz[3 * i + 1] + g.off, xyz[3 * i + 2] + g.off);
 }
@@ -41,6 +42,7 @@ __global__ void k_query(GridView g, const int32_t* __restrict__ xyz, int64_t n, 
 // read: 1.48 ms); the 4-byte form serves widths that are no multiple of 4.
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_export_dense(GridView g, int32_t* __restrict__ out) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t units = (int64_t)g.NX * g.BY * g.BZ * 8;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -155,6 +157,7 @@ __device__ __forceinline__ int line_match(const GridView& g, int x, int y, int z
 // the sphere in (z, y, x) order and testing occupancy bits: 3.7 ms).
 __global__ void __launch_bounds__(128) k_query_nearest(GridView g, const int32_t* __restrict__ xyz, int64_t n,
                                                        int32_t* __restrict__ out) {
+  pdl_enter();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int x = xyz[3 * i] + g.off, y = xyz[3 * i + 1] + g.off, z = xyz[3 * i + 2] + g.off;
     int rx = -1 + g.off, ry = -1 + g.off, rz = -1 + g.off;
@@ -256,6 +259,7 @@ __device__ __forceinline__ float trilinear(const Corner8& c, float tx, float ty,
 
 __global__ void k_clearance_fwd(GridView g, float vs, const float* __restrict__ pts, int64_t T, int64_t P, float tau,
                                 float* __restrict__ cost) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -280,6 +284,7 @@ __global__ void k_clearance_fwd(GridView g, float vs, const float* __restrict__ 
 
 __global__ void k_clearance_bwd(GridView g, float vs, const float* __restrict__ pts, int64_t T, int64_t P, float tau,
                                 const float* __restrict__ gcost, float* __restrict__ gpts) {
+  pdl_enter();
   const int64_t n = T * P;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float* q = pts + i * 3;
@@ -317,6 +322,7 @@ __global__ void k_clearance_bwd(GridView g, float vs, const float* __restrict__ 
 // cost, grad = (1 / vs) grad_t(trilinear), a thread per point.
 __global__ void k_distance_at(GridView g, float vs, const float* __restrict__ pts, int64_t n, float* __restrict__ dist,
                               float* __restrict__ grad) {
+  pdl_enter();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float* q = pts + i * 3;
     int i0, j0, k0;
@@ -354,20 +360,20 @@ unsigned grid_for(int64_t n, int threads) {
 
 cudaError_t launch_query(const GridView& g, const int32_t* xyz, int64_t n, int32_t* out, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  VDB_LAUNCH(k_query, grid_for(n, 256), 256, 0, st, g, xyz, n, out);
+  VDB_LAUNCH_PDL(k_query, grid_for(n, 256), 256, 0, st, g, xyz, n, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_distance_at(const GridView& g, float vs, const float* pts, int64_t n, float* dist, float* grad,
                                cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  VDB_LAUNCH(k_distance_at, grid_for(n, 256), 256, 0, st, g, vs, pts, n, dist, grad);
+  VDB_LAUNCH_PDL(k_distance_at, grid_for(n, 256), 256, 0, st, g, vs, pts, n, dist, grad);
   return cudaGetLastError();
 }
 
 cudaError_t launch_query_nearest(const GridView& g, const int32_t* xyz, int64_t n, int32_t* out, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  VDB_LAUNCH(k_query_nearest, grid_for(n, 128), 128, 0, st, g, xyz, n, out);
+  VDB_LAUNCH_PDL(k_query_nearest, grid_for(n, 128), 128, 0, st, g, xyz, n, out);
   return cudaGetLastError();
 }
 
@@ -472,23 +478,23 @@ cudaError_t launch_export_occupancy(const GridView& g, const int32_t* changed, i
 cudaError_t launch_export_dense(const GridView& g, int32_t* out, cudaStream_t st) {
   const unsigned blocks = grid_for((int64_t)g.NX * g.BY * g.BZ * 8 * 32, 256);
   if (g.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0)
-    VDB_LAUNCH(k_export_dense<true>, blocks, 256, 0, st, g, out);
+    VDB_LAUNCH_PDL(k_export_dense<true>, blocks, 256, 0, st, g, out);
   else
-    VDB_LAUNCH(k_export_dense<false>, blocks, 256, 0, st, g, out);
+    VDB_LAUNCH_PDL(k_export_dense<false>, blocks, 256, 0, st, g, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_clearance_fwd(const GridView& g, float vs, const float* pts, int64_t T, int64_t P, float tau,
                                  float* cost, cudaStream_t st) {
   if (T <= 0) return cudaSuccess;
-  VDB_LAUNCH(k_clearance_fwd, grid_for(T * 32, 256), 256, 0, st, g, vs, pts, T, P, tau, cost);
+  VDB_LAUNCH_PDL(k_clearance_fwd, grid_for(T * 32, 256), 256, 0, st, g, vs, pts, T, P, tau, cost);
   return cudaGetLastError();
 }
 
 cudaError_t launch_clearance_bwd(const GridView& g, float vs, const float* pts, int64_t T, int64_t P, float tau,
                                  const float* gcost, float* gpts, cudaStream_t st) {
   if (T <= 0 || P <= 0) return cudaSuccess;
-  VDB_LAUNCH(k_clearance_bwd, grid_for(T * P, 256), 256, 0, st, g, vs, pts, T, P, tau, gcost, gpts);
+  VDB_LAUNCH_PDL(k_clearance_bwd, grid_for(T * P, 256), 256, 0, st, g, vs, pts, T, P, tau, gcost, gpts);
   return cudaGetLastError();
 }
 

@@ -93,7 +93,8 @@ struct GridView {
   unsigned long long* hslots;  // [hmask+1]
   int32_t* child;     // [node_cap * 4096]
   uint32_t* amask;    // [node_cap * 128] compute-set bits: bit l = bx + 16 by + 256 bz (local)
-  uint32_t* mwork;    // [node_cap * 384] obstacle bits and two dilation stages, same layout
+  uint32_t* mwork;    // [node_cap * 384] obstacle bits (zero between activations) and two dilation stages,
+                      // same layout
   uint32_t* nclaim;   // [node_cap * 128] bricks claimed for allocation by the running ingest (amask layout)
   long long* node_key;  // [node_cap]
   int32_t* mark;      // [node_cap * 3 * 1024] epoch of the last time each run along axis a was queued
@@ -377,7 +378,8 @@ struct UpdArgs {
 cudaError_t ensure_scratch(Scratch& s, size_t bytes);
 
 cudaError_t launch_reset(const GridView& g, cudaStream_t st);
-// n records at rec; with n_dev (nullable) only the first *n_dev of them (clamped to [0, n]).
+// n records at rec; with n_dev (nullable) only the first *n_dev of them (clamped to [0, n]).  The untracked
+// form expects counters C_UNIQUE and C_HAS_ZERO (neighbours) at zero.
 // scr: sort / scan scratch of the global form; vl: the per-voxel last-record table (allocated and
 // set to -1 on first use, cap * 512 words); rslot: one word per record (n entries) for the tracked
 // form's brick slots.
@@ -389,6 +391,7 @@ cudaError_t reserve_ingest(const GridView& g, int64_t n, Scratch& scr, Scratch& 
 cudaError_t launch_begin_update(const GridView& g, cudaStream_t st);
 // dense grid -> bricks (scratch: dense_scratch_bytes(g))
 size_t dense_scratch_bytes(const GridView& g);
+// (resets the grid first; scr holds dense_scratch_bytes(g))
 cudaError_t launch_ingest_dense(const GridView& g, const uint8_t* grid, Scratch& scr, cudaStream_t st);
 cudaError_t launch_activation_full(const GridView& g, cudaStream_t st);
 // every run holding a stored brick, with slot lists when with_slots (windowed form)
@@ -450,7 +453,7 @@ cudaError_t launch_item_slots(const GridView& g, const Tuning& t, const Items& i
 // Kernels that run once per grid: in a batch each grid gets a share of one launch sized to its
 // work (batch_blocks), the shares laid end to end (first[kind][i] = first block of grid i).
 enum BatchKind {
-  BK_RESET = 0, BK_DENSE, BK_DNODES, BK_DALLOC, BK_CLEAR, BK_OBST, BK_HALO, BK_DILATE, BK_ALLOC, BK_ITEMS, BK_NUM
+  BK_RESET = 0, BK_DENSE, BK_DNODES, BK_DALLOC, BK_OBST, BK_HALO, BK_DILATE, BK_ALLOC, BK_ITEMS, BK_NUM
 };
 int batch_blocks(const GridView& g, int kind);
 struct BatchShape {
@@ -469,12 +472,13 @@ cudaError_t launch_ingest_dense_batch(const GridView* views, const BatchShape& b
                                       cudaStream_t st);
 cudaError_t launch_activation_batch(const GridView* views, const BatchShape& b, cudaStream_t st);
 cudaError_t launch_build_items_batch(const GridView* views, const BatchShape& b, const Tuning& t, const Items& it,
-                                     int32_t* items_ctr, cudaStream_t st);
+                                     cudaStream_t st);
 
 // passes (passes.cu)
 bool windowed_form(const GridView& g);
-// pass along `axis` (0 x, 1 y, 2 z) over the queued runs
-cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, cudaStream_t st);
+// pass along `axis` (0 x, 1 y, 2 z) over the queued runs; chained: it follows a kernel of the stream
+// directly, and its launch overlaps that kernel's tail
+cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, bool chained, cudaStream_t st);
 int effective_run(const GridView& g, const Tuning& t, int axis);
 // a bounded device wait that runs out (0: mbarrier phase, 1: pending node), for tests
 cudaError_t launch_wait_selftest(const GridView& g, int which, cudaStream_t st);
