@@ -733,7 +733,7 @@ vdbedt_status vdbedt_update(vdbedt_handle h, vdbedt_update_stats* stats) {
     mark(h, 2);
     // slot lists of the dirty runs (an update that switched to the global form got them with its
     // work lists), then the side stream's branch joins before the passes
-    if (windowed_form(h->g)) CK(h, launch_item_slots(h->g, t, h->items, h->st), "item slots");
+    CK(h, windowed_form(h->g) ? launch_item_slots(h->g, t, h->items, h->st) : launch_init_new(h->g, h->st), "item slots");
     CK(h, cudaStreamWaitEvent(h->st, h->fork.join, 0), "join");
     s = run_passes(h, t, true);
     if (s) return s;
@@ -1205,7 +1205,7 @@ vdbedt_status batch_update(vdbedt_batch* b, vdbedt_update_stats* stats) {
     BCK(b, launch_update_batch_mark(b->d_upd, shape, t, b->items, b->fork, b->st), "mark");
     BCK(b, cudaStreamWaitEvent(b->st, b->fork.join, 0), "join");
     bmark(b, 2);
-    BCK(b, launch_item_slots_batch(b->d_views, t, b->items, b->pool.items_ctr, b->pool.item_cap, b->st), "item slots");
+    BCK(b, launch_item_slots_batch(b->d_views, b->k, t, b->items, b->pool.items_ctr, b->pool.item_cap, b->st), "item slots");
     bmark(b, 3);
     BCK(b, launch_pass(b->pool, t, 0, b->items, false, b->st), "x pass");
     bmark(b, 4);

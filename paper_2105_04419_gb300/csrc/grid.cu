@@ -230,17 +230,6 @@ __device__ __forceinline__ void init_fields_warp(const GridView& g, int slot, in
   for (int q = 0; q < 4; ++q) dd[lane + 32 * q] = w;
 }
 
-// The fields of the slots `ok` lanes hold, a brick at a time by the whole warp (warp-uniform call).
-__device__ __forceinline__ void init_fields_ballot(const GridView& g, bool ok, int slot) {
-  const int lane = threadIdx.x & 31;
-  unsigned todo = __ballot_sync(0xffffffffu, ok);
-  while (todo) {
-    const int b = __ffs(todo) - 1;
-    todo &= todo - 1u;
-    init_fields_warp(g, __shfl_sync(0xffffffffu, slot, b), lane);
-  }
-}
-
 __device__ void init_brick(const GridView& g, int slot, int node, int bx, int by, int bz, bool init_fields) {
   ulonglong2* occ = reinterpret_cast<ulonglong2*>(g.occ + (size_t)slot * 8);
 #pragma unroll
@@ -618,7 +607,8 @@ __global__ void k_apply_set_only(GridView g, const rec_t* __restrict__ rec, int6
 // kernels (rslot).  A "set" record whose brick is not stored yet creates the brick's interior node
 // when it is missing (inline, as the marking kernel does) and claims the brick with a per-node bit
 // (`nclaim`, the amask layout); the claiming thread allocates the brick (slots reserved a warp at a
-// time, fields at dmax^2 written by the whole warp) and publishes its slot in the child table.
+// time; its fields are set with the other new bricks', init_new_fields) and publishes its slot in the child
+// table.
 // Records that lose the claim, or read the child table before the claimer publishes, look the
 // brick up again in the next kernel (rslot -2).  The claimer's record keeps -3 - slot, so that the
 // next kernel, when no record of this ingest tests the bit any more, clears it: `nclaim` is zero
@@ -670,9 +660,8 @@ __global__ void k_rec_slots(US us) {
       const int l = local_brick(bx, by, bz);
       atomicAnd(&g.nclaim[(size_t)node * 128 + (l >> 5)], ~(1u << (l & 31)));
     }
-    if (ok) init_brick(g, slot, node, bx, by, bz, false);
-    init_fields_ballot(g, ok, slot);
     if (ok) {
+      init_brick(g, slot, node, bx, by, bz, false);
       g.child[(size_t)node * kNodeBricks + local_brick(bx, by, bz)] = slot;
       rs = -3 - slot;
     }
@@ -1244,15 +1233,23 @@ __device__ __forceinline__ int warp_reserve_count(int32_t* ctr, int cnt, int* to
 // Storage for the bricks of a row segment whose compute-set bits (`bits` of amask word `word` of
 // `node`; bit b is the brick at x = x16 + (b & 15) of row (y, z)) this thread set first, so that
 // exactly one thread handles each: the ones without storage get slots (places reserved a warp at
-// a time), their metadata from the thread, their fields at dmax^2 from the whole warp
-// (warp-uniform call).
+// a time; warp-uniform call) and their metadata from the thread; their fields are set afterwards with all
+// new bricks' (init_new_fields).
 __device__ void alloc_new_bits(const GridView& g, int node, int word, uint32_t bits, int x16, int y, int z) {
   uint32_t need = 0u;
-  if (node >= 0)
-    for (uint32_t b = bits; b; b &= b - 1u) {
-      const int bit = __ffs(b) - 1;
-      if (g.child[(size_t)node * kNodeBricks + word * 32 + bit] == kNoSlot) need |= 1u << bit;
-    }
+  if (node >= 0 && bits) {
+    // the row's 16 child slots, loaded together
+    const int half = bits > 0xFFFFu ? 16 : 0;
+    const int4* row = reinterpret_cast<const int4*>(g.child + (size_t)node * kNodeBricks + word * 32 + half);
+    int4 c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c[q] = row[q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      need |= ((uint32_t)(c[q].x == kNoSlot) | (uint32_t)(c[q].y == kNoSlot) << 1 | (uint32_t)(c[q].z == kNoSlot) << 2 |
+               (uint32_t)(c[q].w == kNoSlot) << 3) << (4 * q + half);
+    need &= bits;
+  }
   const int cnt = __popc(need);
   int total = 0;
   const int base = warp_reserve_count(&g.counters[C_NBRICKS], cnt, &total);
@@ -1267,9 +1264,6 @@ __device__ void alloc_new_bits(const GridView& g, int node, int word, uint32_t b
     init_brick(g, slot, node, x16 + (bit & 15), y, z, false);
     g.child[(size_t)node * kNodeBricks + word * 32 + bit] = slot;
   }
-  // fields: round r takes each lane's r-th new brick, a brick at a time by the whole warp
-  const int rounds = __reduce_max_sync(0xffffffffu, (unsigned)cnt);
-  for (int r = 0; r < rounds; ++r) init_fields_ballot(g, r < cnt && base + r < g.cap, base + r);
 }
 
 // Allocate every marked brick without storage: a block per (node, 256-brick chunk), a brick per
@@ -1469,67 +1463,104 @@ __global__ void __launch_bounds__(256) k_items_nodes(VS vs, int rx, int ry, int 
   }
 }
 
-// Slots of each queued run's bricks with R bricks of halo on both sides along the axis: a warp per
-// queued run, a lane per slot.  A run lies inside one node and its halo (R <= 6 < 16 bricks)
-// reaches at most the neighbouring node on each side along the axis, so three node lookups (lanes
-// 0-2) serve the whole slot list, read from the child tables.
-__device__ __forceinline__ void run_slots(const GridView& g, int axis, int run, unsigned long long packed,
-                                          int32_t* __restrict__ dst) {
-  const int nb = run + 2 * g.R;
-  const int lane = threadIdx.x & 31;
-  int bx, by, bz;
-  unpack_brick(packed, bx, by, bz);
-  const int ba = axis == 0 ? bx : (axis == 1 ? by : bz);
-  const int Ba = axis == 0 ? g.BX : (axis == 1 ? g.BY : g.BZ);
-  const int NQa = axis == 0 ? g.NX : (axis == 1 ? g.NY : g.NZ);
-  int nq = -1;
-  if (lane < 3) {
-    const int qa = (ba >> 4) + lane - 1;
-    if (qa >= 0 && qa < NQa) {
-      const int qx = axis == 0 ? qa : bx >> 4, qy = axis == 1 ? qa : by >> 4, qz = axis == 2 ? qa : bz >> 4;
-      nq = find_node(g, node_key_at(g, qx, qy, qz));
+// Slots of each queued run's bricks with R bricks of halo on both sides along the axis: a warp per four
+// queued runs, a lane per slot.  A run lies inside one node and its halo (R <= 6 < 16 bricks) reaches at
+// most the neighbouring node on each side along the axis, so three node lookups (lanes 8 u .. 8 u + 2 for
+// run u) serve its slot list, read from the child tables.  Each run is a chain of three dependent reads
+// (run, hash slots, child entries); four at a time keep as many in flight per warp (71,000
+// runs: 17 us, one at a time 23).  view(item): the grid of a run.
+template <class View>
+__device__ __forceinline__ void item_slots(View view, int axis, int run, const unsigned long long* __restrict__ runs, int n,
+                                           int32_t* __restrict__ slots) {
+  const int lane = threadIdx.x & 31, u = lane >> 3, sub = lane & 7;
+  const int nw = (int)gridDim.x * (int)(blockDim.x >> 5);
+  for (int base = 4 * ((int)blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5)); base < n; base += 4 * nw) {
+    unsigned long long packed = 0ull;
+    int nq = -1;
+    if (base + u < n) {
+      packed = runs[base + u];
+      if (sub < 3) {
+        const GridView& g = view(base + u);
+        int bx, by, bz;
+        unpack_brick(packed, bx, by, bz);
+        const int qa = ((axis == 0 ? bx : (axis == 1 ? by : bz)) >> 4) + sub - 1;
+        const int NQa = axis == 0 ? g.NX : (axis == 1 ? g.NY : g.NZ);
+        if (qa >= 0 && qa < NQa)
+          nq = find_node(g, node_key_at(g, axis == 0 ? qa : bx >> 4, axis == 1 ? qa : by >> 4, axis == 2 ? qa : bz >> 4));
+      }
     }
-  }
-  const int n_lo = __shfl_sync(0xffffffffu, nq, 0), n_mid = __shfl_sync(0xffffffffu, nq, 1),
-            n_hi = __shfl_sync(0xffffffffu, nq, 2);
-  int s = -1;
-  const int ca = ba + lane - g.R;  // this slot's brick coordinate along the axis
-  if (lane < nb && ca >= 0 && ca < Ba) {
-    const int node = (ca >> 4) < (ba >> 4) ? n_lo : ((ca >> 4) > (ba >> 4) ? n_hi : n_mid);
-    if (node >= 0) {
-      const int cx = axis == 0 ? ca : bx, cy = axis == 1 ? ca : by, cz = axis == 2 ? ca : bz;
-      s = g.child[(size_t)node * kNodeBricks + local_brick(cx, cy, cz)];
-      if (s >= 0) s += g.slot_base;
+    int s[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      s[v] = -1;
+      const unsigned long long pk = __shfl_sync(0xffffffffu, packed, 8 * v);
+      const int n_lo = __shfl_sync(0xffffffffu, nq, 8 * v), n_mid = __shfl_sync(0xffffffffu, nq, 8 * v + 1),
+                n_hi = __shfl_sync(0xffffffffu, nq, 8 * v + 2);
+      if (base + v < n) {  // warp-uniform
+        const GridView& g = view(base + v);
+        int bx, by, bz;
+        unpack_brick(pk, bx, by, bz);
+        const int ba = axis == 0 ? bx : (axis == 1 ? by : bz), Ba = axis == 0 ? g.BX : (axis == 1 ? g.BY : g.BZ);
+        const int ca = ba + lane - g.R;  // this slot's brick coordinate along the axis
+        if (lane < run + 2 * g.R && ca >= 0 && ca < Ba) {
+          const int node = (ca >> 4) < (ba >> 4) ? n_lo : ((ca >> 4) > (ba >> 4) ? n_hi : n_mid);
+          if (node >= 0) {
+            s[v] = g.child[(size_t)node * kNodeBricks +
+                           local_brick(axis == 0 ? ca : bx, axis == 1 ? ca : by, axis == 2 ? ca : bz)];
+            if (s[v] >= 0) s[v] += g.slot_base;
+          }
+        }
+      }
     }
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+      if (base + v < n) slots[(size_t)(base + v) * kItemSlots + lane] = s[v];
   }
-  dst[lane] = s;
 }
 
-// blockIdx.y = axis
+// Fields of the bricks that the running update stored (slots from its start's count on) at dmax^2: a
+// brick per warp, streaming.  Done here, by the whole GPU at once, rather than where each brick is
+// allocated: the few blocks of the marking that meet the frontier of the stored bricks allocate hundreds each
+// (a lidar frame's marking took 44 us on average with it, 20 without).
+__device__ __forceinline__ void init_new_fields(const GridView& g, int block, int nblocks) {
+  const int end = min(g.counters[C_NBRICKS], g.cap), nw = nblocks * (int)(blockDim.x >> 5);
+  for (int slot = g.counters[C_NB_START] + block * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5); slot < end; slot += nw)
+    init_fields_warp(g, slot, threadIdx.x & 31);
+}
+
+// blockIdx.y = axis; 3: the new bricks' fields
 __global__ void k_item_slots(GridView g, int rx, int ry, int rz, Items it) {
   pdl_enter();
-  if (g.counters[C_BIG]) return;  // the global form's work lists came with their slots
+  if (g.counters[C_BIG]) return;  // the global form's work lists came with their slots, and write every field
   const int axis = (int)blockIdx.y;
-  const int run = axis == 0 ? rx : (axis == 1 ? ry : rz);
-  const int n = min(g.items_ctr[axis], g.item_cap);
-  const int nw = (int)gridDim.x * (int)(blockDim.x >> 5);
-  for (int item = (int)blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5); item < n; item += nw)
-    run_slots(g, axis, run, it.run[axis][item], it.slots[axis] + (size_t)item * kItemSlots);
+  if (axis == 3) {
+    init_new_fields(g, (int)blockIdx.x, (int)gridDim.x);
+    return;
+  }
+  item_slots([&](int) -> const GridView& { return g; }, axis, axis == 0 ? rx : (axis == 1 ? ry : rz), it.run[axis],
+             min(g.items_ctr[axis], g.item_cap), it.slots[axis]);
 }
 
-// The same for a batch's shared queue: each run's grid comes from it.igrid.
-__global__ void k_item_slots_batch(const GridView* __restrict__ views, const int32_t* __restrict__ items_ctr,
+// The envelope form's updates have no slot lists: the new bricks' fields alone.
+__global__ void k_init_new(GridView g) {
+  pdl_enter();
+  if (!g.counters[C_BIG]) init_new_fields(g, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// The same for a batch of k grids' shared queue: each run's grid comes from it.igrid (runs of a grid whose
+// update took the global form are read again to the slots they came with).
+__global__ void k_item_slots_batch(const GridView* __restrict__ views, int k, const int32_t* __restrict__ items_ctr,
                                    int item_cap, int rx, int ry, int rz, Items it) {
   pdl_enter();
   const int axis = (int)blockIdx.y;
-  const int run = axis == 0 ? rx : (axis == 1 ? ry : rz);
-  const int n = min(items_ctr[axis], item_cap);
-  const int nw = (int)gridDim.x * (int)(blockDim.x >> 5);
-  for (int item = (int)blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5); item < n; item += nw) {
-    const GridView g = views[it.igrid[axis][item]];
-    if (g.counters[C_BIG]) continue;  // warp-uniform: that grid's runs came with their slots
-    run_slots(g, axis, run, it.run[axis][item], it.slots[axis] + (size_t)item * kItemSlots);
+  if (axis == 3) {
+    const int i = (int)blockIdx.x % k;
+    if (!views[i].counters[C_BIG]) init_new_fields(views[i], (int)blockIdx.x / k, ((int)gridDim.x - 1 - i) / k + 1);
+    return;
   }
+  const int32_t* igrid = it.igrid[axis];
+  item_slots([&](int item) -> const GridView& { return views[igrid[item]]; }, axis, axis == 0 ? rx : (axis == 1 ? ry : rz),
+             it.run[axis], min(items_ctr[axis], item_cap), it.slots[axis]);
 }
 
 // Update statistics only (launched when they are asked for): the stored bricks each pass
@@ -2072,7 +2103,7 @@ cudaError_t launch_build_items_full(const GridView& g, const Tuning& t, const It
 }
 
 cudaError_t launch_item_slots(const GridView& g, const Tuning& t, const Items& it, cudaStream_t st) {
-  VDB_LAUNCH_PDL(k_item_slots, dim3(405, 3), kT, 0, st, g, t.run[0], t.run[1], t.run[2], it);
+  VDB_LAUNCH_PDL(k_item_slots, dim3(304, 4), kT, 0, st, g, t.run[0], t.run[1], t.run[2], it);
   return cudaGetLastError();
 }
 
@@ -2083,9 +2114,14 @@ cudaError_t launch_count_run_bricks(const GridView* views, const GridView& one, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_item_slots_batch(const GridView* views, const Tuning& t, const Items& it, int32_t* items_ctr,
+cudaError_t launch_init_new(const GridView& g, cudaStream_t st) {
+  VDB_LAUNCH_PDL(k_init_new, 304, kT, 0, st, g);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_item_slots_batch(const GridView* views, int k, const Tuning& t, const Items& it, int32_t* items_ctr,
                                     int item_cap, cudaStream_t st) {
-  VDB_LAUNCH(k_item_slots_batch, dim3(1216, 3), kT, 0, st, views, items_ctr, item_cap, t.run[0], t.run[1], t.run[2],
+  VDB_LAUNCH(k_item_slots_batch, dim3(1216, 4), kT, 0, st, views, k, items_ctr, item_cap, t.run[0], t.run[1], t.run[2],
              it);
   return cudaGetLastError();
 }

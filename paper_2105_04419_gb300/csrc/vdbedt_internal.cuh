@@ -427,8 +427,8 @@ cudaError_t launch_update_batch_ingest(const UpdArgs* d_args, const BatchUpdShap
                                        cudaStream_t st);
 cudaError_t launch_update_batch_mark(const UpdArgs* d_args, const BatchUpdShape& s, const Tuning& t, const Items& it,
                                      const Fork& fk, cudaStream_t st);
-// slot lists of every queued run of a batch (each run's grid from it.igrid)
-cudaError_t launch_item_slots_batch(const GridView* views, const Tuning& t, const Items& it, int32_t* items_ctr,
+// slot lists of every queued run of a batch of k grids (each run's grid from it.igrid)
+cudaError_t launch_item_slots_batch(const GridView* views, int k, const Tuning& t, const Items& it, int32_t* items_ctr,
                                     int item_cap, cudaStream_t st);
 // Update statistics: stored bricks of every run's slot list per axis into each grid's C_XB .. C_ZB
 // (views == nullptr: a single grid `one`).
@@ -445,6 +445,8 @@ cudaError_t launch_ut_pass(const GridView& g, int axis, void* scratch, cudaStrea
 // voxel; y, z: lines whose input changed), marking the next axis's lines where its output changed;
 // lines recomputed are counted in items_ctr[axis].  The z pass also refreshes the brick flags.
 cudaError_t launch_ut_update_pass(const GridView& g, int axis, void* scratch, cudaStream_t st);
+// fields of the bricks that the running update stored (the slot-list kernels below do it too)
+cudaError_t launch_init_new(const GridView& g, cudaStream_t st);
 // slot lists of every queued run (windowed form)
 cudaError_t launch_item_slots(const GridView& g, const Tuning& t, const Items& it, cudaStream_t st);
 
