@@ -119,7 +119,7 @@ __device__ __forceinline__ int isqrt_floor(int v) {
 
 // Smallest position o of [c - isqrt(want), c + isqrt(want)] along y (AXIS 1, field g1) or z (AXIS 2,
 // field g2) through (x, y, z) with field(o) = want - (o - c)^2, its value in `rest`; -1: none.  A
-// brick's eight values are loaded together (planes 128 B apart: a sector each).
+// brick's values in range are loaded together (planes 128 B apart: a sector each).
 template <int AXIS>
 __device__ __forceinline__ int line_match(const GridView& g, int x, int y, int z, int want, NodeCache& nc,
                                           int& rest) {
@@ -132,7 +132,7 @@ __device__ __forceinline__ int line_match(const GridView& g, int x, int y, int z
     const uint16_t* p = (AXIS == 1 ? g.g1 : g.g2) + (size_t)s * kBrickVox + (x & 7) + 8 * ((AXIS == 1 ? z : y) & 7);
     uint16_t v[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = __ldg(p + 64 * q);
+    for (int q = 0; q < 8; ++q) v[q] = abs(8 * b + q - c) <= r ? __ldg(p + 64 * q) : (uint16_t)0xFFFFu;
     int at = -1;
 #pragma unroll
     for (int q = 7; q >= 0; --q) {
