@@ -49,3 +49,23 @@ def test_caller_streams():
         t.join()
     session(V, torch, 3, out)
     assert out == [True, True, True]
+
+
+@pytest.mark.parametrize("pinned", [False, True])
+def test_host_queries_behind_a_running_transform(pinned):
+    import torch
+    import paper_2105_04419_gb300 as V
+    rs = np.random.default_rng(5)
+    occ = (rs.random((64, 90, 130)) < 0.001).astype(np.uint8)
+    m = V.Map(130, 90, 64, 20)
+    grid = torch.from_numpy(occ).cuda()
+    for n in (1, 1000, 300000, 17):  # the buffer grows, then is larger than the call
+        m.set_occupancy_dense(grid)
+        m.global_()
+        q = torch.from_numpy(np.stack([rs.integers(-1, k + 1, n) for k in (130, 90, 64)], 1).astype(np.int32))
+        q = (q.pin_memory() if pinned else q).numpy()
+        ref = np.pad(O.edt_factorised(occ, 20), 1, constant_values=400)
+        assert np.array_equal(m.query(q), ref[q[:, 2] + 1, q[:, 1] + 1, q[:, 0] + 1])
+        grid = torch.from_numpy(np.ascontiguousarray(occ[::-1])).cuda()
+        occ = np.ascontiguousarray(occ[::-1])
+    m.close()
