@@ -1043,7 +1043,7 @@ struct vdbedt_batch {
   Scratch scr;                     // dense-ingest scratch (all grids)
   size_t dense_bytes = 0;          // its size
   int64_t* d_dense_off = nullptr;  // per grid: mask, brick-flag, node-flag element offsets
-  size_t dense_nflag_byte = 0, dense_nflag_words = 0;
+  size_t dense_flag_byte = 0, dense_flag_words = 0;
   Tuning tune;
   std::string err;
   bool profiling = false;
@@ -1407,8 +1407,8 @@ vdbedt_status vdbedt_batch_create(const vdbedt_config* cfgs, int32_t k, vdbedt_b
       nb += (size_t)v.BX * v.BY * v.BZ;
       nk += (size_t)v.NX * v.NY * v.NZ;
     }
-    b->dense_nflag_byte = dbytes + fbytes;
-    b->dense_nflag_words = nkeys_all;
+    b->dense_flag_byte = dbytes;
+    b->dense_flag_words = fbytes / 4 + nkeys_all;
     b->dense_bytes = dbytes + fbytes + ((nkeys_all * 4 + 255) & ~(size_t)255);
     e = cudaMalloc((void**)&b->d_dense_off, sizeof(int64_t) * off.size());
     if (e != cudaSuccess) return bail(e, "device alloc");
@@ -1483,8 +1483,8 @@ vdbedt_status vdbedt_batch_set_occupancy_dense(vdbedt_batch_handle b, const uint
     }
   }
   BCK(b, ensure_scratch(b->scr, b->dense_bytes), "dense scratch");
-  BCK(b, launch_ingest_dense_batch(b->d_views, b->shape, src.data(), b->scr.buf, b->d_dense_off, b->dense_nflag_words,
-                                   (int32_t*)((char*)b->scr.buf + b->dense_nflag_byte), b->st),
+  BCK(b, launch_ingest_dense_batch(b->d_views, b->shape, src.data(), b->scr.buf, b->d_dense_off, b->dense_flag_words,
+                                   (int32_t*)((char*)b->scr.buf + b->dense_flag_byte), b->st),
       "dense ingest");
   if (!on_device) BCK(b, cudaStreamSynchronize(b->st), "sync");
   return VDBEDT_OK;

@@ -814,6 +814,42 @@ __device__ __forceinline__ uint32_t nonzero4(uint32_t w) {
   return (t * 0x00204081u) >> 28;
 }
 
+// The aligned word at address w of the bytes [lo, hi) (its bytes outside them read as zero).
+__device__ __forceinline__ uint32_t load_word(uintptr_t w, uintptr_t lo, uintptr_t hi) {
+  if (w >= lo && w + 4 <= hi) return __ldg(reinterpret_cast<const uint32_t*>(w));
+  uint32_t v = 0u;
+  for (int k = 0; k < 4; ++k)
+    if (w + k >= lo && w + k < hi) v |= (uint32_t)*reinterpret_cast<const uint8_t*>(w + k) << (8 * k);
+  return v;
+}
+
+// Up to 16 voxels (nvx) of each of nr <= 8 rows at any alignment: bit x of m[y] set where byte x of row y is
+// nonzero.  Five aligned words and a funnel shift a row, four rows' loads together (a byte at a time
+// took 50 us of a 100 x 90 x 70 map's ingest).  Not inlined: its registers would cost the aligned forms theirs.
+__device__ __noinline__ void ragged_rows(const uint8_t* rows, int pitch, int nr, int nvx, uintptr_t lo, uintptr_t hi,
+                                         uint32_t* m) {
+  for (int h = 0; h < nr; h += 4) {
+    uint32_t t[4][5], sh[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const uintptr_t at = reinterpret_cast<uintptr_t>(rows + (size_t)(h + r) * pitch);
+      sh[r] = 8u * (uint32_t)(at & 3u);
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        const uintptr_t w = (at & ~(uintptr_t)3) + 4 * q;
+        t[r][q] = h + r < nr && w < at + nvx ? load_word(w, lo, hi) : 0u;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      uint32_t v = 0u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v |= nonzero4(__funnelshift_r(t[r][q], t[r][q + 1], sh[r])) << (4 * q);
+      if (h + r < nr) m[h + r] = v & ((1u << nvx) - 1u);
+    }
+  }
+}
+
 // Scratch of the dense ingest: masks (8 words per brick of the grid, plane-major: plane z of brick
 // lb at dbits[z * bricks + lb]), brick flags, node-key flags.
 // A single grid's pointers are its own; grid i of a batch adds off[3i], off[3i + 1], off[3i + 2].
@@ -834,16 +870,25 @@ struct DenseScratch {
   }
 };
 
-// Pass 1: one warp per unit (a brick row: by, bz and up to kDenseX bricks along x).  The unit's
-// 64 input rows form eight contiguous stretches (one per plane z); each lane loads 16 bytes (two
-// bricks) of each row, a plane's eight loads issued together, and assembles both bricks' mask word
+// Pass 1: one warp per unit (a brick row: by, bz and up to kDenseX bricks along x; in small grids one of its
+// eight planes).  A plane's eight input rows are one contiguous stretch; each lane loads 16 bytes (two
+// bricks) of each row, the eight loads issued together, and assembles both bricks' mask word
 // of that plane in registers -- no shared memory, no block barrier -- and stores it to the
-// plane-major scratch (a warp's stores are one contiguous run).  After the eight planes a lane
-// writes its two bricks' flags and marks their nodes.
+// plane-major scratch (a warp's stores are one contiguous run); where it holds a bit the lane sets the
+// brick's flag and its node's (both cleared before).  With fewer than kDenseRows rows a warp per row leaves
+// the GPU idle while each works through eight planes in turn, so they are spread over eight warps (a
+// 64^3 map's masks 2.5 us, was 6.5); with more, a warp per plane repeats the row's bookkeeping
+// eight times with half the loads in flight (16 maps of 293 M voxels 140 us, a warp per row 65); a batch's
+// grids share the GPU and always take whole rows.
+constexpr int64_t kDenseRows = 1024;
 constexpr int kDenseX = 64;
+__host__ __device__ inline int64_t dense_rows(const GridView& g) {
+  return (int64_t)((g.BX + kDenseX - 1) / kDenseX) * g.BY * g.BZ;
+}
+inline int dense_planes(const GridView& g) { return dense_rows(g) < kDenseRows ? 1 : 8; }  // of a unit
 
 template <class VS, class SRC>
-__global__ void __launch_bounds__(256, 4) k_dense_masks(VS vs, SRC src, DenseScratch ds, bool zero_counters) {
+__global__ void __launch_bounds__(256, 4) k_dense_masks(VS vs, SRC src, DenseScratch ds, int planes, bool zero_counters) {
   pdl_enter();
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
@@ -855,12 +900,16 @@ __global__ void __launch_bounds__(256, 4) k_dense_masks(VS vs, SRC src, DenseScr
   ds.at(gi, dbits, flag, nflag);
   const int64_t nbr = (int64_t)g.BX * g.BY * g.BZ;
   const uint32_t nch = (uint32_t)(g.BX + kDenseX - 1) / kDenseX;
-  const uint32_t nunits = nch * (uint32_t)g.BY * (uint32_t)g.BZ;
+  const int split = planes == 1 ? 3 : 0;
+  const uint64_t nunits = (uint64_t)dense_rows(g) << split;
   const int lane = threadIdx.x & 31;
   const bool v16 = (g.nx % 16) == 0 && (reinterpret_cast<uintptr_t>(grid) & 15u) == 0;
   const bool v8 = (g.nx % 8) == 0 && (reinterpret_cast<uintptr_t>(grid) & 7u) == 0;
+  const uintptr_t lo_end = reinterpret_cast<uintptr_t>(grid), hi_end = lo_end + (size_t)g.nx * g.ny * g.nz;
   const uint32_t nw = (uint32_t)nblk * (blockDim.x >> 5);
-  for (uint32_t u = (uint32_t)bid * (blockDim.x >> 5) + (threadIdx.x >> 5); u < nunits; u += nw) {
+  for (uint64_t unit = (uint32_t)bid * (blockDim.x >> 5) + (threadIdx.x >> 5); unit < nunits; unit += nw) {
+    const int z0 = (int)unit & ((1 << split) - 1);
+    const uint32_t u = (uint32_t)(unit >> split);
     const int ch = (int)(u % nch);
     const uint32_t rest = u / nch;
     const int by = (int)(rest % (uint32_t)g.BY), bz = (int)(rest / (uint32_t)g.BY);
@@ -873,9 +922,9 @@ __global__ void __launch_bounds__(256, 4) k_dense_masks(VS vs, SRC src, DenseScr
     const uint8_t* base = grid + ((size_t)bz * 8 * g.ny + (size_t)by * 8) * g.nx + x0;
     const size_t zstride = (size_t)g.ny * g.nx;
     const int64_t lb = (bx0 + j) + (int64_t)g.BX * (by + (int64_t)g.BY * bz);
-    unsigned long long any0 = 0ull, any1 = 0ull;
+    bool any0 = false, any1 = false;
 #pragma unroll 2
-    for (int z = 0; z < 8; ++z) {
+    for (int z = z0; z < z0 + planes; ++z) {
       const uint8_t* pl = base + (size_t)z * zstride;
       const int nr = z < nplane ? nrow : 0;
       uint32_t m[8];  // row y: bits 0-7 brick j, bits 8-15 brick j + 1
@@ -897,14 +946,11 @@ __global__ void __launch_bounds__(256, 4) k_dense_masks(VS vs, SRC src, DenseScr
 #pragma unroll
         for (int y = 0; y < 8; ++y)
           m[y] = nonzero4(lo[y].x) | (nonzero4(lo[y].y) << 4) | (nonzero4(hi[y].x) << 8) | (nonzero4(hi[y].y) << 12);
-      } else {  // ragged rows: byte loads
+      } else {
+        const int nvx = min(two ? 16 : 8, g.nx - x0);
 #pragma unroll
-        for (int y = 0; y < 8; ++y) {
-          uint32_t v = 0u;
-          if (y < nr)
-            for (int x = 0; x < 16 && x0 + x < g.nx && (x < 8 || two); ++x) v |= (uint32_t)(pl[(size_t)y * g.nx + x] != 0) << x;
-          m[y] = v;
-        }
+        for (int y = 0; y < 8; ++y) m[y] = 0u;
+        ragged_rows(pl, g.nx, nr, nvx, lo_end, hi_end, m);
       }
       unsigned long long a = 0ull, b = 0ull;
 #pragma unroll
@@ -915,15 +961,17 @@ __global__ void __launch_bounds__(256, 4) k_dense_masks(VS vs, SRC src, DenseScr
       unsigned long long* plane = dbits + (size_t)z * nbr;
       plane[lb] = a;
       if (two) plane[lb + 1] = b;
-      any0 |= a;
-      any1 |= b;
+      any0 |= a != 0ull;
+      any1 |= two && b != 0ull;
     }
     const int bx = bx0 + j;
-    flag[lb] = any0 != 0ull;
-    if (any0) nflag[node_key_of(g, bx, by, bz)] = 1;
-    if (two) {
-      flag[lb + 1] = any1 != 0ull;
-      if (any1) nflag[node_key_of(g, bx + 1, by, bz)] = 1;
+    if (any0) {
+      flag[lb] = 1;
+      nflag[node_key_of(g, bx, by, bz)] = 1;
+    }
+    if (any1) {
+      flag[lb + 1] = 1;
+      nflag[node_key_of(g, bx + 1, by, bz)] = 1;
     }
   }
 }
@@ -2071,10 +2119,12 @@ cudaError_t launch_ingest_dense(const GridView& g, const uint8_t* grid, Scratch&
   DenseScratch ds{(unsigned long long*)p, (int32_t*)(p + align_up(nbr * 64)),
                   (int32_t*)(p + align_up(nbr * 64) + align_up(nbr * 4)), nullptr};
   const OneView v{g};
-  // the reset that a dense ingest starts with also clears the node flags; the counters, which its blocks
+  // the reset that a dense ingest starts with also clears the brick and node flags; the counters, which its blocks
   // read, are cleared by the next kernel
-  VDB_LAUNCH_PDL(k_reset_nodes<OneView>, 1024, kT, 0, st, v, ds.nflag, (int64_t)nkeys);
-  VDB_LAUNCH_PDL((k_dense_masks<OneView, OneSrc>), batch_blocks(g, BK_DENSE), kT, 0, st, v, OneSrc{grid}, ds, true);
+  VDB_LAUNCH_PDL(k_reset_nodes<OneView>, 1024, kT, 0, st, v, ds.flag, (int64_t)(align_up(nbr * 4) / 4 + nkeys));
+  const int planes = dense_planes(g);
+  VDB_LAUNCH_PDL((k_dense_masks<OneView, OneSrc>), blocks_for(dense_rows(g) * (8 / planes) * 32), kT, 0, st, v, OneSrc{grid}, ds,
+                 planes, true);
   VDB_LAUNCH_PDL(k_dense_nodes<OneView>, batch_blocks(g, BK_DNODES), kT, 0, st, v, ds);
   VDB_LAUNCH_PDL(k_dense_alloc<OneView>, batch_blocks(g, BK_DALLOC), kT, 0, st, v, ds);
   return cudaGetLastError();
@@ -2134,7 +2184,7 @@ int batch_blocks(const GridView& g, int kind) {
   switch (kind) {
     case BK_RESET: return clamp_blocks(((int64_t)g.node_cap * (kNodeBricks / 4) + g.hmask + t) / t, 1024);  // int4 stores
     case BK_DENSE: {
-      const int64_t units = (int64_t)((g.BX + kDenseX - 1) / kDenseX) * g.BY * g.BZ;  // a warp each
+      const int64_t units = dense_rows(g);  // a warp each
       return clamp_blocks((units * 32 + t - 1) / t, 152 * 16);
     }
     case BK_DNODES: return clamp_blocks(((int64_t)g.NX * g.NY * g.NZ + t - 1) / t, 1024);
@@ -2159,18 +2209,18 @@ cudaError_t launch_reset_batch(const GridView* views, const BatchShape& b, int32
 }
 
 cudaError_t launch_ingest_dense_batch(const GridView* views, const BatchShape& b, const uint8_t* const* srcs,
-                                      void* scratch, const int64_t* offsets, size_t nflag_words, int32_t* nflag0,
+                                      void* scratch, const int64_t* offsets, size_t flag_words, int32_t* flag0,
                                       cudaStream_t st) {
   if (b.k <= 0) return cudaSuccess;
   if (b.k > kBatchMax) return cudaErrorInvalidValue;
   BatchSrc src;
   for (int i = 0; i < kBatchMax; ++i) src.p[i] = i < b.k ? srcs[i] : nullptr;
-  cudaError_t e = cudaMemsetAsync(nflag0, 0, nflag_words * 4, st);
+  cudaError_t e = cudaMemsetAsync(flag0, 0, flag_words * 4, st);
   if (e != cudaSuccess) return e;
   char* p = (char*)scratch;
   DenseScratch ds{(unsigned long long*)p, (int32_t*)p, (int32_t*)p, offsets};
   VDB_LAUNCH((k_dense_masks<BatchViews, BatchSrc>), b.total[BK_DENSE], kT, 0, st,
-             BatchViews{views, b.first[BK_DENSE], b.k}, src, ds, false);
+             BatchViews{views, b.first[BK_DENSE], b.k}, src, ds, 8, false);
   VDB_LAUNCH_PDL(k_dense_nodes<BatchViews>, b.total[BK_DNODES], kT, 0, st, BatchViews{views, b.first[BK_DNODES], b.k}, ds);
   VDB_LAUNCH_PDL(k_dense_alloc<BatchViews>, b.total[BK_DALLOC], kT, 0, st, BatchViews{views, b.first[BK_DALLOC], b.k}, ds);
   return cudaGetLastError();

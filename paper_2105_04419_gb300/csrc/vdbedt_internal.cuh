@@ -467,10 +467,10 @@ struct BatchShape {
 cudaError_t launch_reset_batch(const GridView* views, const BatchShape& b, int32_t* counters_all, size_t n_counters,
                                cudaStream_t st);
 // scratch: grid i's masks, brick flags and node flags start offsets[3i], offsets[3i + 1] and
-// offsets[3i + 2] elements (u64, int32, int32) from the scratch base; nflag0 .. nflag0 +
-// nflag_words covers every grid's node flags
+// offsets[3i + 2] elements (u64, int32, int32) from the scratch base; flag0 .. flag0 +
+// flag_words covers every grid's brick and node flags
 cudaError_t launch_ingest_dense_batch(const GridView* views, const BatchShape& b, const uint8_t* const* srcs,
-                                      void* scratch, const int64_t* offsets, size_t nflag_words, int32_t* nflag0,
+                                      void* scratch, const int64_t* offsets, size_t flag_words, int32_t* flag0,
                                       cudaStream_t st);
 cudaError_t launch_activation_batch(const GridView* views, const BatchShape& b, cudaStream_t st);
 cudaError_t launch_build_items_batch(const GridView* views, const BatchShape& b, const Tuning& t, const Items& it,
