@@ -19,9 +19,9 @@
 // compute, write, and release the stage on its "empty" barrier.  No block-wide barrier sits on
 // the main path, so warps whose windows exit early run ahead.
 //   x (AXIS 0): inputs are the 64-byte occupancy masks.  Each lane expands two x-lines: the line's
-//     occupancy is gathered from the masks of bricks bx-R..bx+R (one byte each) and the nearest
-//     set bit on either side of each voxel is found with clz / ffs on a 64-bit window.  g1 is
-//     stored y-major so that the y pass reads it as planes.
+//     occupancy is gathered from the masks of bricks bx-R..bx+R (one byte each), the nearest set bits outside
+//     the brick found by counts of leading and trailing zeros (x_compute_rows).  g1 is stored y-major so
+//     that the y pass reads it as planes.
 //   y, z (AXIS 1, 2): inputs are 1 KB bricks of g1 / g2.  In the staged column a plane along the
 //     pass axis is 32 words (two voxels per word) and a lane's line is one word per plane, so the
 //     32 lanes of a consumer read 32 consecutive words.
@@ -164,130 +164,99 @@ struct ColShape {
   static constexpr int THREADS = 32 * (RUN + 1);
   static constexpr size_t DATA_BYTES = (size_t)NS * STAGE_BYTES;
   static constexpr size_t META_BYTES = (size_t)NS * META * 4;
-  static constexpr size_t LUT_BYTES = 80;  // x pass: min(d^2, dmax^2), d = 0..32
-  static constexpr size_t SMEM = DATA_BYTES + ((META_BYTES + 15) & ~(size_t)15) + 2 * NS * 8 + LUT_BYTES + 16;
+  static constexpr size_t TABLE_BYTES = AXIS == 0 ? 4096 : 0;  // x pass: ByteTable
+  static constexpr size_t SMEM = DATA_BYTES + ((META_BYTES + 15) & ~(size_t)15) + 2 * NS * 8 + TABLE_BYTES + 16;
 };
 
-// x pass of one brick from the staged masks of bricks w .. w + 2R (64 B each; byte y + 8 z is the
-// x-row (y, z)).  Lane: z = lane & 7, rows y0 = 2 (lane >> 3) and y0 + 1.  g1 is stored y-major.
-// For dmax <= 32 (and R <= 4) a distance of 32 or more is already saturated, so each voxel needs
-// only the 32 line bits on either side: two funnel shifts of 32-bit words and a count of leading
-// zeros (left) and of trailing zeros (right).  Otherwise the 64-bit form covers the whole line.
-template <int R>
-__device__ __forceinline__ void x_compute_rows(const GridView& g, const uint32_t (&rows2)[2 * R + 1], int slot,
-                                               uint32_t inf2, const uint16_t* lut);
+// Distances inside one byte: entry m holds, for voxels 0 .. 7, the distance to the nearest set bit of m (64:
+// none), two voxels to a word.
+struct ByteTable {
+  uint32_t w[256][4];
+  constexpr ByteTable() : w{} {
+    for (int m = 0; m < 256; ++m)
+      for (int x = 0; x < 8; ++x) {
+        uint32_t best = 64;
+        for (int j = 0; j < 8; ++j)
+          if ((m >> j) & 1) {
+            const uint32_t d = (uint32_t)(j < x ? x - j : j - x);
+            if (d < best) best = d;
+          }
+        w[m][x / 2] |= best << (16 * (x & 1));
+      }
+  }
+};
+__device__ const ByteTable kByteTable{};
 
-template <int R>
-__device__ __forceinline__ void x_compute(const GridView& g, const uint8_t* masks, int slot, uint32_t inf2,
-                                          const uint16_t* lut) {
-  constexpr int NBX = 2 * R + 1;
-  const int lane = threadIdx.x & 31;
-  const int z = lane & 7, y0 = (lane >> 3) * 2;
-  uint32_t rows2[NBX];
-#pragma unroll
-  for (int b = 0; b < NBX; ++b) rows2[b] = *reinterpret_cast<const uint16_t*>(masks + b * 64 + y0 + 8 * z);
-  x_compute_rows<R>(g, rows2, slot, inf2, lut);
+// The table in shared memory, copied by the whole block (no barrier).
+__device__ __forceinline__ void load_byte_table(uint4* table) {
+  for (int i = threadIdx.x; i < 256; i += blockDim.x) table[i] = reinterpret_cast<const uint4*>(kByteTable.w)[i];
 }
 
-// The x-line computation of one brick from the lane's two mask bytes of each brick of the window
-// (rows2[b]: bits of x-rows y0 (low byte) and y0 + 1 (high byte) at z, brick bx - R + b).
+// x pass of one brick from the masks of bricks bx - R .. bx + R (64 B each; byte y + 8 z is the x-row (y, z)).
+// Lane: z = lane & 7, rows y0 = 2 (lane >> 3) and y0 + 1, whose bytes of brick b are rows2[b] (low, high).  g1 is
+// stored y-major.  A row's nearest bits outside the brick are one count of leading zeros (left) and one of
+// trailing zeros (right) of the four neighbouring bytes on that side (and of two more for R > 4); from those
+// distances A and B the eight voxels have A + x and B + 7 - x, two to a word, against the distances inside
+// the brick's own byte (a table), and the minimum, at most dmax, is squared.  Bound by issue: about 140
+// instructions a brick and lane for 1 KB written; 1024 x 1024 x 256 tunnel scene, dmax 32: 0.115 ms, 0.106 in runs of 8 (a
+// funnel shift and a count per voxel and side with a table of squares: 0.139).
 template <int R>
 __device__ __forceinline__ void x_compute_rows(const GridView& g, const uint32_t (&rows2)[2 * R + 1], int slot,
-                                               uint32_t inf2, const uint16_t* lut) {
-  constexpr int NBX = 2 * R + 1;
+                                               const uint4* __restrict__ table) {
   const int lane = threadIdx.x & 31;
   const int z = lane & 7, y0 = (lane >> 3) * 2;
+  const uint32_t dmax2 = twice((uint32_t)g.dmax);
+  auto at = [&](int b) -> uint32_t { return b >= 0 && b <= 2 * R ? rows2[b] : 0u; };
+  // the four bytes of bricks b .. b + 3 of either row
+  auto four = [&](int b, uint32_t (&w)[2]) {
+    const uint32_t t01 = __byte_perm(at(b), at(b + 1), 0x5140), t23 = __byte_perm(at(b + 2), at(b + 3), 0x5140);
+    w[0] = __byte_perm(t01, t23, 0x5410);
+    w[1] = __byte_perm(t01, t23, 0x7632);
+  };
+  uint32_t lw[2], rw[2];
+  four(R - 4, lw);
+  four(R + 1, rw);
   bool fin = false;
-  uint32_t w[2][4];
-  bool done = false;
-  if constexpr (R <= 4) {
-    if (g.dmax <= 32) {
-      // E[r][1 + k] holds line bits 32k .. 32k + 31; E[r][0] = 0 stands for positions -32 .. -1.
-      // Byte b of the line is brick b's row: gathered with byte permutes (rows y0 and y0 + 1 are
-      // the low and high bytes of rows2[b]).
-      uint32_t E[2][5] = {{0u, 0u, 0u, 0u, 0u}, {0u, 0u, 0u, 0u, 0u}};
 #pragma unroll
-      for (int k = 1; k <= 3; ++k) {
-        const int b0 = 4 * (k - 1);
-        if (b0 < NBX) {
-          const uint32_t a = rows2[b0], b = b0 + 1 < NBX ? rows2[b0 + 1] : 0u;
-          const uint32_t c = b0 + 2 < NBX ? rows2[b0 + 2] : 0u, d = b0 + 3 < NBX ? rows2[b0 + 3] : 0u;
-          const uint32_t t01 = __byte_perm(a, b, 0x5140), t23 = __byte_perm(c, d, 0x5140);
-          E[0][k] = __byte_perm(t01, t23, 0x5410);
-          E[1][k] = __byte_perm(t01, t23, 0x7632);
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        if ((E[r][1] | E[r][2] | E[r][3]) == 0u) {
-          w[r][0] = w[r][1] = w[r][2] = w[r][3] = inf2;
-          continue;
-        }
-        uint32_t hv[8];
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-          const int P = 8 * R + x + 32;  // position in E
-          const int s0 = P - 31;
-          const uint32_t Lw = __funnelshift_r(E[r][s0 >> 5], E[r][(s0 >> 5) + 1], s0 & 31);  // bit 31 = P
-          const uint32_t Rw = __funnelshift_r(E[r][P >> 5], E[r][(P >> 5) + 1], P & 31);      // bit 0 = P
-          const int d = min(__clz(Lw), __clz(__brev(Rw)));  // 32 when the side is empty
-          fin |= d < g.dmax;                                  // d^2 < dmax^2
-          hv[x] = lut[d];                                     // min(d^2, dmax^2)
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) w[r][q] = hv[2 * q] | (hv[2 * q + 1] << 16);
-      }
-      done = true;
+  for (int r = 0; r < 2; ++r) {
+    const uint32_t own = (rows2[R] >> (8 * r)) & 0xFFu;
+    uint32_t w[4];
+    int A = __clz(lw[r]) + 1, B = __clz(__brev(rw[r])) + 1;  // 33: none in the four bytes
+    if constexpr (R > 4) {
+      // the next two bytes on either side, the nearer one on top (left) or below (right)
+      const uint32_t lf = ((at(R - 5) >> (8 * r)) & 0xFFu) << 8 | ((at(R - 6) >> (8 * r)) & 0xFFu);
+      const uint32_t rf = ((at(R + 5) >> (8 * r)) & 0xFFu) | ((at(R + 6) >> (8 * r)) & 0xFFu) << 8;
+      if (lw[r] == 0u) A = 33 + (lf ? __clz(lf << 16) : 32);
+      if (rw[r] == 0u) B = 33 + (rf ? __ffs(rf) - 1 : 32);
     }
+    if (own == 0u && min(A, B) >= g.dmax) {
+      w[0] = w[1] = w[2] = w[3] = twice((uint32_t)g.INF);
+    } else {
+      fin = true;
+      const uint4 t = table[own];
+      const uint32_t in[4] = {t.x, t.y, t.z, t.w}, a2 = twice((uint32_t)A), b2 = twice((uint32_t)B);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t l = a2 + (uint32_t)(2 * q | (2 * q + 1) << 16), h = b2 + (uint32_t)((7 - 2 * q) | (6 - 2 * q) << 16);
+        const uint32_t d = __vminu2(__vimin3_u16x2(l, h, in[q]), dmax2);
+        const uint32_t lo = d & 0xFFFFu;
+        w[q] = (d >> 16) * (d & 0xFFFF0000u) + lo * lo;
+      }
+    }
+    *reinterpret_cast<uint4*>(g.g1 + (size_t)slot * kBrickVox + (y0 + r) * 64 + z * 8) = make_uint4(w[0], w[1], w[2], w[3]);
   }
-  if (!done) {
-    unsigned long long lo[2] = {0ull, 0ull}, hi[2] = {0ull, 0ull};
-#pragma unroll
-    for (int b = 0; b < NBX; ++b) {
-      const uint32_t two = rows2[b];
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const unsigned long long byte = (two >> (8 * r)) & 0xFFu;
-        if (b < 8)
-          lo[r] |= byte << (8 * b);
-        else
-          hi[r] |= byte << (8 * (b - 8));
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      if ((lo[r] | hi[r]) == 0ull) {
-        w[r][0] = w[r][1] = w[r][2] = w[r][3] = inf2;
-      } else {
-        uint32_t hv[8];
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-          const int p = 8 * R + x;  // position of voxel x in the line (8 <= p < 64 for 1 <= R <= 6)
-          int best = g.INF;
-          const unsigned long long L = lo[r] & ((2ull << p) - 1ull);
-          if (L) {
-            const int dl = p - (63 - __clzll((long long)L));
-            best = min(best, dl * dl);
-          }
-          const unsigned long long Rm = (lo[r] >> p) | (hi[r] << (64 - p));
-          if (Rm) {
-            const int dr = __ffsll((long long)Rm) - 1;
-            best = min(best, dr * dr);
-          }
-          fin |= best < g.INF;
-          hv[x] = (uint32_t)best;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) w[r][q] = hv[2 * q] | (hv[2 * q + 1] << 16);
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < 2; ++r)
-    *reinterpret_cast<uint4*>(g.g1 + (size_t)slot * kBrickVox + (y0 + r) * 64 + z * 8) =
-        make_uint4(w[r][0], w[r][1], w[r][2], w[r][3]);
   const unsigned anyfin = __any_sync(0xffffffffu, fin);
   if (lane == 0) set_flag_bit(g, slot, F_G1FIN, anyfin);
+}
+
+template <int R>
+__device__ __forceinline__ void x_compute(const GridView& g, const uint8_t* masks, int slot, const uint4* table) {
+  const int lane = threadIdx.x & 31;
+  const int z = lane & 7, y0 = (lane >> 3) * 2;
+  uint32_t rows2[2 * R + 1];
+#pragma unroll
+  for (int b = 0; b <= 2 * R; ++b) rows2[b] = *reinterpret_cast<const uint16_t*>(masks + b * 64 + y0 + 8 * z);
+  x_compute_rows<R>(g, rows2, slot, table);
 }
 
 // y or z pass of one brick: the staged column holds planes along the pass axis, 32 words each
@@ -357,7 +326,7 @@ __global__ void __launch_bounds__(32 * (RUN + 1), pass_min_blocks(RUN, AXIS))
   int* meta = reinterpret_cast<int*>(smem + S::DATA_BYTES);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::DATA_BYTES + ((S::META_BYTES + 15) & ~(size_t)15));
   uint64_t* empty = full + NS;
-  uint16_t* lut = reinterpret_cast<uint16_t*>(empty + NS);
+  uint4* table = reinterpret_cast<uint4*>(empty + NS);  // 16-byte aligned: whole pairs of barriers before it
   const int nitems = min(g.items_ctr[AXIS], max_items);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t inf2 = twice((uint32_t)g.INF);
@@ -367,7 +336,7 @@ __global__ void __launch_bounds__(32 * (RUN + 1), pass_min_blocks(RUN, AXIS))
       mbar_init(&empty[s], RUN);
     }
   }
-  if (AXIS == 0 && threadIdx.x <= 32) lut[threadIdx.x] = (uint16_t)min((int)(threadIdx.x * threadIdx.x), g.INF);
+  if (AXIS == 0) load_byte_table(table);
   __syncthreads();
 
   if (warp == 0) {
@@ -432,7 +401,7 @@ __global__ void __launch_bounds__(32 * (RUN + 1), pass_min_blocks(RUN, AXIS))
     if (slot >= 0) {
       const unsigned char* stage = data + (size_t)s * S::STAGE_BYTES;
       if (AXIS == 0)
-        x_compute<R>(g, stage + w * 64, slot, inf2, lut);
+        x_compute<R>(g, stage + w * 64, slot, table);
       else
         window_compute<R, AXIS>(g, reinterpret_cast<const uint32_t*>(stage), m + NB, slot, w, prune, inf2);
     }
@@ -452,12 +421,11 @@ __global__ void __launch_bounds__(256) k_x_direct(GridView g, const int32_t* __r
   const int nitems = min(g.items_ctr[0], max_items);
   const int lane = threadIdx.x & 31;
   const int z = lane & 7, y0 = (lane >> 3) * 2;
-  const uint32_t inf2 = twice((uint32_t)g.INF);
   const int64_t total = (int64_t)nitems * run;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const unsigned char* occ = reinterpret_cast<const unsigned char*>(g.occ);
-  __shared__ uint16_t lut[33];
-  if (threadIdx.x <= 32) lut[threadIdx.x] = (uint16_t)min((int)(threadIdx.x * threadIdx.x), g.INF);
+  __shared__ uint4 table[256];
+  load_byte_table(table);
   __syncthreads();
   for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += nw) {
     const int item = (int)(w / run), j = (int)(w % run);
@@ -471,7 +439,7 @@ __global__ void __launch_bounds__(256) k_x_direct(GridView g, const int32_t* __r
       const int sb = __shfl_sync(0xffffffffu, s, b);
       rows2[b] = sb >= 0 ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(occ + (size_t)sb * 64 + y0 + 8 * z)) : 0u;
     }
-    x_compute_rows<R>(g, rows2, slot, inf2, lut);
+    x_compute_rows<R>(g, rows2, slot, table);
   }
 }
 
@@ -840,7 +808,15 @@ GridView pool_view(const GridView& g) {
   return p;
 }
 
+// Passes over at most this many bricks of capacity are chained to the kernel before them (programmatic
+// launch): there a launch costs as much as the pass (160^3: 65.7 us a call with its export, 70.2 without).
+// A pass that fills the GPU is launched on its own: started early, its blocks take the places that the
+// previous pass's leave one by one, and y and z together took 0.82 ms where they take 0.65 (1024 x 1024 x 256
+// tunnel scene, dmax 32).
+constexpr int kChainBricks = 16384;
+
 cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, bool chained, cudaStream_t st) {
+  chained = chained && g.item_cap <= kChainBricks;
   const bool prune = (t.variant & 3) != 1;
   if (windowed_form(g)) {
     const GridView p = pool_view(g);
