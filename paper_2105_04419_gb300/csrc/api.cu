@@ -398,7 +398,7 @@ vdbedt_status create_impl(const vdbedt_config* cfg, const PoolSlice* slice, vdbe
   AL(g.mwork, node_cap * 384);
   AL(g.nclaim, node_cap * 128);
   AL(g.node_key, node_cap);
-  AL(g.mark, node_cap * 3 * 1024);
+  AL(g.mark, node_cap * (kMarkWords + 1));  // and the list of nodes
   if (slice) {
     g.occ = slice->occ;
     g.g1 = slice->g1;
@@ -441,7 +441,7 @@ vdbedt_status create_impl(const vdbedt_config* cfg, const PoolSlice* slice, vdbe
   cudaMemsetAsync(g.amask, 0, sizeof(uint32_t) * (size_t)node_cap * 128, h->st);
   cudaMemsetAsync(g.mwork, 0, sizeof(uint32_t) * (size_t)node_cap * 384, h->st);
   cudaMemsetAsync(g.nclaim, 0, sizeof(uint32_t) * (size_t)node_cap * 128, h->st);
-  cudaMemsetAsync(g.mark, 0, sizeof(int32_t) * (size_t)node_cap * 3 * 1024, h->st);
+  cudaMemsetAsync(g.mark, 0, sizeof(uint32_t) * (size_t)node_cap * kMarkWords, h->st);
   if (!slice) cudaMemsetAsync(g.counters, 0, sizeof(int32_t) * C_NUM, h->st);
   if (untrunc) {
     cudaMemsetAsync(g.ut_bits, 0, sizeof(uint32_t) * (size_t)ut_bits_words(g), h->st);
@@ -733,9 +733,9 @@ vdbedt_status vdbedt_update(vdbedt_handle h, vdbedt_update_stats* stats) {
     mark(h, 1);
     CK(h, launch_incremental_mark(h->g, t, h->changed, h->items, h->fork, h->st), "mark");
     mark(h, 2);
-    // slot lists of the dirty runs (an update that switched to the global form got them with its
-    // work lists), then the side stream's branch joins before the passes
-    CK(h, windowed_form(h->g) ? launch_item_slots(h->g, t, h->items, h->st) : launch_init_new(h->g, h->st), "item slots");
+    // work lists of the dirty runs (an update that switched to the global form gets its own on the side
+    // stream, whose branch joins before the passes)
+    CK(h, launch_items_dirty(h->g, t, h->items, windowed_form(h->g), h->st), "items");
     CK(h, cudaStreamWaitEvent(h->st, h->fork.join, 0), "join");
     s = run_passes(h, t, true);
     if (s) return s;
@@ -1213,9 +1213,9 @@ vdbedt_status batch_update(vdbedt_batch* b, vdbedt_update_stats* stats) {
     for (vdbedt_map* m : b->maps) clear_stage(m);
     bmark(b, 1);
     BCK(b, launch_update_batch_mark(b->d_upd, shape, t, b->items, b->fork, b->st), "mark");
-    BCK(b, cudaStreamWaitEvent(b->st, b->fork.join, 0), "join");
     bmark(b, 2);
-    BCK(b, launch_item_slots_batch(b->d_views, b->k, t, b->items, b->pool.items_ctr, b->pool.item_cap, b->st), "item slots");
+    BCK(b, launch_items_dirty_batch(b->d_upd, b->k, t, b->items, b->st), "items");
+    BCK(b, cudaStreamWaitEvent(b->st, b->fork.join, 0), "join");
     bmark(b, 3);
     BCK(b, launch_pass(b->pool, t, 0, b->items, false, b->st), "x pass");
     bmark(b, 4);

@@ -136,13 +136,13 @@ __global__ void k_reset_nodes(VS vs, int32_t* __restrict__ clear, int64_t clear_
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
   (void)gi;
-  // per used node: 4096 child slots, 3 x 1024 marks, 128 activity words and 384 work words, all
+  // per used node: 4096 child slots, 128 dirty-run words, 128 activity words and 384 work words, all
   // whole 16-byte vectors (the per-node arrays start at multiples of their node strides)
   const int64_t nn = min(g.counters[C_NNODES], g.node_cap);
   const int64_t stride = (int64_t)nblk * blockDim.x, t0 = (int64_t)bid * blockDim.x + threadIdx.x;
   const int4 none = make_int4(kNoSlot, kNoSlot, kNoSlot, kNoSlot), zero = make_int4(0, 0, 0, 0);
   for (int64_t i = t0; i < nn * (kNodeBricks / 4); i += stride) reinterpret_cast<int4*>(g.child)[i] = none;
-  for (int64_t i = t0; i < nn * (3 * 1024 / 4); i += stride) reinterpret_cast<int4*>(g.mark)[i] = zero;
+  for (int64_t i = t0; i < nn * (kMarkWords / 4); i += stride) reinterpret_cast<int4*>(g.mark)[i] = zero;
   for (int64_t i = t0; i < nn * (128 / 4); i += stride) reinterpret_cast<int4*>(g.amask)[i] = zero;
   for (int64_t i = t0; i < nn * (384 / 4); i += stride) reinterpret_cast<int4*>(g.mwork)[i] = zero;
   for (int64_t i = t0; i < nn * (128 / 4); i += stride) reinterpret_cast<int4*>(g.nclaim)[i] = zero;
@@ -170,6 +170,7 @@ __global__ void k_begin_update(US us) {
     g.counters[C_YB] = 0;
     g.counters[C_ZB] = 0;
     g.counters[C_BIG] = 0;
+    g.counters[C_DIRTY_NODES] = 0;
     g.counters[C_NB_START] = g.counters[C_NBRICKS];
     g.counters[C_EPOCH] += 1;
   }
@@ -195,6 +196,7 @@ __global__ void k_begin_batch_update(const UpdArgs* __restrict__ args, BatchCoun
     g.counters[C_YB] = 0;
     g.counters[C_ZB] = 0;
     g.counters[C_BIG] = 0;
+    g.counters[C_DIRTY_NODES] = 0;
     g.counters[C_NB_START] = g.counters[C_NBRICKS];
     g.counters[C_EPOCH] += 1;
   }
@@ -1349,220 +1351,209 @@ __global__ void __launch_bounds__(256) k_alloc_marked(VS vs, bool zero_items) {
 }
 
 // ---- work items ----
-// Claim the run along `axis` that holds brick (bx, by, bz) (runs are aligned to `run` bricks inside
-// the node) for this epoch: true for the one caller that queues it, with the run's first brick in
-// `packed`.  A plain read first lets runs already claimed in this epoch skip the exchange (a value
-// read before another thread's exchange only leads to the exchange).
-__device__ __forceinline__ bool claim_run(const GridView& g, int axis, int bx, int by, int bz, int node, int run,
-                                          int epoch, unsigned long long& packed) {
-  // run is 4, 8 or 16: a shift and a mask instead of a division
-  const int la = axis == 0 ? bx & 15 : (axis == 1 ? by & 15 : bz & 15);
-  const int l1 = axis == 0 ? by & 15 : bx & 15, l2 = axis == 2 ? by & 15 : bz & 15;
-  int* mk = &g.mark[((size_t)node * 3 + axis) * 1024 + l1 + 16 * (l2 + 16 * (la >> (__ffs(run) - 1)))];
-  if (__ldcg(mk) == epoch || atomicExch(mk, epoch) == epoch) return false;
-  const int back = la & (run - 1);
-  packed = pack_brick(bx - (axis == 0 ? back : 0), by - (axis == 1 ? back : 0), bz - (axis == 2 ? back : 0));
-  return true;
+// An update's dirty runs: per node 32 words for each axis (z, y and x runs; word 8 q + line / 32, q the run
+// along the axis, line = o1 + 16 o2 over the two axes across it, as k_items_nodes numbers them), then the
+// epoch of the node's last entry in the list of nodes with such bits, which follows the nodes' words.  The
+// words are zero between updates: the kernel that queues the runs clears them.
+__device__ __forceinline__ uint32_t* dirty_words(const GridView& g, int node, int axis, int q) {
+  return g.mark + (size_t)node * kMarkWords + axis * 32 + q * 8;
+}
+__device__ __forceinline__ int32_t* dirty_nodes(const GridView& g) {
+  return reinterpret_cast<int32_t*>(g.mark + (size_t)g.node_cap * kMarkWords);
+}
+// Node into the list once per epoch (a plain read first: most nodes are already there).
+__device__ __forceinline__ void list_dirty_node(const GridView& g, int node, uint32_t epoch) {
+  uint32_t* e = g.mark + (size_t)node * kMarkWords + 96;
+  if (__ldcg(e) == epoch || atomicExch(e, epoch) == epoch) return;
+  dirty_nodes(g)[atomicAdd(&g.counters[C_DIRTY_NODES], 1)] = node;
 }
 
-// Append the claimed runs (won[a]: this thread's run along axis a) to the three axes' work lists
-// (block-uniform call; in a batch, igrid records each run's grid): the warps' counts are summed in
-// shared memory and each list's counter word takes one atomic per block -- one per warp would
-// queue thousands of atomics on the same word in a frame's marking.
-__device__ __forceinline__ void emit_runs3(const GridView& g, const bool (&won)[3], const unsigned long long (&packed)[3],
-                                           const Items& it, int grid) {
-  __shared__ int cnt[3], base[3];
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x < 3) cnt[threadIdx.x] = 0;
-  __syncthreads();
-  int off[3];
+// Voxel gap between two bricks d apart along an axis: the nearest voxels of bricks 0 and d are
+// 8 |d| - 7 apart (0 for the same brick).
+__device__ __forceinline__ int brick_gap(int d) {
+  d = abs(d);
+  return d == 0 ? 0 : 8 * d - 7;
+}
+// largest |d| along an axis with brick_gap(d)^2 < rem (rem >= 1, below 2^24: the root is exact)
+__device__ __forceinline__ int gap_reach(int rem) { return ((int)__fsqrt_rn((float)(rem - 1)) + 7) >> 3; }
+
+// Bricks of changed brick c's cube (R bricks around it inside the grid) and its marking units: one per
+// (z run, row), one per y run, one for the x runs.
+struct DirtyCube {
+  int x0, x1, y0, y1, z0, z1, nyr, nz, units;
+  __device__ __forceinline__ DirtyCube(const GridView& g, const int4& c, int ry, int rz) {
+    const int R = g.R;
+    x0 = max(c.x - R, 0), x1 = min(c.x + R, g.BX - 1);
+    y0 = max(c.y - R, 0), y1 = min(c.y + R, g.BY - 1);
+    z0 = max(c.z - R, 0), z1 = min(c.z + R, g.BZ - 1);
+    nyr = y1 - y0 + 1;
+    nz = (z1 >> (__ffs(rz) - 1)) - (z0 >> (__ffs(rz) - 1)) + 1;  // runs are 4, 8 or 16
+    units = nz * nyr + ((y1 >> (__ffs(ry) - 1)) - (y0 >> (__ffs(ry) - 1)) + 1) + 1;
+  }
+};
+
+// Unit u of changed brick c: the bits of the runs along one axis in one row along x (along x itself: of c's
+// x runs).  node(bx, by, bz): the node of a brick, -1 for none (then nothing is stored there).
+template <class Node>
+__device__ __forceinline__ void mark_dirty(const GridView& g, const int4& c, const DirtyCube& k, int u, int rx, int ry,
+                                           int rz, Node node) {
+  const int nzu = k.nz * k.nyr;
+  if (u == k.units - 1) {  // x runs of c's row
+    const int m = gap_reach(g.INF), xa = max(k.x0, c.x - m), xe = min(k.x1, c.x + m);
+    const int line = (c.y & 15) + 16 * (c.z & 15);
+    for (int x = xa & ~(rx - 1); x <= xe; x += rx) {
+      const int n = node(x, c.y, c.z);
+      if (n >= 0) atomicOr(dirty_words(g, n, 0, (x & 15) >> (__ffs(rx) - 1)) + (line >> 5), 1u << (line & 31));
+    }
+    return;
+  }
+  const bool z = u < nzu;
+  const int run = z ? rz : ry, lo = z ? k.z0 : k.y0, hi = z ? k.z1 : k.y1, at = z ? c.z : c.y;
+  const int r = (lo & ~(run - 1)) + (z ? u / k.nyr : u - nzu) * run;  // the run's first brick along the axis
+  const int s = max(r, lo), e = min(r + run - 1, hi);
+  const int by = z ? k.y0 + u % k.nyr : s, bz = z ? s : c.z;
+  // its nearest brick's gap along the axis, and the row's gap across it (y runs: in c's layer)
+  const int ga = brick_gap(at < s ? s - at : (at > e ? at - e : 0)), gr = z ? brick_gap(by - c.y) : 0;
+  const int rem = g.INF - ga * ga - gr * gr;
+  if (rem <= 0) return;
+  const int m = gap_reach(rem), xe = min(k.x1, c.x + m), o2 = (z ? by : bz) & 15;
+  for (int x = max(k.x0, c.x - m); x <= xe;) {  // node by node
+    const int xl = min(xe, x | 15), n = node(x, by, bz);
+    if (n >= 0)
+      atomicOr(dirty_words(g, n, z ? 2 : 1, (r & 15) >> (__ffs(run) - 1)) + (o2 >> 1),
+               (((1u << (xl - x + 1)) - 1u) << (x & 15)) << (16 * (o2 & 1)));
+    x = xl + 1;
+  }
+}
+
+// The runs of a node along one axis: queued where they hold a stored brick (DIRTY: and their dirty bit is set,
+// which is cleared here).  The block's 256 threads cover the 16 x 16 lines of the node across the axis, qrun is
+// the run along it.  A block-wide scan compacts the runs and one atomic reserves their places; the run slot
+// lists are then read straight from the child tables of the node and of its neighbour along the axis
+// (R <= 6 < 16, so the halo reaches at most one node each way), one slot per thread.
+template <bool DIRTY>
+__device__ __forceinline__ void node_runs(const GridView& g, int gi, int node, int axis, int qrun, int run, const Items& it,
+                                          bool with_slots) {
+  __shared__ int wsum[8];
+  __shared__ int base_sh, count_sh;
+  __shared__ int nbr_sh[2];
+  __shared__ unsigned char lines[256];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int R = g.R;
+  bool dirty = true;
+  if (DIRTY) {
+    uint32_t* w = dirty_words(g, node, axis, qrun) + warp;
+    const uint32_t bits = *w;
+    dirty = (bits >> lane & 1u) != 0u;
+    if (!__syncthreads_or(dirty)) return;
+    if (lane == 0 && bits) *w = 0u;
+  }
+  int q[3];
+  node_coords(g, (unsigned long long)g.node_key[node], q[0], q[1], q[2]);
+  const int32_t* ch = g.child + (size_t)node * kNodeBricks;
+  const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
+  const int r0 = qrun * run, nb = run + 2 * R;
+  if (threadIdx.x < 2) {
+    int qq[3] = {q[0], q[1], q[2]};
+    qq[axis] += threadIdx.x == 0 ? -1 : 1;
+    int n2 = -1;
+    if (qq[0] >= 0 && qq[1] >= 0 && qq[2] >= 0 && qq[0] < g.NX && qq[1] < g.NY && qq[2] < g.NZ)
+      n2 = find_node(g, node_key_at(g, qq[0], qq[1], qq[2]));
+    nbr_sh[threadIdx.x] = n2;
+  }
+  const int o1 = threadIdx.x & 15, o2 = threadIdx.x >> 4;
+  bool any = false;
+  if (!DIRTY || dirty) {
+    // the run's child entries along the line, all read before any is tested
+    const int across = (o1 << (4 * a1)) | (o2 << (4 * a2));
+    int c[16];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const unsigned m = __ballot_sync(0xffffffffu, won[a]);
-    int wb = 0;
-    if (lane == 0 && m) wb = atomicAdd(&cnt[a], __popc(m));
-    off[a] = __shfl_sync(0xffffffffu, wb, 0) + __popc(m & ((1u << lane) - 1u));
+    for (int j = 0; j < 16; ++j) c[j] = j < run ? ch[across | ((r0 + j) << (4 * axis))] : -1;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) any |= c[j] >= 0;
+  }
+  const unsigned bal = __ballot_sync(0xffffffffu, any);
+  if (lane == 0) wsum[warp] = __popc(bal);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int tot = 0;
+    for (int w = 0; w < 8; ++w) {
+      const int t = wsum[w];
+      wsum[w] = tot;
+      tot += t;
+    }
+    count_sh = tot;
+    base_sh = tot ? atomicAdd(&g.items_ctr[axis], tot) : 0;
   }
   __syncthreads();
-  if (threadIdx.x < 3) base[threadIdx.x] = cnt[threadIdx.x] ? atomicAdd(&g.items_ctr[threadIdx.x], cnt[threadIdx.x]) : 0;
-  __syncthreads();
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int p = base[a] + off[a];
-    if (won[a] && p < g.item_cap) {
-      it.run[a][p] = packed[a];
-      if (it.igrid[a]) it.igrid[a][p] = grid;
+  const int base = base_sh, cnt = count_sh;
+  if (any) {
+    const int pos = wsum[warp] + __popc(bal & ((1u << lane) - 1u));
+    lines[pos] = (unsigned char)threadIdx.x;
+    const int p = base + pos;
+    if (p < g.item_cap) {
+      int l0[3];
+      l0[axis] = r0;
+      l0[a1] = o1;
+      l0[a2] = o2;
+      it.run[axis][p] = pack_brick(q[0] * 16 + l0[0], q[1] * 16 + l0[1], q[2] * 16 + l0[2]);
+      if (it.igrid[axis]) it.igrid[axis][p] = gi;
     }
   }
+  __syncthreads();
+  if (with_slots) {
+    // four slots per thread and round, their child reads issued before any is written
+    const int total = cnt * nb;
+    for (int idx0 = threadIdx.x; idx0 < total; idx0 += 4 * 256) {
+      int sv[4];
+      int64_t dst[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int idx = idx0 + u * 256;
+        sv[u] = -1;
+        dst[u] = -1;
+        if (idx < total) {
+          const int i = idx / nb, j = idx % nb;
+          const int p = base + i;
+          if (p < g.item_cap) {
+            const int line = lines[i];
+            int c = r0 + j - R, src = node;
+            if (c < 0) {
+              c += 16;
+              src = nbr_sh[0];
+            } else if (c >= 16) {
+              c -= 16;
+              src = nbr_sh[1];
+            }
+            dst[u] = (int64_t)p * kItemSlots + j;
+            // local brick: c along the axis, the line's two coordinates across it
+            const int lb = (c << (4 * axis)) | ((line & 15) << (4 * a1)) | ((line >> 4) << (4 * a2));
+            if (src >= 0) sv[u] = g.child[(size_t)src * kNodeBricks + lb];
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (dst[u] >= 0) it.slots[axis][dst[u]] = sv[u] >= 0 ? sv[u] + g.slot_base : -1;
+    }
+  }
+  __syncthreads();
 }
 
 // Global form: every run that holds a stored brick, found node by node.  Block = (node, axis, run
-// index along the axis); its 256 threads cover the 16 x 16 lines of the node across the axis.  A
-// block-wide scan compacts the runs and one atomic reserves their places; the run slot lists are
-// then read straight from the child tables of the node and of its neighbour along the axis
-// (R <= 6 < 16, so the halo reaches at most one node each way), one slot per thread.
+// index along the axis).
 template <class VS>
 __global__ void __launch_bounds__(256) k_items_nodes(VS vs, int rx, int ry, int rz, Items it, bool with_slots) {
   pdl_enter();
   int bid, nblk, gi;
   const GridView g = vs.get(bid, nblk, gi);
   if (vs.skip(g)) return;
-  __shared__ int wsum[8];
-  __shared__ int base_sh, count_sh;
-  __shared__ int nbr_sh[2];
-  __shared__ unsigned char lines[256];
   const int nn = min(g.counters[C_NNODES], g.node_cap);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int R = g.R;
   for (int b = bid; b < nn * 12; b += nblk) {
-    const int node = b / 12, axis = (b % 12) / 4, qrun = b % 4;
+    const int axis = (b % 12) / 4, qrun = b % 4;
     const int run = axis == 0 ? rx : (axis == 1 ? ry : rz);
     if (qrun >= 16 / run) continue;  // block-uniform
-    int q[3];
-    node_coords(g, (unsigned long long)g.node_key[node], q[0], q[1], q[2]);
-    const int32_t* ch = g.child + (size_t)node * kNodeBricks;
-    const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
-    const int r0 = qrun * run, nb = run + 2 * R;
-    if (threadIdx.x < 2) {
-      int qq[3] = {q[0], q[1], q[2]};
-      qq[axis] += threadIdx.x == 0 ? -1 : 1;
-      int n2 = -1;
-      if (qq[0] >= 0 && qq[1] >= 0 && qq[2] >= 0 && qq[0] < g.NX && qq[1] < g.NY && qq[2] < g.NZ)
-        n2 = find_node(g, node_key_at(g, qq[0], qq[1], qq[2]));
-      nbr_sh[threadIdx.x] = n2;
-    }
-    const int o1 = threadIdx.x & 15, o2 = threadIdx.x >> 4;
-    bool any = false;
-    {
-      // the run's child entries along the line, all read before any is tested
-      const int across = (o1 << (4 * a1)) | (o2 << (4 * a2));
-      int c[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) c[j] = j < run ? ch[across | ((r0 + j) << (4 * axis))] : -1;
-#pragma unroll
-      for (int j = 0; j < 16; ++j) any |= c[j] >= 0;
-    }
-    const unsigned bal = __ballot_sync(0xffffffffu, any);
-    if (lane == 0) wsum[warp] = __popc(bal);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int tot = 0;
-      for (int w = 0; w < 8; ++w) {
-        const int t = wsum[w];
-        wsum[w] = tot;
-        tot += t;
-      }
-      count_sh = tot;
-      base_sh = tot ? atomicAdd(&g.items_ctr[axis], tot) : 0;
-    }
-    __syncthreads();
-    const int base = base_sh, cnt = count_sh;
-    if (any) {
-      const int pos = wsum[warp] + __popc(bal & ((1u << lane) - 1u));
-      lines[pos] = (unsigned char)threadIdx.x;
-      const int p = base + pos;
-      if (p < g.item_cap) {
-        int l0[3];
-        l0[axis] = r0;
-        l0[a1] = o1;
-        l0[a2] = o2;
-        it.run[axis][p] = pack_brick(q[0] * 16 + l0[0], q[1] * 16 + l0[1], q[2] * 16 + l0[2]);
-        if (it.igrid[axis]) it.igrid[axis][p] = gi;
-      }
-    }
-    __syncthreads();
-    if (with_slots) {
-      // four slots per thread and round, their child reads issued before any is written
-      const int total = cnt * nb;
-      for (int idx0 = threadIdx.x; idx0 < total; idx0 += 4 * 256) {
-        int sv[4];
-        int64_t dst[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int idx = idx0 + u * 256;
-          sv[u] = -1;
-          dst[u] = -1;
-          if (idx < total) {
-            const int i = idx / nb, j = idx % nb;
-            const int p = base + i;
-            if (p < g.item_cap) {
-              const int line = lines[i];
-              int c = r0 + j - R, src = node;
-              if (c < 0) {
-                c += 16;
-                src = nbr_sh[0];
-              } else if (c >= 16) {
-                c -= 16;
-                src = nbr_sh[1];
-              }
-              dst[u] = (int64_t)p * kItemSlots + j;
-              // local brick: c along the axis, the line's two coordinates across it
-              const int lb = (c << (4 * axis)) | ((line & 15) << (4 * a1)) | ((line >> 4) << (4 * a2));
-              if (src >= 0) sv[u] = g.child[(size_t)src * kNodeBricks + lb];
-            }
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (dst[u] >= 0) it.slots[axis][dst[u]] = sv[u] >= 0 ? sv[u] + g.slot_base : -1;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Slots of each queued run's bricks with R bricks of halo on both sides along the axis: a warp per four
-// queued runs, a lane per slot.  A run lies inside one node and its halo (R <= 6 < 16 bricks) reaches at
-// most the neighbouring node on each side along the axis, so three node lookups (lanes 8 u .. 8 u + 2 for
-// run u) serve its slot list, read from the child tables.  Each run is a chain of three dependent reads
-// (run, hash slots, child entries); four at a time keep as many in flight per warp (71,000
-// runs: 17 us, one at a time 23).  view(item): the grid of a run.
-template <class View>
-__device__ __forceinline__ void item_slots(View view, int axis, int run, const unsigned long long* __restrict__ runs, int n,
-                                           int32_t* __restrict__ slots) {
-  const int lane = threadIdx.x & 31, u = lane >> 3, sub = lane & 7;
-  const int nw = (int)gridDim.x * (int)(blockDim.x >> 5);
-  for (int base = 4 * ((int)blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5)); base < n; base += 4 * nw) {
-    unsigned long long packed = 0ull;
-    int nq = -1;
-    if (base + u < n) {
-      packed = runs[base + u];
-      if (sub < 3) {
-        const GridView& g = view(base + u);
-        int bx, by, bz;
-        unpack_brick(packed, bx, by, bz);
-        const int qa = ((axis == 0 ? bx : (axis == 1 ? by : bz)) >> 4) + sub - 1;
-        const int NQa = axis == 0 ? g.NX : (axis == 1 ? g.NY : g.NZ);
-        if (qa >= 0 && qa < NQa)
-          nq = find_node(g, node_key_at(g, axis == 0 ? qa : bx >> 4, axis == 1 ? qa : by >> 4, axis == 2 ? qa : bz >> 4));
-      }
-    }
-    int s[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      s[v] = -1;
-      const unsigned long long pk = __shfl_sync(0xffffffffu, packed, 8 * v);
-      const int n_lo = __shfl_sync(0xffffffffu, nq, 8 * v), n_mid = __shfl_sync(0xffffffffu, nq, 8 * v + 1),
-                n_hi = __shfl_sync(0xffffffffu, nq, 8 * v + 2);
-      if (base + v < n) {  // warp-uniform
-        const GridView& g = view(base + v);
-        int bx, by, bz;
-        unpack_brick(pk, bx, by, bz);
-        const int ba = axis == 0 ? bx : (axis == 1 ? by : bz), Ba = axis == 0 ? g.BX : (axis == 1 ? g.BY : g.BZ);
-        const int ca = ba + lane - g.R;  // this slot's brick coordinate along the axis
-        if (lane < run + 2 * g.R && ca >= 0 && ca < Ba) {
-          const int node = (ca >> 4) < (ba >> 4) ? n_lo : ((ca >> 4) > (ba >> 4) ? n_hi : n_mid);
-          if (node >= 0) {
-            s[v] = g.child[(size_t)node * kNodeBricks +
-                           local_brick(axis == 0 ? ca : bx, axis == 1 ? ca : by, axis == 2 ? ca : bz)];
-            if (s[v] >= 0) s[v] += g.slot_base;
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < 4; ++v)
-      if (base + v < n) slots[(size_t)(base + v) * kItemSlots + lane] = s[v];
+    node_runs<false>(g, gi, b / 12, axis, qrun, run, it, with_slots);
   }
 }
 
@@ -1576,39 +1567,28 @@ __device__ __forceinline__ void init_new_fields(const GridView& g, int block, in
     init_fields_warp(g, slot, threadIdx.x & 31);
 }
 
-// blockIdx.y = axis; 3: the new bricks' fields
-__global__ void k_item_slots(GridView g, int rx, int ry, int rz, Items it) {
+// An update's work lists, from the dirty bits of its listed nodes (blockIdx.z 0), and beside them the fields of
+// the bricks that it stored (1).  The global form's lists come from k_items_nodes, and its passes write every
+// field.  A run is queued by one block, so no run is claimed and no slot list is built from a queue:
+// claiming each run with an exchange while marking and reading slot lists back from the queue took 20 + 17 us
+// of a lidar frame on average.
+template <class US>
+__global__ void __launch_bounds__(256) k_items_dirty(US us, int rx, int ry, int rz, Items it, bool with_slots) {
   pdl_enter();
-  if (g.counters[C_BIG]) return;  // the global form's work lists came with their slots, and write every field
-  const int axis = (int)blockIdx.y;
-  if (axis == 3) {
+  const UpdArgs A = us.get();
+  const GridView& g = A.g;
+  if (big_update(g)) return;
+  if (blockIdx.z == 1) {
     init_new_fields(g, (int)blockIdx.x, (int)gridDim.x);
     return;
   }
-  item_slots([&](int) -> const GridView& { return g; }, axis, axis == 0 ? rx : (axis == 1 ? ry : rz), it.run[axis],
-             min(g.items_ctr[axis], g.item_cap), it.slots[axis]);
-}
-
-// The envelope form's updates have no slot lists: the new bricks' fields alone.
-__global__ void k_init_new(GridView g) {
-  pdl_enter();
-  if (!g.counters[C_BIG]) init_new_fields(g, (int)blockIdx.x, (int)gridDim.x);
-}
-
-// The same for a batch of k grids' shared queue: each run's grid comes from it.igrid (runs of a grid whose
-// update took the global form are read again to the slots they came with).
-__global__ void k_item_slots_batch(const GridView* __restrict__ views, int k, const int32_t* __restrict__ items_ctr,
-                                   int item_cap, int rx, int ry, int rz, Items it) {
-  pdl_enter();
-  const int axis = (int)blockIdx.y;
-  if (axis == 3) {
-    const int i = (int)blockIdx.x % k;
-    if (!views[i].counters[C_BIG]) init_new_fields(views[i], (int)blockIdx.x / k, ((int)gridDim.x - 1 - i) / k + 1);
-    return;
+  const int nn = min(g.counters[C_DIRTY_NODES], g.node_cap);
+  for (int b = (int)blockIdx.x; b < nn * 12; b += (int)gridDim.x) {
+    const int axis = (b % 12) / 4, qrun = b % 4;
+    const int run = axis == 0 ? rx : (axis == 1 ? ry : rz);
+    if (qrun >= 16 / run) continue;  // block-uniform
+    node_runs<true>(g, (int)blockIdx.y, dirty_nodes(g)[b / 12], axis, qrun, run, it, with_slots);
   }
-  const int32_t* igrid = it.igrid[axis];
-  item_slots([&](int item) -> const GridView& { return views[igrid[item]]; }, axis, axis == 0 ? rx : (axis == 1 ? ry : rz),
-             it.run[axis], min(items_ctr[axis], item_cap), it.slots[axis]);
 }
 
 // Update statistics only (launched when they are asked for): the stored bricks each pass
@@ -1630,15 +1610,8 @@ __global__ void k_count_run_bricks(const GridView* __restrict__ views, GridView 
 }
 
 // ---- incremental ----
-// Voxel gap between two bricks d apart along an axis: the nearest voxels of bricks 0 and d are
-// 8 |d| - 7 apart (0 for the same brick).
-__device__ __forceinline__ int brick_gap(int d) {
-  d = abs(d);
-  return d == 0 ? 0 : 8 * d - 7;
-}
-
 // For every changed brick c: refresh its obstacle flag; if it holds obstacles, mark its dilation
-// (the bricks within R that must be stored); and queue its dirty runs.
+// (the bricks within R that must be stored); and mark its dirty runs.
 // Dirty sets: D(v) depends only on obstacles closer than dmax (Eq. 1 with the truncation), so a
 // flip in c can change D only in bricks whose nearest voxels lie closer than dmax to c's -- the
 // ball of radius dmax around c at brick granularity, about half the cube of R bricks.  Such a brick
@@ -1647,24 +1620,25 @@ __device__ __forceinline__ int brick_gap(int d) {
 // passes).  The in-plane values g2 change only in c's z layer, within dmax in the plane (a disk):
 // those bricks also need the in-plane pass; the x-line values g1 change only in c's x row: those
 // bricks also need the x pass.
+// Dirty runs are bits per node, OR-ed a row along x at a time (one unit of mark_dirty: for dmax 32 and runs
+// of 4, 32 to 41 per changed brick; no value comes back, nothing is waited for), and queued node by node
+// by k_items_dirty.  Runs are aligned to their length (4, 8 or 16) inside nodes, hence at multiples of it in
+// grid coordinates.
 // With at most two changed bricks per block, a block per changed brick: its first threads find
 // (or, for an obstacle-holding c, create) the interior nodes c's cube spans (at most 4 per axis:
 // 2R + 1 <= 47 bricks), then a thread per row (y, z) of the cube sets the row's x extent in the
-// allocation masks, and a thread per (column, z run) of the cube queues the run once if one of its
-// bricks is in the ball (and c's y run and x run in c's layer).  Runs are aligned to their length
-// (4, 8 or 16) inside nodes, hence at multiples of it in grid coordinates.  With more changed bricks
+// allocation masks, beside a thread per unit.  With more changed bricks
 // per block (a batch's share of the launch, a large update), a thread per (changed brick, row) and
-// then per (changed brick, offset in its cube), each with its own node lookups, keeps every thread
+// then per (changed brick, unit), each with its own node lookups, keeps every thread
 // of the GPU busy instead.
 template <class US>
-__global__ void __launch_bounds__(256, 6) k_changed_mark(US us, int rx, int ry, int rz, Items it, bool mark) {
+__global__ void __launch_bounds__(256, 6) k_changed_mark(US us, int rx, int ry, int rz) {
   pdl_enter();
   __shared__ int nodes[64];
   __shared__ int obst_sh;
   const UpdArgs A = us.get();
   const GridView& g = A.g;
   const int32_t* __restrict__ changed = A.changed;
-  const int grid = (int)blockIdx.y;
   const int nc = min(g.counters[C_CHANGED], g.cap);
   const int R = g.R, side = 2 * R + 1;
   // an update that takes the global form leaves all this to the gated kernels of the side stream
@@ -1672,7 +1646,7 @@ __global__ void __launch_bounds__(256, 6) k_changed_mark(US us, int rx, int ry, 
     if (blockIdx.x == 0 && threadIdx.x == 0) g.counters[C_BIG] = 1;
     return;
   }
-  const int epoch = g.counters[C_EPOCH];
+  const uint32_t epoch = (uint32_t)g.counters[C_EPOCH];
   if (nc > 2 * (int)gridDim.x) {
     // dilation: a thread per (changed brick, row), the rounds block-uniform
     const int rows = side * side, nseg = (side + 15) / 16 + 1;
@@ -1714,42 +1688,21 @@ __global__ void __launch_bounds__(256, 6) k_changed_mark(US us, int rx, int ry, 
         alloc_new_bits(g, node, word, added, x16, y, z);
       }
     }
-    if (!mark) return;
-    // dirty runs: a thread per (changed brick, offset in its cube); a warp spans at most two changed
-    // bricks (a cube has at least 27 offsets), whose obstacle bits its first and last lanes read
-    const int vol = side * side * side;
-    const int lane = threadIdx.x & 31;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < (int64_t)nc * vol;
-         base += (int64_t)gridDim.x * blockDim.x) {
-      const int64_t i = base + threadIdx.x;
-      const long long bi = i < (int64_t)nc * vol ? (long long)(i / vol) : -1ll;
-      const long long b0 = __shfl_sync(0xffffffffu, bi, 0), b31 = __shfl_sync(0xffffffffu, bi, 31);
-      bool o = false;
-      if (lane == 0 && b0 >= 0) o = brick_has_obstacle(g, changed[b0]);
-      if (lane == 31 && b31 >= 0) o = brick_has_obstacle(g, changed[b31]);
-      const bool o0 = __shfl_sync(0xffffffffu, o, 0), o31 = __shfl_sync(0xffffffffu, o, 31);
-      bool wx = false, wy = false, wz = false;
-      unsigned long long px = 0, py = 0, pz = 0;
-      if (bi >= 0) {
-        const int r = (int)(i % vol);
-        const int dx = r % side - R, dy = (r / side) % side - R, dz = r / (side * side) - R;
-        const int s = changed[bi];
-        const int4 c = g.bcoord[s];
-        const int bx = c.x + dx, by = c.y + dy, bz = c.z + dz;
-        const int gx = brick_gap(dx), gy = brick_gap(dy), gz = brick_gap(dz);
-        if ((unsigned)bx < (unsigned)g.BX && (unsigned)by < (unsigned)g.BY && (unsigned)bz < (unsigned)g.BZ &&
-            gx * gx + gy * gy + gz * gz < g.INF) {
-          const bool obst = bi == b0 ? o0 : o31;
-          const unsigned long long key = node_key_of(g, bx, by, bz);
-          const int node = obst ? get_or_create_node(g, key) : find_node(g, key);
-          if (node >= 0 && (obst || g.child[(size_t)node * kNodeBricks + local_brick(bx, by, bz)] >= 0)) {
-            if (dy == 0 && dz == 0) wx = claim_run(g, 0, bx, by, bz, node, rx, epoch, px);
-            if (dz == 0) wy = claim_run(g, 1, bx, by, bz, node, ry, epoch, py);
-            wz = claim_run(g, 2, bx, by, bz, node, rz, epoch, pz);
-          }
-        }
-      }
-      emit_runs3(g, {wx, wy, wz}, {px, py, pz}, it, grid);
+    // dirty runs: a thread per (changed brick, unit)
+    const int umax = side * (side / rz + 2) + side / ry + 3;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)nc * umax;
+         i += (int64_t)gridDim.x * blockDim.x) {
+      const int s = changed[i / umax], u = (int)(i % umax);
+      const int4 c = g.bcoord[s];
+      const DirtyCube k(g, c, ry, rz);
+      if (u >= k.units) continue;
+      const bool obst = brick_has_obstacle(g, s);
+      mark_dirty(g, c, k, u, rx, ry, rz, [&](int bx, int by, int bz) {
+        const unsigned long long key = node_key_of(g, bx, by, bz);
+        const int n = obst ? get_or_create_node(g, key) : find_node(g, key);
+        if (n >= 0) list_dirty_node(g, n, epoch);
+        return n;
+      });
     }
     return;
   }
@@ -1757,9 +1710,8 @@ __global__ void __launch_bounds__(256, 6) k_changed_mark(US us, int rx, int ry, 
     const int s = changed[i];
     __syncthreads();  // the table of the block's previous brick is no longer read
     const int4 c = g.bcoord[s];
-    const int x0 = max(c.x - R, 0), x1 = min(c.x + R, g.BX - 1);
-    const int y0 = max(c.y - R, 0), y1 = min(c.y + R, g.BY - 1);
-    const int z0 = max(c.z - R, 0), z1 = min(c.z + R, g.BZ - 1);
+    const DirtyCube k(g, c, ry, rz);
+    const int x0 = k.x0, x1 = k.x1, y0 = k.y0, y1 = k.y1, z0 = k.z0, z1 = k.z1;
     const int qx0 = x0 >> 4, qy0 = y0 >> 4, qz0 = z0 >> 4;
     const int nqx = (x1 >> 4) - qx0 + 1, nqy = (y1 >> 4) - qy0 + 1, nqz = (z1 >> 4) - qz0 + 1;
     const int nq = nqx * nqy * nqz;  // at most 4^3
@@ -1810,79 +1762,13 @@ __global__ void __launch_bounds__(256, 6) k_changed_mark(US us, int rx, int ry, 
         }
       }
     }
-    if (!mark) continue;  // block-uniform
-    // dirty runs: a thread per (column, z run) of the cube, block-uniform rounds (the lists' places
-    // are reserved a warp at a time); runs are 4, 8 or 16 bricks (shifts, not divisions)
-    const int r0 = z0 & ~(rz - 1), nruns = ((z1 - r0) >> (__ffs(rz) - 1)) + 1;
-    const int ncx = x1 - x0 + 1, ncol = ncx * (y1 - y0 + 1), total = ncol * nruns;
-    for (int u0 = 0; u0 < total; u0 += (int)blockDim.x) {
-      const int u = u0 + (int)threadIdx.x;
-      bool wx = false, wy = false, wz = false;
-      unsigned long long px = 0, py = 0, pz = 0;
-      if (u < total) {
-        const int zr = u / ncol, col = u - zr * ncol;
-        const int cy = col / ncx;
-        const int bx = x0 + (col - cy * ncx), by = y0 + cy;
-        const int zs = max(r0 + zr * rz, z0), ze = min(r0 + zr * rz + rz - 1, z1);
-        const int node = nodes[((bx >> 4) - qx0) + nqx * (((by >> 4) - qy0) + nqy * ((zs >> 4) - qz0))];
-        const int gx = brick_gap(bx - c.x), gy = brick_gap(by - c.y), in_plane = gx * gx + gy * gy;
-        if (node >= 0 && in_plane < g.INF) {
-          const int32_t* ch = g.child + (size_t)node * kNodeBricks;
-          bool any = false;
-          for (int bz = zs; bz <= ze; ++bz) {
-            const bool stored = obst || ch[local_brick(bx, by, bz)] >= 0;
-            const int gz = brick_gap(bz - c.z);
-            any |= stored && in_plane + gz * gz < g.INF;
-            if (bz == c.z && stored) {
-              if (by == c.y) wx = claim_run(g, 0, bx, by, bz, node, rx, epoch, px);
-              wy = claim_run(g, 1, bx, by, bz, node, ry, epoch, py);
-            }
-          }
-          if (any) wz = claim_run(g, 2, bx, by, zs, node, rz, epoch, pz);
-        }
-      }
-      emit_runs3(g, {wx, wy, wz}, {px, py, pz}, it, grid);
-    }
-  }
-}
-
-// Dirty runs of a batch's update, queued after the bricks the dilation added are stored (so that
-// the marking overlaps the batch's gated global-form branch instead of preceding it): a thread per
-// (changed brick, offset in its cube), the ball and disk rules of k_changed_mark, stored bricks
-// read from the child tables.
-template <class US>
-__global__ void __launch_bounds__(256) k_mark_runs(US us, int rx, int ry, int rz, Items it) {
-  pdl_enter();
-  const UpdArgs A = us.get();
-  const GridView& g = A.g;
-  const int32_t* __restrict__ changed = A.changed;
-  const int grid = (int)blockIdx.y;
-  if (g.counters[C_BIG]) return;
-  const int nc = min(g.counters[C_CHANGED], g.cap);
-  const int epoch = g.counters[C_EPOCH];
-  const int R = g.R, side = 2 * R + 1, vol = side * side * side;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < (int64_t)nc * vol;
-       base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    bool wx = false, wy = false, wz = false;
-    unsigned long long px = 0, py = 0, pz = 0;
-    if (i < (int64_t)nc * vol) {
-      const int r = (int)(i % vol);
-      const int dx = r % side - R, dy = (r / side) % side - R, dz = r / (side * side) - R;
-      const int4 c = g.bcoord[changed[i / vol]];
-      const int bx = c.x + dx, by = c.y + dy, bz = c.z + dz;
-      const int gx = brick_gap(dx), gy = brick_gap(dy), gz = brick_gap(dz);
-      if ((unsigned)bx < (unsigned)g.BX && (unsigned)by < (unsigned)g.BY && (unsigned)bz < (unsigned)g.BZ &&
-          gx * gx + gy * gy + gz * gz < g.INF) {
-        const int node = find_node(g, node_key_of(g, bx, by, bz));
-        if (node >= 0 && g.child[(size_t)node * kNodeBricks + local_brick(bx, by, bz)] >= 0) {
-          if (dy == 0 && dz == 0) wx = claim_run(g, 0, bx, by, bz, node, rx, epoch, px);
-          if (dz == 0) wy = claim_run(g, 1, bx, by, bz, node, ry, epoch, py);
-          wz = claim_run(g, 2, bx, by, bz, node, rz, epoch, pz);
-        }
-      }
-    }
-    emit_runs3(g, {wx, wy, wz}, {px, py, pz}, it, grid);
+    // dirty runs: the units on other warps than the first rows of the dilation, and the nodes into the list
+    if (threadIdx.x >= 192 && (int)threadIdx.x - 192 < nq && nodes[threadIdx.x - 192] >= 0)
+      list_dirty_node(g, nodes[threadIdx.x - 192], epoch);
+    for (int u = (int)((threadIdx.x + 160) & 255); u < k.units; u += 256)
+      mark_dirty(g, c, k, u, rx, ry, rz, [&](int bx, int by, int bz) {
+        return nodes[((bx >> 4) - qx0) + nqx * (((by >> 4) - qy0) + nqy * ((bz >> 4) - qz0))];
+      });
   }
 }
 
@@ -1940,9 +1826,8 @@ cudaError_t update_mark_kernels(US us, GV gv, int k, int node_cap, int R, bool w
     if (e != cudaSuccess) return e;
   }
   // incremental form, for the others: the changed bricks' flags, their dilation (with storage for
-  // the bricks it adds) and, for a single grid, their dirty runs; a batch's dirty runs after that
-  VDB_LAUNCH_PDL(k_changed_mark<US>, dim3(share(2432), k), kT, 0, st, us, t.run[0], t.run[1], t.run[2], it, k == 1);
-  if (k > 1) VDB_LAUNCH_PDL(k_mark_runs<US>, dim3(share(2432), k), kT, 0, st, us, t.run[0], t.run[1], t.run[2], it);
+  // the bricks it adds) and their dirty runs
+  VDB_LAUNCH_PDL(k_changed_mark<US>, dim3(share(2432), k), kT, 0, st, us, t.run[0], t.run[1], t.run[2]);
   return cudaGetLastError();
 }
 
@@ -2152,8 +2037,10 @@ cudaError_t launch_build_items_full(const GridView& g, const Tuning& t, const It
   return cudaGetLastError();
 }
 
-cudaError_t launch_item_slots(const GridView& g, const Tuning& t, const Items& it, cudaStream_t st) {
-  VDB_LAUNCH_PDL(k_item_slots, dim3(304, 4), kT, 0, st, g, t.run[0], t.run[1], t.run[2], it);
+cudaError_t launch_items_dirty(const GridView& g, const Tuning& t, const Items& it, bool with_slots, cudaStream_t st) {
+  UpdArgs a{};
+  a.g = g;
+  VDB_LAUNCH_PDL(k_items_dirty<UpdOne>, dim3(912, 1, 2), kT, 0, st, UpdOne{a}, t.run[0], t.run[1], t.run[2], it, with_slots);
   return cudaGetLastError();
 }
 
@@ -2164,15 +2051,11 @@ cudaError_t launch_count_run_bricks(const GridView* views, const GridView& one, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_init_new(const GridView& g, cudaStream_t st) {
-  VDB_LAUNCH_PDL(k_init_new, 304, kT, 0, st, g);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_item_slots_batch(const GridView* views, int k, const Tuning& t, const Items& it, int32_t* items_ctr,
-                                    int item_cap, cudaStream_t st) {
-  VDB_LAUNCH(k_item_slots_batch, dim3(1216, 4), kT, 0, st, views, k, items_ctr, item_cap, t.run[0], t.run[1], t.run[2],
-             it);
+cudaError_t launch_items_dirty_batch(const UpdArgs* d_args, int k, const Tuning& t, const Items& it, cudaStream_t st) {
+  if (k <= 0) return cudaSuccess;
+  const unsigned share = 912 / k > 16 ? 912 / k : 16;
+  VDB_LAUNCH_PDL(k_items_dirty<UpdBatch>, dim3(share, k, 2), kT, 0, st, UpdBatch{d_args}, t.run[0], t.run[1], t.run[2], it,
+                 true);
   return cudaGetLastError();
 }
 

@@ -63,7 +63,7 @@ enum Counter : int {
   C_OBST = 12,
   C_NB_START = 13,  // stored bricks when the running update began (its global-vs-incremental choice)
   C_EPOCH = 14,  // incremental update epoch (run and brick dedupe marks)
-  C_SPARE = 15,  // unused
+  C_DIRTY_NODES = 15,  // nodes listed with dirty runs in the running update
   C_XB = 16,  // stored bricks in the update's dirty runs per axis (x, y, z: three consecutive words)
   C_YB = 17,
   C_ZB = 18,
@@ -76,6 +76,8 @@ constexpr uint32_t F_OBST = 1u;    // holds an occupied voxel
 constexpr uint32_t F_FINITE = 2u;  // holds a voxel with D < dmax^2
 constexpr uint32_t F_G2FIN = 4u;   // holds a voxel with in-plane value g2 < dmax^2
 constexpr uint32_t F_G1FIN = 8u;   // holds a voxel with x-line value g1 < dmax^2
+
+constexpr int kMarkWords = 128;  // per node: 3 axes x 32 words of dirty-run bits, the list epoch, padding
 
 struct GridView {
   int nx, ny, nz;     // voxels
@@ -97,7 +99,7 @@ struct GridView {
                       // same layout
   uint32_t* nclaim;   // [node_cap * 128] bricks claimed for allocation by the running ingest (amask layout)
   long long* node_key;  // [node_cap]
-  int32_t* mark;      // [node_cap * 3 * 1024] epoch of the last time each run along axis a was queued
+  uint32_t* mark;     // [node_cap * kMarkWords] an update's dirty runs, then the [node_cap] nodes that hold any
   unsigned long long* occ;  // [cap * 8]
   uint16_t* g1;       // [cap * 512]
   uint16_t* g2;       // [cap * 512]
@@ -427,9 +429,8 @@ cudaError_t launch_update_batch_ingest(const UpdArgs* d_args, const BatchUpdShap
                                        cudaStream_t st);
 cudaError_t launch_update_batch_mark(const UpdArgs* d_args, const BatchUpdShape& s, const Tuning& t, const Items& it,
                                      const Fork& fk, cudaStream_t st);
-// slot lists of every queued run of a batch of k grids (each run's grid from it.igrid)
-cudaError_t launch_item_slots_batch(const GridView* views, int k, const Tuning& t, const Items& it, int32_t* items_ctr,
-                                    int item_cap, cudaStream_t st);
+// work lists of the dirty runs of k grids (d_args: their arguments in device memory)
+cudaError_t launch_items_dirty_batch(const UpdArgs* d_args, int k, const Tuning& t, const Items& it, cudaStream_t st);
 // Update statistics: stored bricks of every run's slot list per axis into each grid's C_XB .. C_ZB
 // (views == nullptr: a single grid `one`).
 cudaError_t launch_count_run_bricks(const GridView* views, const GridView& one, const int32_t* items_ctr, int item_cap,
@@ -445,10 +446,8 @@ cudaError_t launch_ut_pass(const GridView& g, int axis, void* scratch, cudaStrea
 // voxel; y, z: lines whose input changed), marking the next axis's lines where its output changed;
 // lines recomputed are counted in items_ctr[axis].  The z pass also refreshes the brick flags.
 cudaError_t launch_ut_update_pass(const GridView& g, int axis, void* scratch, cudaStream_t st);
-// fields of the bricks that the running update stored (the slot-list kernels below do it too)
-cudaError_t launch_init_new(const GridView& g, cudaStream_t st);
-// slot lists of every queued run (windowed form)
-cudaError_t launch_item_slots(const GridView& g, const Tuning& t, const Items& it, cudaStream_t st);
+// an update's work lists from its dirty runs (with slot lists: windowed form), and its new bricks' fields
+cudaError_t launch_items_dirty(const GridView& g, const Tuning& t, const Items& it, bool with_slots, cudaStream_t st);
 
 // The same steps for every grid of a batch at once: one launch per step (views: device array of
 // the k grids' views; each block finds its grid through the shape's block shares).
