@@ -1434,18 +1434,21 @@ __device__ __forceinline__ void mark_dirty(const GridView& g, const int4& c, con
 
 // The runs of a node along one axis: queued where they hold a stored brick (DIRTY: and their dirty bit is set,
 // which is cleared here).  The block's 256 threads cover the 16 x 16 lines of the node across the axis, qrun is
-// the run along it.  A block-wide scan compacts the runs and one atomic reserves their places; the run slot
-// lists are then read straight from the child tables of the node and of its neighbour along the axis
-// (R <= 6 < 16, so the halo reaches at most one node each way), one slot per thread.
-template <bool DIRTY>
-__device__ __forceinline__ void node_runs(const GridView& g, int gi, int node, int axis, int qrun, int run, const Items& it,
-                                          bool with_slots) {
+// the run along it.  A thread reads its line's child entries, the run's and (NBQ > 0: 4 NBQ >= run + 2 R
+// slots) its halo's of R bricks on both sides, which reach at most the neighbouring node each way
+// (R <= 6 < 16); a block-wide scan compacts the runs, one atomic reserves their places, and each thread
+// stores its slot list as vectors.  Bound by the chain of dependent reads: those of the node itself are
+// issued before the neighbours are known and counted, the neighbours' while the places are reserved
+// (19 us for the 300,000 runs of a 1024 x 1024 x 256 tunnel scene, 21 with a line along x read entry by entry; with
+// the slots read again from the compacted queue, one per thread, that scene's call took 7 us more, a batch of
+// 16 maps with its update 26 us more).
+template <bool DIRTY, int NBQ>
+__device__ __forceinline__ void node_runs(const GridView& g, int gi, int node, int axis, int qrun, int run, const Items& it) {
   __shared__ int wsum[8];
-  __shared__ int base_sh, count_sh;
+  __shared__ int base_sh;
   __shared__ int nbr_sh[2];
-  __shared__ unsigned char lines[256];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int R = g.R;
+  const int R = NBQ ? g.R : 0;
   bool dirty = true;
   if (DIRTY) {
     uint32_t* w = dirty_words(g, node, axis, qrun) + warp;
@@ -1456,28 +1459,43 @@ __device__ __forceinline__ void node_runs(const GridView& g, int gi, int node, i
   }
   int q[3];
   node_coords(g, (unsigned long long)g.node_key[node], q[0], q[1], q[2]);
-  const int32_t* ch = g.child + (size_t)node * kNodeBricks;
   const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
   const int r0 = qrun * run, nb = run + 2 * R;
-  if (threadIdx.x < 2) {
+  const int o1 = threadIdx.x & 15, o2 = threadIdx.x >> 4;
+  const int across = (o1 << (4 * a1)) | (o2 << (4 * a2));
+  // child entries along the line, c[j + sh] the one of brick r0 - R + j; first those of this node.  A line along
+  // x is contiguous: read as vectors, from the last multiple of 4 bricks on (which no node boundary splits).
+  constexpr int N = NBQ ? 4 * NBQ : 16;
+  const int sh = NBQ && axis == 0 ? (r0 - R) & 3 : 0, x0 = r0 - R - sh;
+  int c[N + 4];
+#pragma unroll
+  for (int j = 0; j < N + 4; ++j) c[j] = -1;
+  auto quad = [&](int j, int n) {
+    const int4 v = *reinterpret_cast<const int4*>(g.child + (size_t)n * kNodeBricks + (across | ((x0 + j) & 15)));
+    c[j] = v.x, c[j + 1] = v.y, c[j + 2] = v.z, c[j + 3] = v.w;
+  };
+  if (NBQ && axis == 0) {
+#pragma unroll
+    for (int j = 0; j < N + 4; j += 4)
+      if (dirty && j < nb + sh && (unsigned)(x0 + j) < 16u) quad(j, node);
+  } else {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int x = r0 + j - R;
+      if (dirty && j < nb && (unsigned)x < 16u) c[j] = g.child[(size_t)node * kNodeBricks + (across | (x << (4 * axis)))];
+    }
+  }
+  if (NBQ && threadIdx.x >= 254) {
     int qq[3] = {q[0], q[1], q[2]};
-    qq[axis] += threadIdx.x == 0 ? -1 : 1;
+    qq[axis] += threadIdx.x == 254 ? -1 : 1;
     int n2 = -1;
     if (qq[0] >= 0 && qq[1] >= 0 && qq[2] >= 0 && qq[0] < g.NX && qq[1] < g.NY && qq[2] < g.NZ)
       n2 = find_node(g, node_key_at(g, qq[0], qq[1], qq[2]));
-    nbr_sh[threadIdx.x] = n2;
+    nbr_sh[threadIdx.x - 254] = n2;
   }
-  const int o1 = threadIdx.x & 15, o2 = threadIdx.x >> 4;
   bool any = false;
-  if (!DIRTY || dirty) {
-    // the run's child entries along the line, all read before any is tested
-    const int across = (o1 << (4 * a1)) | (o2 << (4 * a2));
-    int c[16];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) c[j] = j < run ? ch[across | ((r0 + j) << (4 * axis))] : -1;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) any |= c[j] >= 0;
-  }
+  for (int j = 0; j < N + 4; ++j) any |= j >= R + sh && j < R + sh + run && c[j] >= 0;
   const unsigned bal = __ballot_sync(0xffffffffu, any);
   if (lane == 0) wsum[warp] = __popc(bal);
   __syncthreads();
@@ -1488,62 +1506,56 @@ __device__ __forceinline__ void node_runs(const GridView& g, int gi, int node, i
       wsum[w] = tot;
       tot += t;
     }
-    count_sh = tot;
     base_sh = tot ? atomicAdd(&g.items_ctr[axis], tot) : 0;
   }
-  __syncthreads();
-  const int base = base_sh, cnt = count_sh;
-  if (any) {
-    const int pos = wsum[warp] + __popc(bal & ((1u << lane) - 1u));
-    lines[pos] = (unsigned char)threadIdx.x;
-    const int p = base + pos;
-    if (p < g.item_cap) {
-      int l0[3];
-      l0[axis] = r0;
-      l0[a1] = o1;
-      l0[a2] = o2;
-      it.run[axis][p] = pack_brick(q[0] * 16 + l0[0], q[1] * 16 + l0[1], q[2] * 16 + l0[2]);
-      if (it.igrid[axis]) it.igrid[axis][p] = gi;
-    }
-  }
-  __syncthreads();
-  if (with_slots) {
-    // four slots per thread and round, their child reads issued before any is written
-    const int total = cnt * nb;
-    for (int idx0 = threadIdx.x; idx0 < total; idx0 += 4 * 256) {
-      int sv[4];
-      int64_t dst[4];
+  if (NBQ && any && axis == 0) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int idx = idx0 + u * 256;
-        sv[u] = -1;
-        dst[u] = -1;
-        if (idx < total) {
-          const int i = idx / nb, j = idx % nb;
-          const int p = base + i;
-          if (p < g.item_cap) {
-            const int line = lines[i];
-            int c = r0 + j - R, src = node;
-            if (c < 0) {
-              c += 16;
-              src = nbr_sh[0];
-            } else if (c >= 16) {
-              c -= 16;
-              src = nbr_sh[1];
-            }
-            dst[u] = (int64_t)p * kItemSlots + j;
-            // local brick: c along the axis, the line's two coordinates across it
-            const int lb = (c << (4 * axis)) | ((line & 15) << (4 * a1)) | ((line >> 4) << (4 * a2));
-            if (src >= 0) sv[u] = g.child[(size_t)src * kNodeBricks + lb];
-          }
-        }
+    for (int j = 0; j < N + 4; j += 4) {
+      const int x = x0 + j;
+      if (j < nb + sh && (unsigned)x >= 16u) {
+        const int src = nbr_sh[x < 0 ? 0 : 1];
+        if (src >= 0) quad(j, src);
       }
+    }
+  } else if (NBQ && any) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (dst[u] >= 0) it.slots[axis][dst[u]] = sv[u] >= 0 ? sv[u] + g.slot_base : -1;
+    for (int j = 0; j < N; ++j) {
+      const int x = r0 + j - R;
+      if (j < nb && (unsigned)x >= 16u) {
+        const int src = nbr_sh[x < 0 ? 0 : 1];
+        if (src >= 0) c[j] = g.child[(size_t)src * kNodeBricks + (across | ((x & 15) << (4 * axis)))];
+      }
     }
   }
   __syncthreads();
+  const int p = base_sh + wsum[warp] + __popc(bal & ((1u << lane) - 1u));
+  if (any && p < g.item_cap) {
+    int l0[3];
+    l0[axis] = r0;
+    l0[a1] = o1;
+    l0[a2] = o2;
+    it.run[axis][p] = pack_brick(q[0] * 16 + l0[0], q[1] * 16 + l0[1], q[2] * 16 + l0[2]);
+    if (it.igrid[axis]) it.igrid[axis][p] = gi;
+    int4* slots = reinterpret_cast<int4*>(it.slots[axis] + (size_t)p * kItemSlots);
+    auto pool = [&](int j) {
+      const int s = sh & 2 ? (sh & 1 ? c[j + 3] : c[j + 2]) : (sh & 1 ? c[j + 1] : c[j]);
+      return s >= 0 ? s + g.slot_base : -1;
+    };
+#pragma unroll
+    for (int v = 0; v < NBQ; ++v) slots[v] = make_int4(pool(4 * v), pool(4 * v + 1), pool(4 * v + 2), pool(4 * v + 3));
+  }
+  __syncthreads();  // wsum, base_sh and nbr_sh are free again
+}
+
+// The form of node_runs for runs of this length (without slot lists: the envelope form, any R).
+template <bool DIRTY>
+__device__ __forceinline__ void node_runs_of(const GridView& g, int gi, int node, int axis, int qrun, int run, const Items& it,
+                                             bool with_slots) {
+  const int nb = run + 2 * g.R;
+  if (!with_slots) node_runs<DIRTY, 0>(g, gi, node, axis, qrun, run, it);
+  else if (nb <= 12) node_runs<DIRTY, 3>(g, gi, node, axis, qrun, run, it);
+  else if (nb <= 16) node_runs<DIRTY, 4>(g, gi, node, axis, qrun, run, it);
+  else node_runs<DIRTY, 7>(g, gi, node, axis, qrun, run, it);
 }
 
 // Global form: every run that holds a stored brick, found node by node.  Block = (node, axis, run
@@ -1559,7 +1571,7 @@ __global__ void __launch_bounds__(256) k_items_nodes(VS vs, int rx, int ry, int 
     const int axis = (b % 12) / 4, qrun = b % 4;
     const int run = axis == 0 ? rx : (axis == 1 ? ry : rz);
     if (qrun >= 16 / run) continue;  // block-uniform
-    node_runs<false>(g, gi, b / 12, axis, qrun, run, it, with_slots);
+    node_runs_of<false>(g, gi, b / 12, axis, qrun, run, it, with_slots);
   }
 }
 
@@ -1593,7 +1605,7 @@ __global__ void __launch_bounds__(256) k_items_dirty(US us, int rx, int ry, int 
     const int axis = (b % 12) / 4, qrun = b % 4;
     const int run = axis == 0 ? rx : (axis == 1 ? ry : rz);
     if (qrun >= 16 / run) continue;  // block-uniform
-    node_runs<true>(g, (int)blockIdx.y, dirty_nodes(g)[b / 12], axis, qrun, run, it, with_slots);
+    node_runs_of<true>(g, (int)blockIdx.y, dirty_nodes(g)[b / 12], axis, qrun, run, it, with_slots);
   }
 }
 
