@@ -209,9 +209,9 @@ void mark(vdbedt_map* h, int i) {
   if (h->profiling && !capturing(h)) cudaEventRecord(h->ev[i], h->st);
 }
 
-Tuning effective_tuning(const vdbedt_map* h) {
+Tuning effective_tuning(const vdbedt_map* h, bool whole) {
   Tuning t = h->tune;
-  for (int a = 0; a < 3; ++a) t.run[a] = effective_run(h->g, h->tune, a);
+  for (int a = 0; a < 3; ++a) t.run[a] = effective_run(h->g, h->tune, a, whole);
   return t;
 }
 
@@ -236,7 +236,7 @@ void clear_stage(vdbedt_map* h) {
 }
 
 vdbedt_status do_global(vdbedt_map* h) {
-  const Tuning t = effective_tuning(h);
+  const Tuning t = effective_tuning(h, true);
   mark(h, 0);
   if (h->stage_n > 0) {
     CK(h, cudaMemsetAsync(h->g.counters + C_UNIQUE, 0, 2 * sizeof(int32_t), h->st), "memset");  // and C_HAS_ZERO
@@ -720,7 +720,7 @@ vdbedt_status vdbedt_update(vdbedt_handle h, vdbedt_update_stats* stats) {
     mark(h, 6);
     h->ev_recorded = h->profiling && !capturing(h);
   } else {
-    const Tuning t = effective_tuning(h);
+    const Tuning t = effective_tuning(h, false);
     mark(h, 0);
     CK(h, launch_begin_update(h->g, h->st), "begin update");
     if (h->stage_n > 0) {
@@ -1119,7 +1119,7 @@ vdbedt_status batch_global(vdbedt_batch* b) {
     return VDBEDT_OK;
   }
   Tuning t = b->tune;
-  for (int a = 0; a < 3; ++a) t.run[a] = effective_run(g0, b->tune, a);
+  for (int a = 0; a < 3; ++a) t.run[a] = effective_run(g0, b->tune, a, true);
   bmark(b, 0);
   // staged records: applied grid by grid (the sort-based ingest keeps per-grid scratch)
   for (vdbedt_map* m : b->maps) {
@@ -1177,7 +1177,7 @@ vdbedt_status batch_update(vdbedt_batch* b, vdbedt_update_stats* stats) {
     }
   } else {
     Tuning t = b->tune;
-    for (int a = 0; a < 3; ++a) t.run[a] = effective_run(g0, b->tune, a);
+    for (int a = 0; a < 3; ++a) t.run[a] = effective_run(g0, b->tune, a, false);
     // The grids' arguments in device memory stay fixed while staging does not reallocate (every
     // grid reads its record count from its device count word), so a captured update replays with
     // the same arguments; they are uploaded again only when they change, outside a capture.

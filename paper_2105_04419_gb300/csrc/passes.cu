@@ -790,7 +790,6 @@ cudaError_t launch_wait_selftest(const GridView& g, int which, cudaStream_t st) 
 
 bool windowed_form(const GridView& g) { return g.windowed != 0; }
 
-int effective_run(const GridView& g, const Tuning& t, int axis) { return windowed_form(g) ? t.run[axis] : kEnvRun; }
 
 // The windowed kernels address bricks by pool slot (the slot lists hold local slot + slot_base):
 // their view has the per-brick pointers moved back to the first slot of the pool.
@@ -814,6 +813,16 @@ GridView pool_view(const GridView& g) {
 // previous pass's leave one by one, and y and z together took 0.82 ms where they take 0.65 (1024 x 1024 x 256
 // tunnel scene, dmax 32).
 constexpr int kChainBricks = 16384;
+
+// Runs of 8 bricks share their halo over twice as many outputs as runs of 4 and halve the work lists: for whole
+// transforms that fill the GPU, with halos of three bricks or more (1024 x 1024 x 256 tunnel scene: dmax 32
+// lists 22 us, x 115, y 313, z 336 with 4, 16, 107, 305, 317 with 8; dmax 24 249 and 278, 248 and 266; at dmax
+// 8 y takes 121 and 131).  Updates keep 4: their dirty runs are short.
+int effective_run(const GridView& g, const Tuning& t, int axis, bool whole) {
+  if (!windowed_form(g)) return kEnvRun;
+  if (t.run[axis]) return t.run[axis];
+  return whole && g.item_cap > kChainBricks && g.R >= 3 ? 8 : 4;
+}
 
 cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, bool chained, cudaStream_t st) {
   chained = chained && g.item_cap <= kChainBricks;

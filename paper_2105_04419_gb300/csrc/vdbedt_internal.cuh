@@ -323,7 +323,7 @@ constexpr int kVariantXDirect = 4;
 constexpr int kBigUpdate = 24;
 constexpr int kVariantEnvelope = 8;
 struct Tuning {
-  int run[3] = {4, 4, 4};  // bricks per work item along x, y, z
+  int run[3] = {0, 0, 0};  // bricks per work item along x, y, z (0: by the grid's size and radius)
   int variant = 3;
 };
 
@@ -480,7 +480,8 @@ bool windowed_form(const GridView& g);
 // pass along `axis` (0 x, 1 y, 2 z) over the queued runs; chained: it follows a kernel of the stream
 // directly, and its launch overlaps that kernel's tail
 cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, bool chained, cudaStream_t st);
-int effective_run(const GridView& g, const Tuning& t, int axis);
+// bricks per run along `axis` (whole: a whole transform, not an update)
+int effective_run(const GridView& g, const Tuning& t, int axis, bool whole);
 // a bounded device wait that runs out (0: mbarrier phase, 1: pending node), for tests
 cudaError_t launch_wait_selftest(const GridView& g, int which, cudaStream_t st);
 

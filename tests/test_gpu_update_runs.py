@@ -126,3 +126,20 @@ def test_dirty_runs_of_a_batch():
             f.set_occupancy_dense(occ[i])
             f.global_()
             assert torch.equal(b.maps[i].export_dense(on_device=True), f.export_dense(on_device=True))
+
+
+@pytest.mark.parametrize("dmax", [17, 24, 32, 45])
+def test_whole_transform_runs(dmax):
+    """A map large enough for the longer runs, ragged on every axis, against runs of 4 and of 16."""
+    import paper_2105_04419_gb300 as V
+    nz, ny, nx = 205, 333, 421
+    g = torch.Generator(device="cuda").manual_seed(dmax)
+    occ = (torch.rand((nz, ny, nx), device="cuda", generator=g) < 1e-5).to(torch.uint8)
+    fields = []
+    for run in (0, 4, 16):
+        m = V.Map(nx, ny, nz, dmax)
+        m.set_tuning(x_run=run, y_run=run, z_run=run)
+        m.set_occupancy_dense(occ)
+        m.global_()
+        fields.append(m.export_dense(on_device=True))
+    assert torch.equal(fields[0], fields[1]) and torch.equal(fields[0], fields[2])
