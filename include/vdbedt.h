@@ -262,7 +262,7 @@ vdbedt_status vdbedt_clearance_backward(vdbedt_handle h, const float* pts, int64
 
 /* Tuning of the transform passes (0 = automatic for any field).
  *   x_run, y_run, z_run: bricks per work item of the pass along that axis (4, 8 or 16; 0: 8 for
- *            whole transforms of large grids with dmax above 16, 4 otherwise);
+ *            whole transforms of large grids with dmax above 17, 4 otherwise);
  *   variant: 0 automatic, 1 full windowed minimum, 3 windowed minimum with early exit and skips
  *            (the default; both exact); adding 4 (5 or 7) runs the x pass with plain loads instead
  *            of the bulk-copy ring; 8 the lower-envelope form of all three passes (exact, O(1)
