@@ -243,8 +243,9 @@ __device__ __forceinline__ void corners(const GridView& g, float vs, int i0, int
     const int a = q & 1, b = (q >> 1) & 1, e = q >> 2;
     D[q] = s >= 0 ? g.dist[(size_t)s * kBrickVox + ((i0 + a) & 7) + 8 * ((j0 + b) & 7) + 64 * ((k0 + e) & 7)] : g.INF;
   }
+  // rounded by themselves: a difference of equal corners stays zero, which a product fused into it would not
 #pragma unroll
-  for (int q = 0; q < 8; ++q) c.d[q] = vs * sqrtf((float)D[q]);
+  for (int q = 0; q < 8; ++q) c.d[q] = __fmul_rn(vs, sqrtf((float)D[q]));
 }
 
 __device__ __forceinline__ float trilinear(const Corner8& c, float tx, float ty, float tz) {
