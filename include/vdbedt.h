@@ -76,9 +76,9 @@ typedef enum {
  * every voxel while the grid holds no obstacle (and for queries outside the grid).  dmax must be 0.
  * A bounded grid only, with (nx-1)^2 + (ny-1)^2 + (nz-1)^2 < 2^31 - 1 so that every distance fits
  * int32, and every brick stored from creation (max_bricks and max_nodes 0 or at least the grid's):
- * about 6.2 KB per 8^3 brick (32-bit intermediates) plus 8 bytes per voxel of line scratch (nx
- * rounded up to 32) and three sets of dirty lines, all allocated at creation.  The transform
- * runs whole lines of the grid (x: nearest occupied voxel of the row; y, z: lower envelope of the
+ * about 6.2 KB per 8^3 brick (32-bit intermediates) plus three sets of dirty lines and, where ny or nz is
+ * above 1,496, 8 bytes per voxel of line scratch (nx rounded up to 32), all allocated at creation.  The transform
+ * runs whole lines of the grid (x: nearest occupied voxel of the row; y, z: minimum of the
  * parabolas rooted at the line's values).  vdbedt_update applies the staged records and recomputes
  * only the lines they reach, exactly: the x rows holding a flipped voxel, then the y lines on which
  * g1 changed, then the z lines on which g2 changed (each pass's output on a line depends only on
@@ -130,7 +130,7 @@ typedef struct {
 /* Create a handle for an nx x ny x nz grid with no obstacles (every D = dmax^2; VDBEDT_D_NONE when
  * untruncated).
  * Allocates the grid's storage for cfg->max_bricks bricks (about 4.1 KB each) and cfg->max_nodes
- * interior nodes (about 30 KB each) up front; the record stage and the ingest scratch grow on
+ * interior nodes (about 19 KB each) up front; the record stage and the ingest scratch grow on
  * demand (vdbedt_set_occupancy_counted reserves them ahead).  With both capacities set, the memory
  * follows the mapped part of the grid, not its size: a grid may span up to 2^32 bricks (e.g.
  * 16384 x 16384 x 8184 voxels) with obstacles in a small part of it.  Record-driven ingest and
@@ -216,9 +216,8 @@ vdbedt_status vdbedt_update(vdbedt_handle h, vdbedt_update_stats* stats);
 vdbedt_status vdbedt_query(vdbedt_handle h, const int32_t* xyz, int64_t n, int32_t* out_sqdist, int on_device);
 
 /* Nearest obstacle of n voxels: out_xyz[3k .. 3k + 2] is the occupied voxel o that D(v) measures
- * to -- the obstacle the paper's map keeps beside each cell's distance (Sec. IV-B) -- found among
- * the lattice points with |o - v|^2 = D(v) in increasing (z, y, x) order, so ties go to the
- * smallest (z, y, x).  (-1, -1, -1) for voxels outside the grid or with D = dmax^2 (no obstacle
+ * to -- the obstacle the paper's map keeps beside each cell's distance (Sec. IV-B) -- the one with the
+ * smallest (z, y, x) among those with |o - v|^2 = D(v).  (-1, -1, -1) for voxels outside the grid or with D = dmax^2 (no obstacle
  * closer than dmax).  Reads the current field (after vdbedt_global / vdbedt_update).  on_device
  * as for vdbedt_query.  EINVAL on an untruncated grid. */
 vdbedt_status vdbedt_query_nearest(vdbedt_handle h, const int32_t* xyz, int64_t n, int32_t* out_xyz, int on_device);
@@ -265,8 +264,8 @@ vdbedt_status vdbedt_clearance_backward(vdbedt_handle h, const float* pts, int64
  *            whole transforms of large grids with dmax above 17, 4 otherwise);
  *   variant: 0 automatic, 1 full windowed minimum, 3 windowed minimum with early exit and skips
  *            (the default; both exact); adding 4 (5 or 7) runs the x pass with plain loads instead
- *            of the bulk-copy ring; 8 the lower-envelope form of all three passes (exact, O(1)
- *            amortised work per voxel whatever the window, runs of 16 bricks: the separable
+ *            of the bulk-copy ring; 8 the envelope form of all three passes (exact, work that
+ *            follows the distances instead of the window, runs of 16 bricks: the separable
  *            transform of Eq. 1 line by line).  Grids with dmax above 45 always take the envelope
  *            form.  Switching between the windowed and envelope forms changes how intermediate
  *            fields are stored, so the next vdbedt_update recomputes the whole field (as
