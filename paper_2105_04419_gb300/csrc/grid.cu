@@ -1920,7 +1920,7 @@ cudaError_t reserve_ingest(const GridView& g, int64_t n, Scratch& scr, Scratch& 
 cudaError_t launch_begin_update(const GridView& g, cudaStream_t st) {
   UpdArgs a{};
   a.g = g;
-  VDB_LAUNCH(k_begin_update<UpdOne>, 1, 32, 0, st, UpdOne{a});
+  VDB_LAUNCH_PDL(k_begin_update<UpdOne>, 1, 32, 0, st, UpdOne{a});
   return cudaGetLastError();
 }
 
@@ -2174,7 +2174,7 @@ cudaError_t launch_incremental_mark(const GridView& g, const Tuning& t, const in
 cudaError_t launch_update_batch_ingest(const UpdArgs* d_args, const BatchUpdShape& s, const BatchCounts& counts,
                                        cudaStream_t st) {
   if (s.k <= 0) return cudaSuccess;
-  VDB_LAUNCH(k_begin_batch_update, dim3(1, s.k), 32, 0, st, d_args, counts);
+  VDB_LAUNCH_PDL(k_begin_batch_update, dim3(1, s.k), 32, 0, st, d_args, counts);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return update_ingest_kernels(UpdBatch{d_args}, s.k, s.max_n, st);
