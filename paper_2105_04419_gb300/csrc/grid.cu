@@ -1,15 +1,16 @@
 // Building and maintaining the sparse brick grid on the device.
 //
 //   ingest (global form)  staged occupancy records -> brick keys of "set" records -> unique list
-//            (one flag per brick of the grid, compacted with one atomic per warp, when records are
-//            many; an LSD radix sort + unique + compaction when they are few) -> nodes created first
+//            (one flag per brick of the grid, compacted with one atomic per block, when records are
+//            many or the grid mostly has storage; an LSD radix sort + unique + compaction for few
+//            records on large sparse grids) -> nodes created first
 //            (one thread per flagged node key) -> bricks allocated (slots reserved with one
 //            atomic per block) -> occupancy bits set (OR-ed into a dense mask during the count, or
 //            per record).  Several records for one voxel: the last one wins -- a per-voxel
 //            last-record table (atomicMax of the record index) picks it whenever a record clears a
 //            voxel.
-//   ingest (incremental form)  only the bricks of "set" records that are not stored yet are
-//            appended to a list and allocated; every voxel's last record is applied through the
+//   ingest (incremental form)  the bricks of "set" records that are not stored yet are claimed
+//            and allocated by one record each; every voxel's last record is applied through the
 //            last-record table and each flip's brick joins the changed list once.
 //   dense ingest  a whole occupancy grid -> per-brick masks in a scratch (sector-complete loads),
 //            then nodes, then the occupied bricks.
@@ -19,7 +20,8 @@
 //            dilation computed from its 3 x 3 x 3 node neighbourhood, absent bricks allocated.
 //   items    work lists for the passes: runs of bricks along x, y and z with their slot lists.
 //   incremental marking  bricks whose occupancy changed -> their dilation (allocated) -> dirty
-//            runs: x within R along x, in-plane within R in x and y, z within R in x, y and z.
+//            runs as bits per node: x within dmax along x, in-plane within dmax, z within dmax in space ->
+//            work lists from the bits.
 //   batches  the per-grid kernels take a view source: one grid, or every grid of a batch with
 //            block shares of one launch.
 #include "vdbedt_internal.cuh"

@@ -153,7 +153,7 @@ __device__ __forceinline__ int line_match(const GridView& g, int x, int y, int z
 // g1(x, oy, oz) = g2 - (oy - y)^2, and g1 is the squared distance to the obstacle along x; the first
 // match on each line is the smallest oz, then oy.  2 sqrt(D) + 1 reads a line instead of the
 // O(D) rows of the lattice sphere |o - v|^2 = D.  Bound by the random sector reads (about 30 per
-// query at dmax 32): 2^20 voxels of a 512 x 512 x 256 tunnel scene 0.24 ms = 4.4e9 queries/s (walking
+// query at dmax 32): 2^20 voxels of a 512 x 512 x 256 tunnel scene 0.18 ms = 5.8e9 queries/s (walking
 // the sphere in (z, y, x) order and testing occupancy bits: 3.7 ms).
 __global__ void __launch_bounds__(128) k_query_nearest(GridView g, const int32_t* __restrict__ xyz, int64_t n,
                                                        int32_t* __restrict__ out) {
