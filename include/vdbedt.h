@@ -212,7 +212,8 @@ vdbedt_status vdbedt_update(vdbedt_handle h, vdbedt_update_stats* stats);
 
 /* D at n voxel coordinates; coordinates outside the grid or in unstored bricks give dmax^2
  * (VDBEDT_D_NONE when untruncated).
- * on_device != 0: xyz and out_sqdist are device pointers; otherwise host pointers (the call waits). */
+ * on_device != 0: xyz and out_sqdist are device pointers; otherwise host pointers (the call waits), read in
+ * the order of the handle's stream: work queued there, or joined by vdbedt_wait_stream, may still fill them. */
 vdbedt_status vdbedt_query(vdbedt_handle h, const int32_t* xyz, int64_t n, int32_t* out_sqdist, int on_device);
 
 /* Nearest obstacle of n voxels: out_xyz[3k .. 3k + 2] is the occupied voxel o that D(v) measures

@@ -60,7 +60,6 @@ struct vdbedt_map {
   Scratch scr;
   Scratch vlast;  // per-voxel last-record table of the ordered ingest
   Scratch io;  // host-input staging on the device
-  Scratch qio;  // host queries: coordinates and results on the device
   Scratch uts;  // line stacks of the untruncated transform
   Items items{};
   int32_t* changed = nullptr;
@@ -480,7 +479,6 @@ void destroy_impl(vdbedt_map* h) {
   if (h->scr.buf) cudaFree(h->scr.buf);
   if (h->vlast.buf) cudaFree(h->vlast.buf);
   if (h->io.buf) cudaFree(h->io.buf);
-  if (h->qio.buf) cudaFree(h->qio.buf);
   if (h->uts.buf) cudaFree(h->uts.buf);
   if (h->h_pinned) cudaFreeHost(h->h_pinned);
   for (int i = 0; i < 7; ++i)
@@ -775,19 +773,12 @@ vdbedt_status vdbedt_query(vdbedt_handle h, const int32_t* xyz, int64_t n, int32
     CK(h, launch_query(h->g, xyz, n, out_sqdist, h->st), "query");
     return VDBEDT_OK;
   }
-  // The coordinates have a buffer of their own (free: each call waits for its kernel), so that page-locked
-  // ones are copied on the side stream while the handle's stream still runs what was queued before: 2^20
-  // voxels behind a transform of a 512 x 512 x 256 scene wait 60 us less for their 12 MB.
+  // the coordinates are copied on the handle's stream: work queued there may still be writing page-locked ones
   size_t bx = ((size_t)n * 12 + 255) & ~(size_t)255;
-  CK(h, ensure_scratch(h->qio, bx + (size_t)n * 4), "io alloc");
-  int32_t* dxyz = (int32_t*)h->qio.buf;
-  int32_t* dout = (int32_t*)((char*)h->qio.buf + bx);
-  const bool beside = mapped_host(xyz) != nullptr;
-  CK(h, cudaMemcpyAsync(dxyz, xyz, (size_t)n * 12, cudaMemcpyHostToDevice, beside ? h->fork.side : h->st), "h2d");
-  if (beside) {
-    CK(h, cudaEventRecord(h->fork.join, h->fork.side), "h2d");
-    CK(h, cudaStreamWaitEvent(h->st, h->fork.join, 0), "h2d");
-  }
+  CK(h, ensure_scratch(h->io, bx + (size_t)n * 4), "io alloc");
+  int32_t* dxyz = (int32_t*)h->io.buf;
+  int32_t* dout = (int32_t*)((char*)h->io.buf + bx);
+  CK(h, cudaMemcpyAsync(dxyz, xyz, (size_t)n * 12, cudaMemcpyHostToDevice, h->st), "h2d");
   CK(h, launch_query(h->g, dxyz, n, dout, h->st), "query");
   s = device_errors(h);
   if (s) return s;
@@ -952,7 +943,7 @@ vdbedt_status vdbedt_get_info(vdbedt_handle h, vdbedt_info* info) {
   info->capacity_bricks = h->g.cap;
   info->nodes = h->h_pinned[C_NNODES];
   info->device_bytes =
-      (int64_t)(h->device_bytes + h->scr.bytes + h->vlast.bytes + h->io.bytes + h->qio.bytes +
+      (int64_t)(h->device_bytes + h->scr.bytes + h->vlast.bytes + h->io.bytes +
                 (sizeof(rec_t) + sizeof(int32_t)) * h->stage_cap);
   info->R = h->g.R;
   info->error_bits = h->h_pinned[C_ERR];

@@ -69,3 +69,42 @@ def test_host_queries_behind_a_running_transform(pinned):
         grid = torch.from_numpy(np.ascontiguousarray(occ[::-1])).cuda()
         occ = np.ascontiguousarray(occ[::-1])
     m.close()
+
+
+@pytest.mark.parametrize("call", ["query", "query_nearest", "set_occupancy"])
+@pytest.mark.parametrize("joined", [False, True])
+def test_host_arrays_are_read_in_the_stream_s_order(call, joined):
+    """A page-locked array that a copy still queued on the map's stream (or on one it was made to wait for) fills."""
+    import torch
+    import paper_2105_04419_gb300 as V
+    from paper_2105_04419_gb300 import lib as L
+    rs = np.random.default_rng(7)
+    occ = (rs.random((64, 90, 130)) < 0.001).astype(np.uint8)
+    own, side = torch.cuda.Stream(), torch.cuda.Stream()
+    m = V.Map(130, 90, 64, 20, stream=own)
+    for n in (1, 1000, 200000):
+        m.set_occupancy_dense(occ)
+        m.global_()
+        xyz = np.stack([rs.integers(0, k, n) for k in (130, 90, 64)], 1).astype(np.int32)
+        there = torch.from_numpy(xyz).cuda()
+        pinned = torch.zeros((n, 3), dtype=torch.int32).pin_memory()
+        one = torch.ones(n, dtype=torch.uint8).pin_memory().numpy()
+        want = getattr(m, call)(xyz) if call != "set_occupancy" else None
+        if call == "query":
+            m.query(pinned.numpy())  # the buffers are there: nothing in the call below waits for an allocation
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side if joined else own):
+            torch.cuda._sleep(20_000_000)  # about ten milliseconds
+            pinned.copy_(there, non_blocking=True)
+            if joined:
+                assert L.load().vdbedt_wait_stream(m.handle, side.cuda_stream) == 0
+            if call == "set_occupancy":
+                m.set_occupancy(pinned.numpy(), one)
+            else:
+                assert np.array_equal(getattr(m, call)(pinned.numpy()), want), n
+        if call == "set_occupancy":
+            m.update()
+            now = occ.copy()
+            now[xyz[:, 2], xyz[:, 1], xyz[:, 0]] = 1
+            assert np.array_equal(m.export_dense(), O.edt_factorised(now, 20)), n
+    m.close()
