@@ -398,7 +398,8 @@ void* vdbedt_stream(vdbedt_handle h);
  * waiting on the host: vdbedt_wait_stream makes the handle's later work wait for what is queued on
  * `stream` now (inputs produced there); vdbedt_join_stream makes later work on `stream` wait for what is
  * queued on the handle's stream now (results used there).  Any thread; works under stream capture as an
- * event recorded on one stream and waited for on the other does. */
+ * event recorded on one stream and waited for on the other does.  ECUDA: CUDA refuses the ordering (a stream under
+ * capture against one that is not); nothing was queued and the handle stays usable. */
 vdbedt_status vdbedt_wait_stream(vdbedt_handle h, void* stream);
 vdbedt_status vdbedt_join_stream(vdbedt_handle h, void* stream);
 

@@ -198,6 +198,19 @@ vdbedt_status ensure_stage(vdbedt_map* h, int64_t need) {
   return VDBEDT_OK;
 }
 
+// Later work on `after` waits for what is queued on `before` now.  An ordering that CUDA refuses (one of the
+// streams is being captured and the other is not) queued nothing: it is reported, and the handle stays usable.
+vdbedt_status order_streams(vdbedt_map* h, cudaStream_t before, cudaStream_t after, const char* where) {
+  DeviceGuard guard(h->device);
+  std::lock_guard<std::mutex> one(h->order_lock);
+  cudaError_t e = cudaEventRecord(h->order, before);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(after, h->order, 0);
+  if (e == cudaSuccess) return VDBEDT_OK;
+  cudaGetLastError();  // not left for the next launch's check
+  h->err = std::string(where) + ": " + cudaGetErrorString(e);
+  return VDBEDT_ECUDA;
+}
+
 bool capturing(const vdbedt_map* h) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(h->st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
@@ -954,22 +967,12 @@ void* vdbedt_stream(vdbedt_handle h) { return h ? (void*)h->st : nullptr; }
 
 vdbedt_status vdbedt_wait_stream(vdbedt_handle h, void* stream) {
   vdbedt_status s = check_handle(h);
-  if (s) return s;
-  DeviceGuard guard(h->device);
-  std::lock_guard<std::mutex> one(h->order_lock);
-  CK(h, cudaEventRecord(h->order, (cudaStream_t)stream), "wait stream");
-  CK(h, cudaStreamWaitEvent(h->st, h->order, 0), "wait stream");
-  return VDBEDT_OK;
+  return s ? s : order_streams(h, (cudaStream_t)stream, h->st, "wait stream");
 }
 
 vdbedt_status vdbedt_join_stream(vdbedt_handle h, void* stream) {
   vdbedt_status s = check_handle(h);
-  if (s) return s;
-  DeviceGuard guard(h->device);
-  std::lock_guard<std::mutex> one(h->order_lock);
-  CK(h, cudaEventRecord(h->order, h->st), "join stream");
-  CK(h, cudaStreamWaitEvent((cudaStream_t)stream, h->order, 0), "join stream");
-  return VDBEDT_OK;
+  return s ? s : order_streams(h, h->st, (cudaStream_t)stream, "join stream");
 }
 
 vdbedt_status vdbedt_set_profiling(vdbedt_handle h, int on) {

@@ -108,3 +108,38 @@ def test_host_arrays_are_read_in_the_stream_s_order(call, joined):
             now[xyz[:, 2], xyz[:, 1], xyz[:, 0]] = 1
             assert np.array_equal(m.export_dense(), O.edt_factorised(now, 20)), n
     m.close()
+
+
+@pytest.mark.parametrize("captured", ["map", "caller"])
+def test_a_refused_stream_order_leaves_the_map_usable(captured):
+    """A call from a stream outside the capture of the map's own (or the reverse) is refused; later calls answer."""
+    import ctypes
+    import torch
+    import paper_2105_04419_gb300 as V
+    from paper_2105_04419_gb300 import lib as L
+    rt = ctypes.CDLL("libcudart.so.13")
+    occ = (np.random.default_rng(3).random((20, 30, 40)) < 0.01).astype(np.uint8)
+    side = torch.cuda.Stream()
+    m = V.Map(40, 30, 20, 8)
+    m.set_occupancy_dense(occ)
+    m.global_()
+    q = torch.zeros((5, 3), dtype=torch.int32, device="cuda")
+    want = m.query(q).cpu()
+    torch.cuda.synchronize()
+    stream = ctypes.c_void_p((m.stream if captured == "map" else side).cuda_stream)
+    graph = ctypes.c_void_p()
+    assert rt.cudaStreamBeginCapture(stream, 2) == 0  # relaxed
+    try:
+        if captured == "map":
+            with pytest.raises(RuntimeError):
+                m.query(q)
+        else:
+            assert L.load().vdbedt_join_stream(m.handle, side.cuda_stream) != 0
+    finally:
+        rt.cudaStreamEndCapture(stream, ctypes.byref(graph))
+        rt.cudaGetLastError()
+        if graph:
+            rt.cudaGraphDestroy(graph)
+    assert torch.equal(m.query(q).cpu(), want)
+    assert np.array_equal(m.export_dense(), O.edt_factorised(occ, 8))
+    m.close()
