@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "../../include/vdbedt.h"
@@ -39,22 +40,23 @@ static __device__ __align__(256) uint16_t g_noalloc_scratch[2 * kMaxVoxels];
 std::atomic<uint16_t*> g_scratch_ptr[kMaxDevices];
 
 // x: nearest occupied voxel along the x-line within dmax - 1, squared, saturated at dmax^2.  A warp per
-// stretch of 640 voxels of a row: ballots over its bytes and 192 more on each side give 32 words of bits,
-// one per lane, and a word of those that are not empty, so that a voxel has its nearest set bits by counts
-// of leading and trailing zeros of its own word and of the nearest other one.  117 x 96 x 83, dmax 24:
-// 4.6 us (a thread per voxel scanning bytes outward: 27).
-constexpr int kWords = 20, kHalo = 6;  // output words of a warp, and words looked at on either side (192 >= dmax)
-__global__ void __launch_bounds__(128) k_dense_x(const uint8_t* __restrict__ occ, int nx, int64_t nrows, int dmax,
-                                                 uint16_t* __restrict__ g1) {
+// stretch of `words` words of 32 voxels of a row: ballots over its bytes and `halo` words more on each side
+// (at least dmax - 1 voxels; words + 2 halo <= 32) give the words of bits, one per lane, and a word of those
+// that are not empty, so that a voxel has its nearest set bits by counts of leading and trailing zeros of its
+// own word and of the nearest other one.  117 x 96 x 83, dmax 24: 4.6 us (a thread per voxel scanning bytes
+// outward: 27).
+__global__ void __launch_bounds__(128) k_dense_x(const uint8_t* __restrict__ occ, int nx, int64_t nrows, int dmax, int words,
+                                                 int halo, uint16_t* __restrict__ g1) {
   vdbedt::pdl_enter();
   const int lane = threadIdx.x & 31, cap = dmax * dmax;
-  const int nch = (nx + 32 * kWords - 1) / (32 * kWords);
+  const int nch = (nx + 32 * words - 1) / (32 * words);
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < nrows * nch; t += nw) {
     const int64_t row = nch == 1 ? t : t / nch;
-    const int x0 = (int)(t - row * nch) * 32 * kWords - 32 * kHalo;  // position of word 0's first bit
+    const int x0 = ((int)(t - row * nch) * words - halo) * 32;  // position of word 0's first bit
     const uint8_t* src = occ + row * nx;
-    const int j0 = x0 < 0 ? kHalo : 0, j1 = min(32, (nx - x0 + 31) >> 5);  // words inside the row
+    const int j0 = x0 < 0 ? -x0 / 32 : 0;                                   // words inside the row
+    const int j1 = min(words + 2 * halo, (nx - x0 + 31) >> 5);
     uint32_t word = 0u;  // this lane's word
     for (int j = j0; j < j1; j += 4) {
       uint8_t v[4];
@@ -70,7 +72,7 @@ __global__ void __launch_bounds__(128) k_dense_x(const uint8_t* __restrict__ occ
       }
     }
     const uint32_t some = __ballot_sync(0xffffffffu, word != 0u);
-    for (int c = kHalo; c < min(j1, kHalo + kWords); ++c) {
+    for (int c = halo; c < min(j1, halo + words); ++c) {
       const uint32_t w = __shfl_sync(0xffffffffu, word, c);
       const uint32_t before = some & ((1u << c) - 1u), after = (some >> c) >> 1;
       const int b = before ? 31 - __clz(before) : 0, a = after ? c + __ffs(after) : 31;
@@ -84,13 +86,57 @@ __global__ void __launch_bounds__(128) k_dense_x(const uint8_t* __restrict__ occ
   }
 }
 
+// The same for rows of at most 32 voxels: a warp per 32 / nx whole rows, one load and one ballot for all of
+// them.  A call on 1 x 2048 x 1024, dmax 12: 34 us (354 with a warp per row, 84 with a thread per voxel).
+__global__ void __launch_bounds__(128) k_dense_x_narrow(const uint8_t* __restrict__ occ, int nx, int64_t nrows, int dmax,
+                                                        uint16_t* __restrict__ g1) {
+  vdbedt::pdl_enter();
+  const int lane = threadIdx.x & 31, cap = dmax * dmax;
+  const int per = 32 / nx, r = lane / nx, x = lane - r * nx;  // rows of a warp, this lane's row and voxel
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t * per < nrows; t += nw) {
+    const bool in = r < per && t * per + r < nrows;
+    const int64_t at = t * per * nx + lane;
+    const uint32_t all = __ballot_sync(0xffffffffu, in && __ldg(occ + at) != 0);
+    const uint32_t w = (all >> (lane - x)) & (0xffffffffu >> (32 - nx));
+    const uint32_t le = w & ((2u << x) - 1u), ge = w >> x;
+    const int dl = le ? x - (31 - __clz(le)) : dmax, dr = ge ? __ffs(ge) - 1 : dmax, d = min(min(dl, dr), dmax);
+    if (in) g1[at] = (uint16_t)min(d * d, cap);
+  }
+}
+
+// y (AXIS 1) or z (AXIS 2) of lines of up to kShortLine positions: a thread per output, outward along its line
+// (eight outputs a thread would mostly lie past the end).  A call on 1000 x 1000 x 2 takes 30.3 us, 31.1 by eights;
+// on 666 x 1000 x 3 30.1 and 28.1.
+constexpr int kShortLine = 2;
+template <int AXIS>
+__global__ void __launch_bounds__(128) k_dense_short(const uint16_t* __restrict__ in, int nx, int ny, int nz, int dmax,
+                                                     uint16_t* __restrict__ out16, int32_t* __restrict__ out32) {
+  vdbedt::pdl_enter();
+  const int64_t n = (int64_t)nx * ny * nz, stride = AXIS == 1 ? (int64_t)nx : (int64_t)nx * ny;
+  const int cap = dmax * dmax, len = AXIS == 1 ? ny : nz, reach = min(dmax, len);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int c = len == 1 ? 0 : (AXIS == 1 ? (int)((i / nx) % ny) : (int)(i / stride));
+    int best = min((int)__ldg(in + i), cap);
+    for (int d = 1; d < reach && d * d < best; ++d) {
+      if (c - d >= 0) best = min(best, d * d + (int)__ldg(in + i - d * stride));
+      if (c + d < len) best = min(best, d * d + (int)__ldg(in + i + d * stride));
+    }
+    if (AXIS == 2)
+      out32[i] = best;
+    else
+      out16[i] = (uint16_t)best;
+  }
+}
+
 // y (AXIS 1) or z (AXIS 2): min over |d| < dmax of d^2 + the previous field at offset d.  A thread per
 // eight outputs along the axis (a warp's threads along x): the eight inputs among themselves, then plane by
 // plane outward on both sides, each loaded once for all eight; every fourth plane the walk stops
 // when the square of the next offset reaches the largest minimum.  (d + k)^2 = d^2 + 2 d k + k^2: the
 // minima are kept less k^2, a multiply-add and half a three-way minimum per candidate and output.  Bound by
 // the latency of the loads at such sizes: 117 x 96 x 83, dmax 24: about 6 us each, their launches
-// overlapping the pass before (a thread per output: 14.5).
+// overlapping the pass before (a thread per output: 14.5).  No offset reaches past the line: those of a line
+// of up to eight positions are all among themselves.
 template <int AXIS>
 __global__ void __launch_bounds__(128) k_dense_win(const uint16_t* __restrict__ in, int nx, int ny, int nz, int dmax,
                                                    uint16_t* __restrict__ out16, int32_t* __restrict__ out32) {
@@ -98,6 +144,7 @@ __global__ void __launch_bounds__(128) k_dense_win(const uint16_t* __restrict__ 
   const int cap = dmax * dmax, len = AXIS == 1 ? ny : nz, nb = (len + 7) / 8;
   const int64_t stride = AXIS == 1 ? (int64_t)nx : (int64_t)nx * ny;
   const int64_t n = AXIS == 1 ? (int64_t)nx * nb * nz : (int64_t)nx * ny * nb;
+  const int reach = nb == 1 ? 1 : min(dmax, len);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     int b;          // eighth of the line
     int64_t line;   // its first voxel
@@ -124,7 +171,7 @@ __global__ void __launch_bounds__(128) k_dense_win(const uint16_t* __restrict__ 
         acc[k] = m - k * k;
       }
     }
-    for (int d = 1; d < dmax; d += 4) {
+    for (int d = 1; d < reach; d += 4) {
       int lo[4], hi[4], mx = 0;
 #pragma unroll
       for (int k = 0; k < 8; ++k) mx = max(mx, acc[k] + k * k);
@@ -208,13 +255,26 @@ extern "C" vdbedt_status vdbedt_edt_dense_noalloc(const uint8_t* occ, int32_t nx
   uint16_t* g1 = scratch;
   uint16_t* g2 = scratch + kMaxVoxels;
   const int64_t nrows = (int64_t)ny * nz;
-  VDB_LAUNCH(k_dense_x, blocks(nrows * ((nx + 32 * kWords - 1) / (32 * kWords)) * 32), 128, 0, st, occ, nx, nrows, dmax, g1);
+  if (nx <= 32) {
+    VDB_LAUNCH(k_dense_x_narrow, blocks((nrows + 32 / nx - 1) / (32 / nx) * 32), 128, 0, st, occ, nx, nrows, dmax, g1);
+  } else {
+    // stretches of four words at least, longer where the GPU is full without: few long rows (1000 x 1000 x 1)
+    // would leave it idle while a warp each works through twenty words
+    // (kMaxVoxels allows 127,100 words of rows: at most 15, with 2 x 6 of the halo below 32)
+    const int halo = (dmax + 31) / 32, words = (int)std::max<int64_t>(4, nrows * ((nx + 31) / 32) / 8192);
+    VDB_LAUNCH(k_dense_x, blocks(nrows * ((nx + 32 * words - 1) / (32 * words)) * 32), 128, 0, st, occ, nx, nrows, dmax, words,
+               halo, g1);
+  }
   if (cudaGetLastError() != cudaSuccess) return noalloc_fail(VDBEDT_ECUDA, "vdbedt_edt_dense_noalloc: x launch");
-  VDB_LAUNCH_PDL(k_dense_win<1>, blocks((int64_t)nx * ((ny + 7) / 8) * nz), 128, 0, st, (const uint16_t*)g1, (int)nx, (int)ny,
-                 (int)nz, (int)dmax, g2, (int32_t*)nullptr);
-  if (cudaGetLastError() != cudaSuccess) return noalloc_fail(VDBEDT_ECUDA, "vdbedt_edt_dense_noalloc: y launch");
-  VDB_LAUNCH_PDL(k_dense_win<2>, blocks(nrows / nz * ((nz + 7) / 8) * nx), 128, 0, st, (const uint16_t*)g2, (int)nx, (int)ny,
-                 (int)nz, (int)dmax, (uint16_t*)nullptr, out);
-  if (cudaGetLastError() != cudaSuccess) return noalloc_fail(VDBEDT_ECUDA, "vdbedt_edt_dense_noalloc: z launch");
+  const auto line = [&](auto wide, auto brief, int len, const uint16_t* in, uint16_t* out16, int32_t* out32) {
+    const bool is_short = len <= kShortLine;
+    VDB_LAUNCH_PDL(is_short ? brief : wide, blocks(is_short ? n : n / len * ((len + 7) / 8)), 128, 0, st, in, (int)nx, (int)ny, (int)nz,
+                   (int)dmax, out16, out32);
+    return cudaGetLastError();
+  };
+  if (line(k_dense_win<1>, k_dense_short<1>, ny, g1, g2, nullptr) != cudaSuccess)
+    return noalloc_fail(VDBEDT_ECUDA, "vdbedt_edt_dense_noalloc: y launch");
+  if (line(k_dense_win<2>, k_dense_short<2>, nz, g2, nullptr, out) != cudaSuccess)
+    return noalloc_fail(VDBEDT_ECUDA, "vdbedt_edt_dense_noalloc: z launch");
   return VDBEDT_OK;
 }
