@@ -39,3 +39,26 @@ def test_batch_grids():
     for m, g in zip(b.maps, grids):
         q = all_voxels(g.shape)
         assert np.array_equal(m.query_nearest(q), O.nearest_obstacle(g, 12, q))
+
+
+@pytest.mark.parametrize("p", [0.25, 0.45, 0.97])
+@pytest.mark.parametrize("dmax", [1, 2, 8, 50])
+def test_crowded_maps(p, dmax):
+    """Warps whose lanes all have an obstacle within one voxel, and warps where some have not."""
+    import paper_2105_04419_gb300 as V
+    occ = scattered((11, 13, 19), p, dmax)
+    occ[2:7, 3:8, 4:13] = 0
+    m = gpu_global(occ, dmax)
+    q = all_voxels(occ.shape)
+    outside = q[::5] + np.array([19, 0, 0], np.int32)
+    q = np.concatenate([q, outside, q[::-1]])
+    assert np.array_equal(m.query_nearest(q), O.nearest_obstacle(occ, dmax, q))
+    m.synchronize()
+    u = V.Map(0, 0, 0, dmax, unbounded=True, max_bricks=20000, max_nodes=64)
+    z, y, x = np.nonzero(occ)
+    shift = np.array([-13, -10, -9], np.int32)
+    u.set_occupancy(np.stack([x, y, z], 1).astype(np.int32) + shift, np.ones(len(x), np.uint8))
+    u.global_()
+    want = O.nearest_obstacle(occ, dmax, q[: occ.size])
+    assert np.array_equal(u.query_nearest(q[: occ.size] + shift), np.where(want < 0, want, want + shift))
+    u.synchronize()
