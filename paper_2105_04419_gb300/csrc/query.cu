@@ -89,6 +89,18 @@ __global__ void __launch_bounds__(256) k_export_dense(GridView g, int32_t* __res
   }
 }
 
+// Fields narrower than a brick: a thread per voxel.  A warp per plane of a brick row would have 8 x nx outputs:
+// 1 x 1024 x 1024 takes 25 us, 50 so; 7 x 1024 x 512 25 and 28; from a brick's width on the warp is faster (8 x 1024 x
+// 1024: 53 and 47).
+__global__ void __launch_bounds__(256) k_export_narrow(GridView g, int32_t* __restrict__ out) {
+  pdl_enter();
+  const int64_t total = (int64_t)g.nx * g.ny * g.nz;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / g.nx;
+    out[i] = sqdist_at(g, (int)(i - r * g.nx), (int)(r % g.ny), (int)(r / g.ny));
+  }
+}
+
 // A thread's last node lookup (key, node): the bricks of one query mostly fall in one interior node,
 // so most lookups skip the hash table.
 struct NodeCache {
@@ -498,8 +510,9 @@ cudaError_t launch_export_occupancy(const GridView& g, const int32_t* changed, i
 }
 
 cudaError_t launch_export_dense(const GridView& g, int32_t* out, cudaStream_t st) {
-  const unsigned blocks = grid_for((int64_t)g.NX * g.BY * g.BZ * 8 * 32, 256);
-  const auto kernel = g.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0 ? k_export_dense<true> : k_export_dense<false>;
+  const bool narrow = g.nx < kBrick, vec = g.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+  const unsigned blocks = grid_for(narrow ? (int64_t)g.nx * g.ny * g.nz : (int64_t)g.NX * g.BY * g.BZ * 8 * 32, 256);
+  const auto kernel = narrow ? k_export_narrow : (vec ? k_export_dense<true> : k_export_dense<false>);
   // small fields are chained to the pass before (as the passes are); behind one that fills the GPU the blocks
   // that start early keep its shared-memory split, and a 1024 x 1024 x 256 field takes 0.09 ms longer
   if ((int64_t)g.BX * g.BY * g.BZ <= 16384)

@@ -26,3 +26,14 @@ def test_export_matches_oracle(shape, offset):
     got = out.cpu().numpy()
     assert np.array_equal(got[offset:offset + occ.size].reshape(shape), O.edt_factorised(occ, 9))
     assert (got[:offset] == -7).all() and (got[offset + occ.size:] == -7).all()
+
+
+@pytest.mark.parametrize("nx", [1, 2, 3, 4, 5, 6, 7, 8])
+def test_narrow_maps(nx):
+    """Maps of a brick's width and less: a thread per exported voxel."""
+    rs = np.random.default_rng(nx)
+    for shape in ((1, 1, nx), (130, 13, nx), (9, 200, nx)):
+        occ = (rs.random(shape) < 0.01).astype(np.uint8)
+        m = gpu_global(occ, 10)
+        assert np.array_equal(m.export_dense(), O.edt_factorised(occ, 10)), shape
+        m.close()
