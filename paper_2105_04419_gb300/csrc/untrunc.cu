@@ -413,8 +413,10 @@ __host__ __device__ inline size_t line_smem(int n) {
   return nb * 8 * 128 + nb * 128 + (nb + 1) * 64;
 }
 
+// At most 40 registers a thread: blocks of 1,024 (the longest lines) stay launchable whatever the compiler, and
+// three blocks of 512 fit an SM.
 template <int AXIS, bool UPD>
-__global__ void k_ut_line(GridView g, const int32_t* __restrict__ in, int32_t* __restrict__ out) {
+__global__ void __maxnreg__(40) k_ut_line(GridView g, const int32_t* __restrict__ in, int32_t* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = AXIS == 1 ? g.ny : g.nz, nb = line_bricks(n), nc = AXIS == 1 ? g.nz : g.ny;
   uint32_t* val = reinterpret_cast<uint32_t*>(smem);               // [8 nb][32]
