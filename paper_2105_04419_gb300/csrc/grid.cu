@@ -205,9 +205,8 @@ __global__ void k_begin_batch_update(const UpdArgs* __restrict__ args, BatchCoun
 }
 
 // ---- brick allocation ----
-// Fill a freshly allocated brick: empty occupancy, coordinates, flags (no plane holds a value below
-// dmax^2); with `init_fields` also g1, g2 and D at dmax^2 (bricks added by an incremental update may
-// be read before a pass writes them).
+// Coordinates and flags of a freshly allocated brick (no plane holds a value below dmax^2).  Its g1, g2 and D are
+// written by the passes, and before an update's by init_new_fields.
 __device__ __forceinline__ void init_brick_meta(const GridView& g, int slot, int node, int bx, int by, int bz) {
   g.bcoord[slot] = make_int4(bx, by, bz, node);
   g.bflags[slot] = 0u;
@@ -234,19 +233,11 @@ __device__ __forceinline__ void init_fields_warp(const GridView& g, int slot, in
   for (int q = 0; q < 4; ++q) dd[lane + 32 * q] = w;
 }
 
-__device__ void init_brick(const GridView& g, int slot, int node, int bx, int by, int bz, bool init_fields) {
+// The same with an empty occupancy.
+__device__ __forceinline__ void init_brick(const GridView& g, int slot, int node, int bx, int by, int bz) {
   ulonglong2* occ = reinterpret_cast<ulonglong2*>(g.occ + (size_t)slot * 8);
 #pragma unroll
   for (int q = 0; q < 4; ++q) occ[q] = make_ulonglong2(0ull, 0ull);
-  if (init_fields) {
-    const uint32_t p = field_inf2(g);
-    uint4* dst = reinterpret_cast<uint4*>(g.g2 + (size_t)slot * kBrickVox);
-    for (int q = 0; q < 64; ++q) dst[q] = make_uint4(p, p, p, p);
-    uint4* d1 = reinterpret_cast<uint4*>(g.g1 + (size_t)slot * kBrickVox);
-    for (int q = 0; q < 64; ++q) d1[q] = make_uint4(p, p, p, p);
-    int4* dd = reinterpret_cast<int4*>(g.dist + (size_t)slot * kBrickVox);
-    for (int q = 0; q < 128; ++q) dd[q] = make_int4(g.INF, g.INF, g.INF, g.INF);
-  }
   init_brick_meta(g, slot, node, bx, by, bz);
 }
 
@@ -302,14 +293,14 @@ __device__ __forceinline__ int64_t rec_count(int64_t n, const int32_t* n_dev) {
   for (int64_t i##_base = (int64_t)blockIdx.x * blockDim.x, i = i##_base + threadIdx.x; i##_base < (n); \
        i##_base += (int64_t)gridDim.x * blockDim.x, i = i##_base + threadIdx.x)
 
-// Places for the lanes with `want` in a list counted by *ctr: one atomic per warp (warp-uniform
-// call); returns the lane's place (meaningful where want).
 // Sets a flag word that only ever goes from 0 to 1, reading it first (L2): once one warp has set
 // it the others find it set and issue no atomic on the shared word.
 __device__ __forceinline__ void set_once(int32_t* flag) {
   if (!__ldcg(flag)) atomicOr(flag, 1);
 }
 
+// Places for the lanes with `want` in a list counted by *ctr: one atomic per warp (warp-uniform
+// call); returns the lane's place (meaningful where want).
 __device__ __forceinline__ int warp_reserve(int32_t* ctr, bool want) {
   const unsigned m = __ballot_sync(0xffffffffu, want);
   if (!m) return 0;
@@ -517,7 +508,7 @@ __global__ void k_compact_keys(const uint32_t* __restrict__ keys, const int32_t*
 }
 
 // Bricks of the unique keys: node found or inserted, slot reserved with one atomic per block.
-__global__ void k_alloc_obstacle_bricks(GridView g, const uint32_t* __restrict__ uniq, int64_t n, bool init,
+__global__ void k_alloc_obstacle_bricks(GridView g, const uint32_t* __restrict__ uniq, int64_t n,
                                         const unsigned long long* __restrict__ dbits) {
   pdl_enter();
   const int64_t cnt = min((int64_t)g.counters[C_UNIQUE], n);
@@ -551,7 +542,7 @@ __global__ void k_alloc_obstacle_bricks(GridView g, const uint32_t* __restrict__
 #pragma unroll
           for (int q = 0; q < 4; ++q) dst[q] = src[q];
         } else {
-          init_brick(g, slot, node, bx, by, bz, init);
+          init_brick(g, slot, node, bx, by, bz);
         }
         *e = slot;
       }
@@ -660,7 +651,7 @@ __global__ void k_rec_slots(US us) {
       atomicAnd(&g.nclaim[(size_t)node * 128 + (l >> 5)], ~(1u << (l & 31)));
     }
     if (ok) {
-      init_brick(g, slot, node, bx, by, bz, false);
+      init_brick(g, slot, node, bx, by, bz);
       g.child[(size_t)node * kNodeBricks + local_brick(bx, by, bz)] = slot;
       rs = -3 - slot;
     }
@@ -691,23 +682,12 @@ __device__ __forceinline__ int64_t rec_voxel(const GridView& g, rec_t packed) {
   return (int64_t)s * 512 + ((r.x & 7) + 8 * (r.y & 7) + 64 * (r.z & 7));
 }
 
-__device__ __forceinline__ void rec_last(const GridView& g, const rec_t* __restrict__ rec, int64_t n_max,
-                                         const int32_t* n_dev, bool force, int32_t* __restrict__ vlast) {
-  if (!force && !g.counters[C_HAS_ZERO]) return;
-  const int64_t n = rec_count(n_max, n_dev);
-  GRID_STRIDE(i, n) {
-    if (i < n) {
-      const int64_t key = rec_voxel(g, rec[i]);
-      if (key >= 0) atomicMax(&vlast[key], (int)i);
-    }
-  }
-}
-
-// Flips are counted; with `track` the brick is appended once per epoch to the changed list.
+// Flips are counted; with TRACK (an update) the brick is appended once per epoch to the changed list, and each
+// record's brick slot comes from rslot.
+template <bool TRACK>
 __device__ __forceinline__ void apply_last(const GridView& g, const rec_t* __restrict__ rec, int64_t n_max,
-                                           const int32_t* n_dev, bool force, bool track, int32_t* __restrict__ vlast,
-                                           int32_t* __restrict__ changed, const int32_t* __restrict__ rslot = nullptr) {
-  if (!force && !g.counters[C_HAS_ZERO]) return;
+                                           const int32_t* n_dev, int32_t* __restrict__ vlast,
+                                           int32_t* __restrict__ changed, const int32_t* __restrict__ rslot) {
   const int64_t n = rec_count(n_max, n_dev);
   const int epoch = g.counters[C_EPOCH];
   GRID_STRIDE(j, n) {
@@ -716,7 +696,7 @@ __device__ __forceinline__ void apply_last(const GridView& g, const rec_t* __res
     if (j < n) {
       const rec_t packed = rec[j];
       int64_t key;
-      if (rslot) {
+      if (TRACK) {
         const int sl = rslot[j];
         key = sl >= 0 ? (int64_t)sl * 512 + rec_in_brick(packed) : -1;
       } else {
@@ -731,9 +711,9 @@ __device__ __forceinline__ void apply_last(const GridView& g, const rec_t* __res
         if (cur != ((packed >> 63) != 0ull)) {
           atomicXor(word, bit);
           flip = true;
-          first = track && atomicExch(&g.bepoch[s], epoch) != epoch;
+          first = TRACK && atomicExch(&g.bepoch[s], epoch) != epoch;
           slot = s;
-          if (track && g.ut_bits) {
+          if (TRACK && g.ut_bits) {
             // untruncated grid (brick s at bx + BX (by + BY bz)): the voxel's x row is dirty
             const int64_t row = (int64_t)(s / g.BX) * 64 + (v >> 3);
             atomicOr(&g.ut_bits[row >> 5], 1u << (row & 31));
@@ -743,22 +723,32 @@ __device__ __forceinline__ void apply_last(const GridView& g, const rec_t* __res
     }
     // the changed list: each brick once per epoch, a block's bricks with one atomic (as the flip
     // count): the counter words see one atomic per block, not one per warp
-    const int p = block_agg_add(&g.counters[C_CHANGED], first, nullptr);
-    if (first) changed[p] = slot;
+    if (TRACK) {
+      const int p = block_agg_add(&g.counters[C_CHANGED], first, nullptr);
+      if (first) changed[p] = slot;
+    }
     block_agg_add(&g.counters[C_FLIPS], flip, nullptr);
   }
 }
 
-__global__ void k_rec_last(GridView g, const rec_t* __restrict__ rec, int64_t n_max, const int32_t* n_dev, bool force,
+__global__ void k_rec_last(GridView g, const rec_t* __restrict__ rec, int64_t n_max, const int32_t* n_dev,
                            int32_t* __restrict__ vlast) {
   pdl_enter();
-  rec_last(g, rec, n_max, n_dev, force, vlast);
+  if (!g.counters[C_HAS_ZERO]) return;
+  const int64_t n = rec_count(n_max, n_dev);
+  GRID_STRIDE(i, n) {
+    if (i < n) {
+      const int64_t key = rec_voxel(g, rec[i]);
+      if (key >= 0) atomicMax(&vlast[key], (int)i);
+    }
+  }
 }
 
 __global__ void k_apply_last(GridView g, const rec_t* __restrict__ rec, int64_t n_max, const int32_t* n_dev,
-                             bool force, bool track, int32_t* __restrict__ vlast, int32_t* __restrict__ changed) {
+                             int32_t* __restrict__ vlast) {
   pdl_enter();
-  apply_last(g, rec, n_max, n_dev, force, track, vlast, changed);
+  if (!g.counters[C_HAS_ZERO]) return;
+  apply_last<false>(g, rec, n_max, n_dev, vlast, nullptr, nullptr);
 }
 
 // The tracked forms (incremental update): every record, flips tracked, each record's brick slot
@@ -794,7 +784,7 @@ template <class US>
 __global__ void k_upd_apply_last(US us) {
   pdl_enter();
   const UpdArgs A = us.get();
-  apply_last(A.g, A.rec, A.n, A.n_dev, true, true, A.vlast, A.changed, A.rslot);
+  apply_last<true>(A.g, A.rec, A.n, A.n_dev, A.vlast, A.changed, A.rslot);
 }
 
 // ---- dense ingest ----
@@ -1273,8 +1263,6 @@ __global__ void __launch_bounds__(256) k_dilate_nodes(VS vs) {
   }
 }
 
-// Mark bricks within Chebyshev radius R of brick (bx,by,bz) in amask: one (dy, dz) row (used by the
-// incremental form, where few bricks change).
 // Places for `cnt` items of each lane in a list counted by *ctr: one atomic per warp (warp-uniform
 // call); returns the lane's first place.  *total receives the warp's sum.
 __device__ __forceinline__ int warp_reserve_count(int32_t* ctr, int cnt, int* total) {
@@ -1322,7 +1310,7 @@ __device__ void alloc_new_bits(const GridView& g, int node, int word, uint32_t b
       set_error(g, kErrOverflow);
       continue;
     }
-    init_brick(g, slot, node, x16 + (bit & 15), y, z, false);
+    init_brick(g, slot, node, x16 + (bit & 15), y, z);
     g.child[(size_t)node * kNodeBricks + word * 32 + bit] = slot;
   }
 }
@@ -1354,7 +1342,7 @@ __global__ void __launch_bounds__(256) k_alloc_marked(VS vs, bool zero_items) {
       } else {
         int nxn, nyn, nzn;
         node_coords(g, (unsigned long long)g.node_key[node], nxn, nyn, nzn);
-        init_brick(g, slot, node, nxn * 16 + (l & 15), nyn * 16 + ((l >> 4) & 15), nzn * 16 + (l >> 8), false);
+        init_brick(g, slot, node, nxn * 16 + (l & 15), nyn * 16 + ((l >> 4) & 15), nzn * 16 + (l >> 8));
         g.child[(size_t)node * kNodeBricks + l] = slot;
       }
     }
@@ -1900,15 +1888,15 @@ static bool counting_ingest(const GridView& g, int64_t n) {
   const int64_t nbr_all = (int64_t)g.BX * g.BY * g.BZ;
   return n >= nbr_all / 4 || (nbr_all <= kFlagBricks && nbr_all <= 4 * (int64_t)g.cap);
 }
-static bool dense_bits_ingest(const GridView& g, int64_t n, bool track) {
+static bool dense_bits_ingest(const GridView& g, int64_t n) {
   const int64_t nbr_all = (int64_t)g.BX * g.BY * g.BZ;
   // the dense mask is indexed by a 32-bit word number (8 words per brick)
-  return n >= nbr_all / 4 && !track && nbr_all * 8 < (int64_t)0xFFFFFFFFll;
+  return n >= nbr_all / 4 && nbr_all * 8 < (int64_t)0xFFFFFFFFll;
 }
-static size_t ingest_scratch_bytes(const GridView& g, int64_t n, bool track) {
+static size_t ingest_scratch_bytes(const GridView& g, int64_t n) {
   const int64_t nbr_all = (int64_t)g.BX * g.BY * g.BZ;
   const bool counting = counting_ingest(g, n);
-  const bool dense_bits = dense_bits_ingest(g, n, track);
+  const bool dense_bits = dense_bits_ingest(g, n);
   const int64_t m = counting && nbr_all > n ? nbr_all : n;  // brick flags only on the counting path
   const size_t nb4 = align_up((size_t)m * 4);
   const size_t nkeys_al = ((size_t)g.NX * g.NY * g.NZ + 63) & ~(size_t)63;
@@ -1928,7 +1916,7 @@ static cudaError_t ensure_vlast(const GridView& g, Scratch& vl, cudaStream_t st)
 
 cudaError_t reserve_ingest(const GridView& g, int64_t n, Scratch& scr, Scratch& vl, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  cudaError_t e = g.unbounded ? cudaSuccess : ensure_scratch(scr, ingest_scratch_bytes(g, n, false));
+  cudaError_t e = g.unbounded ? cudaSuccess : ensure_scratch(scr, ingest_scratch_bytes(g, n));
   if (e != cudaSuccess) return e;
   return ensure_vlast(g, vl, st);
 }
@@ -1969,10 +1957,10 @@ cudaError_t launch_ingest_records(const GridView& g, const rec_t* rec, int64_t n
   if (track || g.unbounded) return launch_ingest_tracked(g, rec, n, n_dev, changed, rslot, vl, st);
   const int64_t nbr_all = (int64_t)g.BX * g.BY * g.BZ;
   const bool counting = counting_ingest(g, n);
-  const bool dense_bits = dense_bits_ingest(g, n, track);
+  const bool dense_bits = dense_bits_ingest(g, n);
   const int64_t m = counting && nbr_all > n ? nbr_all : n;  // brick flags only on the counting path
   const size_t nb4 = align_up((size_t)m * 4);
-  cudaError_t e = ensure_scratch(scr, ingest_scratch_bytes(g, n, track));
+  cudaError_t e = ensure_scratch(scr, ingest_scratch_bytes(g, n));
   if (e != cudaSuccess) return e;
   e = ensure_vlast(g, vl, st);
   if (e != cudaSuccess) return e;
@@ -2007,8 +1995,8 @@ cudaError_t launch_ingest_records(const GridView& g, const rec_t* rec, int64_t n
     VDB_LAUNCH(k_mark_record_bricks, nbk, kT, 0, st, g, rec, n, n_dev, flag, dbits);
     VDB_LAUNCH_PDL(k_compact_flag_index, blocks_for((int64_t)nbr), kT, 0, st, g, flag, (int64_t)nbr, ka, nflag);
     VDB_LAUNCH_PDL(k_create_flagged_nodes, blocks_for(nkeys), kT, 0, st, g, nflag, nkeys);
-    VDB_LAUNCH_PDL(k_alloc_obstacle_bricks, blocks_for((int64_t)nbr), kT, 0, st, g, ka, (int64_t)nbr, track, dbits);
-    if (!track && !dbits) VDB_LAUNCH_PDL(k_apply_set_only, nbk, kT, 0, st, g, rec, n, n_dev);
+    VDB_LAUNCH_PDL(k_alloc_obstacle_bricks, blocks_for((int64_t)nbr), kT, 0, st, g, ka, (int64_t)nbr, dbits);
+    if (!dbits) VDB_LAUNCH_PDL(k_apply_set_only, nbk, kT, 0, st, g, rec, n, n_dev);
   } else {
     // LSD radix sort of the brick keys, unique, compaction
     VDB_LAUNCH(k_rec_brick_keys, nbk, kT, 0, st, g, rec, n, n_dev, ka);
@@ -2026,12 +2014,12 @@ cudaError_t launch_ingest_records(const GridView& g, const rec_t* rec, int64_t n
     if (e != cudaSuccess) return e;
     VDB_LAUNCH(k_flag_key_nodes, blocks_for(n), kT, 0, st, g, uniq, n, nflag);
     VDB_LAUNCH_PDL(k_create_flagged_nodes, blocks_for(nkeys), kT, 0, st, g, nflag, nkeys);
-    VDB_LAUNCH_PDL(k_alloc_obstacle_bricks, blocks_for(n), kT, 0, st, g, uniq, n, track, nullptr);
-    if (!track) VDB_LAUNCH_PDL(k_apply_set_only, nbk, kT, 0, st, g, rec, n, n_dev);
+    VDB_LAUNCH_PDL(k_alloc_obstacle_bricks, blocks_for(n), kT, 0, st, g, uniq, n, nullptr);
+    VDB_LAUNCH_PDL(k_apply_set_only, nbk, kT, 0, st, g, rec, n, n_dev);
   }
-  // ordered path (its kernels return at once when no record clears a voxel and flips are untracked)
-  VDB_LAUNCH_PDL(k_rec_last, nbk, kT, 0, st, g, rec, n, n_dev, track, vlast);
-  VDB_LAUNCH_PDL(k_apply_last, nbk, kT, 0, st, g, rec, n, n_dev, track, track, vlast, changed);
+  // ordered path (its kernels return at once when no record clears a voxel)
+  VDB_LAUNCH_PDL(k_rec_last, nbk, kT, 0, st, g, rec, n, n_dev, vlast);
+  VDB_LAUNCH_PDL(k_apply_last, nbk, kT, 0, st, g, rec, n, n_dev, vlast);
   return cudaGetLastError();
 }
 
