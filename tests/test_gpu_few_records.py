@@ -28,3 +28,26 @@ def test_flags_and_sort_agree(n):
         m.set_occupancy(xyz, val)
         m.global_()
         assert first_mismatch(m.export_dense(), want) is None, kw
+
+
+@pytest.mark.parametrize("max_bricks,n", [(300, 700), (300, 30), (3600, 700)])
+def test_more_bricks_than_fit(max_bricks, n):
+    """Sorted records whose own bricks, or whose dilation, exceed the capacity, and flagged ones (from a quarter of the
+    grid's bricks on): refused at the next synchronisation, and a reset map takes what fits."""
+    import paper_2105_04419_gb300 as V
+    nx, ny, nz, dmax = 261, 197, 130, 10  # 14,025 bricks
+    rs = np.random.default_rng(n + max_bricks)
+    xyz = np.stack([rs.integers(0, k, n) for k in (nx, ny, nz)], 1).astype(np.int32)
+    m = V.Map(nx, ny, nz, dmax, max_bricks=max_bricks)
+    m.set_occupancy(xyz, np.ones(n, np.uint8))
+    m.global_()
+    with pytest.raises(V.VdbedtError) as e:
+        m.synchronize()
+    assert e.value.code == "EOVERFLOW"
+    m.reset()
+    occ = np.zeros((nz, ny, nx), np.uint8)
+    occ[xyz[0, 2], xyz[0, 1], xyz[0, 0]] = 1
+    m.set_occupancy(xyz[:1], np.ones(1, np.uint8))
+    m.global_()
+    assert first_mismatch(m.export_dense(), O.edt_factorised(occ, dmax)) is None
+    m.close()
