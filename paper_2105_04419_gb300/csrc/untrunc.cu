@@ -13,6 +13,8 @@
 //      int32 and each product one widening multiply (below 2^48).
 // kNone marks a row, plane or grid without an obstacle.  Only voxels inside the grid are read or
 // written; g1 and g2 hold int32 here (their arrays are allocated twice as large).
+#include <algorithm>
+
 #include "line_min.cuh"
 #include "vdbedt_internal.cuh"
 
@@ -413,10 +415,8 @@ __host__ __device__ inline size_t line_smem(int n) {
   return nb * 8 * 128 + nb * 128 + (nb + 1) * 64;
 }
 
-// At most 40 registers a thread: blocks of 1,024 (the longest lines) stay launchable whatever the compiler, and
-// three blocks of 512 fit an SM.
 template <int AXIS, bool UPD>
-__global__ void __maxnreg__(40) k_ut_line(GridView g, const int32_t* __restrict__ in, int32_t* __restrict__ out) {
+__global__ void k_ut_line(GridView g, const int32_t* __restrict__ in, int32_t* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = AXIS == 1 ? g.ny : g.nz, nb = line_bricks(n), nc = AXIS == 1 ? g.nz : g.ny;
   uint32_t* val = reinterpret_cast<uint32_t*>(smem);               // [8 nb][32]
@@ -522,7 +522,13 @@ cudaError_t launch_line(const GridView& g, const int32_t* in, int32_t* out, cuda
   const cudaError_t e = cudaFuncSetAttribute(k_ut_line<AXIS, UPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)line_smem(kLineMax));
   if (e != cudaSuccess) return e;
-  const int threads = n <= 64 ? 128 : (n <= 128 ? 256 : (n <= 768 ? 512 : 1024));
+  // blocks of up to 1,024 where the compiled kernel's registers allow them (any whole number of warps serves;
+  // declared bounds or registers made the compiler's code 1 % slower)
+  static const int most = [] {
+    cudaFuncAttributes a{};
+    return cudaFuncGetAttributes(&a, k_ut_line<AXIS, UPD>) == cudaSuccess ? a.maxThreadsPerBlock & ~31 : 256;
+  }();
+  const int threads = std::min(n <= 64 ? 128 : (n <= 128 ? 256 : (n <= 768 ? 512 : 1024)), most);
   VDB_LAUNCH((k_ut_line<AXIS, UPD>), (unsigned)tiles, threads, line_smem(n), st, g, in, out);
   return cudaGetLastError();
 }
