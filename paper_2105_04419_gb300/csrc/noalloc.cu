@@ -40,23 +40,25 @@ static __device__ __align__(256) uint16_t g_noalloc_scratch[2 * kMaxVoxels];
 std::atomic<uint16_t*> g_scratch_ptr[kMaxDevices];
 
 // x: nearest occupied voxel along the x-line within dmax - 1, squared, saturated at dmax^2.  A warp per
-// stretch of `words` words of 32 voxels of a row: ballots over its bytes and `halo` words more on each side
-// (at least dmax - 1 voxels; words + 2 halo <= 32) give the words of bits, one per lane, and a word of those
-// that are not empty, so that a voxel has its nearest set bits by counts of leading and trailing zeros of its
-// own word and of the nearest other one.  117 x 96 x 83, dmax 24: 4.6 us (a thread per voxel scanning bytes
-// outward: 27).
-__global__ void __launch_bounds__(128) k_dense_x(const uint8_t* __restrict__ occ, int nx, int64_t nrows, int dmax, int words,
-                                                 int halo, uint16_t* __restrict__ g1) {
+// stretch of WORDS words of 32 voxels of a row: ballots over its bytes and HALO words more on each side
+// (at least dmax - 1 voxels) give the words of bits, one per lane, and a word of those that are not empty, so
+// that a voxel has its nearest set bits by counts of leading and trailing zeros of its own word and of the
+// nearest other one.  117 x 96 x 83, dmax 24: 4.6 us (a thread per voxel scanning bytes outward: 27).
+// Stretches of 20 words; of four where a few long rows would leave the GPU idle while a warp each works through
+// twenty (a call on 1000 x 1000 x 1, dmax 12: 20 us, was 43).
+template <int WORDS, int HALO>
+__global__ void __launch_bounds__(128) k_dense_x(const uint8_t* __restrict__ occ, int nx, int64_t nrows, int dmax,
+                                                 uint16_t* __restrict__ g1) {
+  static_assert(WORDS + 2 * HALO <= 32, "a word per lane");
   vdbedt::pdl_enter();
   const int lane = threadIdx.x & 31, cap = dmax * dmax;
-  const int nch = (nx + 32 * words - 1) / (32 * words);
+  const int nch = (nx + 32 * WORDS - 1) / (32 * WORDS);
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < nrows * nch; t += nw) {
     const int64_t row = nch == 1 ? t : t / nch;
-    const int x0 = ((int)(t - row * nch) * words - halo) * 32;  // position of word 0's first bit
+    const int x0 = ((int)(t - row * nch) * WORDS - HALO) * 32;  // position of word 0's first bit
     const uint8_t* src = occ + row * nx;
-    const int j0 = x0 < 0 ? -x0 / 32 : 0;                                   // words inside the row
-    const int j1 = min(words + 2 * halo, (nx - x0 + 31) >> 5);
+    const int j0 = max(0, -(x0 >> 5)), j1 = min(WORDS + 2 * HALO, (nx - x0 + 31) >> 5);  // words inside the row
     uint32_t word = 0u;  // this lane's word
     for (int j = j0; j < j1; j += 4) {
       uint8_t v[4];
@@ -72,7 +74,7 @@ __global__ void __launch_bounds__(128) k_dense_x(const uint8_t* __restrict__ occ
       }
     }
     const uint32_t some = __ballot_sync(0xffffffffu, word != 0u);
-    for (int c = halo; c < min(j1, halo + words); ++c) {
+    for (int c = HALO; c < min(j1, HALO + WORDS); ++c) {
       const uint32_t w = __shfl_sync(0xffffffffu, word, c);
       const uint32_t before = some & ((1u << c) - 1u), after = (some >> c) >> 1;
       const int b = before ? 31 - __clz(before) : 0, a = after ? c + __ffs(after) : 31;
@@ -110,11 +112,11 @@ __global__ void __launch_bounds__(128) k_dense_x_narrow(const uint8_t* __restric
 // on 666 x 1000 x 3 30.1 and 28.1.
 constexpr int kShortLine = 2;
 template <int AXIS>
-__global__ void __launch_bounds__(128) k_dense_short(const uint16_t* __restrict__ in, int nx, int ny, int nz, int dmax,
+__global__ void __launch_bounds__(128) k_dense_short(const uint16_t* __restrict__ in, int nx, int ny, int nz, int dmax, int reach,
                                                      uint16_t* __restrict__ out16, int32_t* __restrict__ out32) {
   vdbedt::pdl_enter();
   const int64_t n = (int64_t)nx * ny * nz, stride = AXIS == 1 ? (int64_t)nx : (int64_t)nx * ny;
-  const int cap = dmax * dmax, len = AXIS == 1 ? ny : nz, reach = min(dmax, len);
+  const int cap = dmax * dmax, len = AXIS == 1 ? ny : nz;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int c = len == 1 ? 0 : (AXIS == 1 ? (int)((i / nx) % ny) : (int)(i / stride));
     int best = min((int)__ldg(in + i), cap);
@@ -135,16 +137,14 @@ __global__ void __launch_bounds__(128) k_dense_short(const uint16_t* __restrict_
 // when the square of the next offset reaches the largest minimum.  (d + k)^2 = d^2 + 2 d k + k^2: the
 // minima are kept less k^2, a multiply-add and half a three-way minimum per candidate and output.  Bound by
 // the latency of the loads at such sizes: 117 x 96 x 83, dmax 24: about 6 us each, their launches
-// overlapping the pass before (a thread per output: 14.5).  No offset reaches past the line: those of a line
-// of up to eight positions are all among themselves.
+// overlapping the pass before (a thread per output: 14.5).  reach: where the walk ends, at most dmax.
 template <int AXIS>
-__global__ void __launch_bounds__(128) k_dense_win(const uint16_t* __restrict__ in, int nx, int ny, int nz, int dmax,
+__global__ void __launch_bounds__(128) k_dense_win(const uint16_t* __restrict__ in, int nx, int ny, int nz, int dmax, int reach,
                                                    uint16_t* __restrict__ out16, int32_t* __restrict__ out32) {
   vdbedt::pdl_enter();
   const int cap = dmax * dmax, len = AXIS == 1 ? ny : nz, nb = (len + 7) / 8;
   const int64_t stride = AXIS == 1 ? (int64_t)nx : (int64_t)nx * ny;
   const int64_t n = AXIS == 1 ? (int64_t)nx * nb * nz : (int64_t)nx * ny * nb;
-  const int reach = nb == 1 ? 1 : min(dmax, len);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     int b;          // eighth of the line
     int64_t line;   // its first voxel
@@ -258,18 +258,19 @@ extern "C" vdbedt_status vdbedt_edt_dense_noalloc(const uint8_t* occ, int32_t nx
   if (nx <= 32) {
     VDB_LAUNCH(k_dense_x_narrow, blocks((nrows + 32 / nx - 1) / (32 / nx) * 32), 128, 0, st, occ, nx, nrows, dmax, g1);
   } else {
-    // stretches of four words at least, longer where the GPU is full without: few long rows (1000 x 1000 x 1)
-    // would leave it idle while a warp each works through twenty words
-    // (kMaxVoxels allows 127,100 words of rows: at most 15, with 2 x 6 of the halo below 32)
-    const int halo = (dmax + 31) / 32, words = (int)std::max<int64_t>(4, nrows * ((nx + 31) / 32) / 8192);
-    VDB_LAUNCH(k_dense_x, blocks(nrows * ((nx + 32 * words - 1) / (32 * words)) * 32), 128, 0, st, occ, nx, nrows, dmax, words,
-               halo, g1);
+    // (rows of up to four words are one stretch either way)
+    const bool few = nx > 128 && nrows * ((nx + 639) / 640) < 8192;
+    const int64_t warps = nrows * (few ? (nx + 127) / 128 : (nx + 639) / 640);
+    const auto kernel = !few ? k_dense_x<20, 6> : (dmax <= 32 ? k_dense_x<4, 1> : k_dense_x<4, 6>);
+    VDB_LAUNCH(kernel, blocks(warps * 32), 128, 0, st, occ, nx, nrows, dmax, g1);
   }
   if (cudaGetLastError() != cudaSuccess) return noalloc_fail(VDBEDT_ECUDA, "vdbedt_edt_dense_noalloc: x launch");
   const auto line = [&](auto wide, auto brief, int len, const uint16_t* in, uint16_t* out16, int32_t* out32) {
     const bool is_short = len <= kShortLine;
+    // no offset reaches past the line; eight positions or fewer are all among themselves
+    const int reach = is_short || len > 8 ? std::min((int)dmax, len) : 1;
     VDB_LAUNCH_PDL(is_short ? brief : wide, blocks(is_short ? n : n / len * ((len + 7) / 8)), 128, 0, st, in, (int)nx, (int)ny, (int)nz,
-                   (int)dmax, out16, out32);
+                   (int)dmax, reach, out16, out32);
     return cudaGetLastError();
   };
   if (line(k_dense_win<1>, k_dense_short<1>, ny, g1, g2, nullptr) != cudaSuccess)
