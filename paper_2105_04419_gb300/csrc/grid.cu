@@ -516,9 +516,14 @@ __global__ void k_alloc_obstacle_bricks(GridView g, const uint32_t* __restrict__
     int bx = 0, by = 0, bz = 0, node = -1;
     int* e = nullptr;
     bool need = false;
-    uint32_t lb = 0;
+    ulonglong2 mask[4];  // the records' bits, loaded while the node is looked up
     if (j < cnt) {
-      lb = uniq[j];
+      const uint32_t lb = uniq[j];
+      if (dbits) {
+        const ulonglong2* src = reinterpret_cast<const ulonglong2*>(dbits + (size_t)lb * 8);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mask[q] = src[q];
+      }
       bx = (int)(lb % (uint32_t)g.BX);
       int rest = (int)(lb / (uint32_t)g.BX);
       by = rest % g.BY;
@@ -531,7 +536,6 @@ __global__ void k_alloc_obstacle_bricks(GridView g, const uint32_t* __restrict__
     }
     int total = 0;
     const int slot = block_agg_add(&g.counters[C_NBRICKS], need, &total);
-    const ulonglong2* src = dbits ? reinterpret_cast<const ulonglong2*>(dbits + (size_t)lb * 8) : nullptr;
     if (need) {
       if (slot >= g.cap) {
         set_error(g, kErrOverflow);
@@ -540,7 +544,7 @@ __global__ void k_alloc_obstacle_bricks(GridView g, const uint32_t* __restrict__
           init_brick_meta(g, slot, node, bx, by, bz);
           ulonglong2* dst = reinterpret_cast<ulonglong2*>(g.occ + (size_t)slot * 8);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) dst[q] = src[q];
+          for (int q = 0; q < 4; ++q) dst[q] = mask[q];
         } else {
           init_brick(g, slot, node, bx, by, bz);
         }
@@ -550,11 +554,11 @@ __global__ void k_alloc_obstacle_bricks(GridView g, const uint32_t* __restrict__
       const int sl = *e;
       if (sl >= 0 && sl < g.cap) {
         ulonglong2* dst = reinterpret_cast<ulonglong2*>(g.occ + (size_t)sl * 8);
+        ulonglong2 old[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          ulonglong2 a = src[q], b = dst[q];
-          dst[q] = make_ulonglong2(a.x | b.x, a.y | b.y);
-        }
+        for (int q = 0; q < 4; ++q) old[q] = dst[q];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dst[q] = make_ulonglong2(mask[q].x | old[q].x, mask[q].y | old[q].y);
       }
     }
     if (threadIdx.x == 0 && total) atomicAdd(&g.counters[C_NEW_BRICKS], total);
