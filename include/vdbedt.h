@@ -131,7 +131,9 @@ typedef struct {
  * untruncated).
  * Allocates the grid's storage for cfg->max_bricks bricks (about 4.1 KB each) and cfg->max_nodes
  * interior nodes (about 19 KB each) up front; the record stage and the ingest scratch grow on
- * demand (vdbedt_set_occupancy_counted reserves them ahead).  With both capacities set, the memory
+ * demand (vdbedt_set_occupancy_counted reserves them ahead).  Where the grid has at most 4 M bricks and storage for a
+ * quarter of them, the scratch is 16 bytes per brick of the grid even for one record (64 MB at 4 M bricks).  With both
+ * capacities set, the memory
  * follows the mapped part of the grid, not its size: a grid may span up to 2^32 bricks (e.g.
  * 16384 x 16384 x 8184 voxels) with obstacles in a small part of it.  Record-driven ingest and
  * updates work at any grid size; the dense entry points and vdbedt_export_dense scale with the grid.
@@ -268,9 +270,9 @@ vdbedt_status vdbedt_clearance_backward(vdbedt_handle h, const float* pts, int64
  *            of the bulk-copy ring; 8 the envelope form of all three passes (exact, work that
  *            follows the distances instead of the window, runs of 16 bricks: the separable
  *            transform of Eq. 1 line by line).  Grids with dmax above 45 always take the envelope
- *            form.  Switching between the windowed and envelope forms changes how intermediate
- *            fields are stored, so the next vdbedt_update recomputes the whole field (as
- *            vdbedt_global).  Other values are EINVAL, and so is any call on an untruncated grid. */
+ *            form.  After a switch between the windowed and envelope forms the next vdbedt_update
+ *            recomputes the whole field (as vdbedt_global), although both store it alike.  Other
+ *            values are EINVAL, and so is any call on an untruncated grid. */
 typedef struct {
   int32_t x_run, y_run, z_run, variant;
 } vdbedt_tuning;

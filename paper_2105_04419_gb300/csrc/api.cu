@@ -924,7 +924,8 @@ vdbedt_status vdbedt_set_tuning(vdbedt_handle h, const vdbedt_tuning* t) {
   h->tune.run[1] = t->y_run ? t->y_run : d.run[1];
   h->tune.run[2] = t->z_run ? t->z_run : d.run[2];
   h->tune.variant = v ? v : d.variant;
-  // after a change of form the next update recomputes the whole field
+  // after a change of form the next update recomputes the whole field, as the header promises (the fields themselves
+  // are stored alike)
   const int windowed = (h->cfg.dmax <= 45 && h->g.R >= 1 && h->g.R <= 6 && h->tune.variant != kVariantEnvelope) ? 1 : 0;
   if (windowed != h->g.windowed) {
     h->g.windowed = windowed;

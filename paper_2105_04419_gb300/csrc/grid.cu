@@ -672,6 +672,7 @@ __global__ void k_rec_slots(US us) {
 // first kernel raises it with atomicMax, the second applies each voxel's winning record and puts
 // the entry back to -1, so vlast is all -1 between ingests.  Both run only when some record
 // clears a voxel, or when flips are tracked.
+
 // voxel index of a record inside its brick
 __device__ __forceinline__ int rec_in_brick(rec_t packed) {
   const int4 r = unpack_rec(packed);
@@ -886,7 +887,9 @@ struct DenseScratch {
 // the GPU idle while each works through eight planes in turn, so they are spread over eight warps (a
 // 64^3 map's masks 2.5 us, was 6.5); with more, a warp per plane repeats the row's bookkeeping
 // eight times with half the loads in flight (16 maps of 293 M voxels 140 us, a warp per row 65); a batch's
-// grids share the GPU and always take whole rows.
+// grids share the GPU and always take whole rows.  Around the line (whole ingest, planes spread / whole rows):
+// 625 rows 17.6 / 17.8 us, 1,024 22.1 / 18.3, 1,444 28.3 / 21.6; of ragged rows, whose loads take longer, 625
+// 22.5 / 38.7, 1,024 28.7 / 39.3, 1,444 35.9 / 45.5, 2,601 67.6 / 60.4.
 constexpr int64_t kDenseRows = 1024;
 constexpr int kDenseX = 64;
 __host__ __device__ inline int64_t dense_rows(const GridView& g) {
@@ -1880,13 +1883,13 @@ static size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 // and a compaction (few records).  Bits: in the global form, when every record sets a voxel, the
 // records' bits go to the bricks directly (many records: OR-ed into a dense scratch mask during the
 // counting pass and copied whole at allocation; few records: OR-ed per record).  Whenever a record
-// clears a voxel, or flips are tracked, each voxel's last record decides its bit through the
-// per-voxel last-record table (largest record index per voxel, then applied and reset).  With
-// tracking, each flipped voxel's brick is appended once to `changed`.
+// clears a voxel, each voxel's last record decides its bit through the per-voxel last-record table (largest
+// record index per voxel, then applied and reset).  Updates (tracked) take launch_ingest_tracked.
 //
 // Few records take the flags too where a flag per brick of the grid is small beside its storage (at least a quarter
 // of its bricks have some) and quick to clear and compact: the sort's 18 launches cost more than 4 M flags
 // (66,000 records: 35 us on a 1024 x 1024 x 256 grid, 51 us on 4 M bricks; sorted 155 and 162; one record on 64^3 21 and 83).
+// Their scratch is 16 bytes a brick of the grid however few they are, at most 64 MB beside 4 GB or more of bricks.
 constexpr int64_t kFlagBricks = (int64_t)1 << 22;
 static bool counting_ingest(const GridView& g, int64_t n) {
   const int64_t nbr_all = (int64_t)g.BX * g.BY * g.BZ;

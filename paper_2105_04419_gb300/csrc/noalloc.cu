@@ -112,8 +112,8 @@ __global__ void __launch_bounds__(128) k_dense_x_narrow(const uint8_t* __restric
 // on 666 x 1000 x 3 30.1 and 28.1.
 constexpr int kShortLine = 2;
 template <int AXIS>
-__global__ void __launch_bounds__(128) k_dense_short(const uint16_t* __restrict__ in, int nx, int ny, int nz, int dmax, int reach,
-                                                     uint16_t* __restrict__ out16, int32_t* __restrict__ out32) {
+__global__ void __launch_bounds__(128) k_dense_short(const uint16_t* __restrict__ in, int nx, int ny, int nz, int dmax,
+                                                     int reach, uint16_t* __restrict__ out16, int32_t* __restrict__ out32) {
   vdbedt::pdl_enter();
   const int64_t n = (int64_t)nx * ny * nz, stride = AXIS == 1 ? (int64_t)nx : (int64_t)nx * ny;
   const int cap = dmax * dmax, len = AXIS == 1 ? ny : nz;
@@ -269,8 +269,8 @@ extern "C" vdbedt_status vdbedt_edt_dense_noalloc(const uint8_t* occ, int32_t nx
     const bool is_short = len <= kShortLine;
     // no offset reaches past the line; eight positions or fewer are all among themselves
     const int reach = is_short || len > 8 ? std::min((int)dmax, len) : 1;
-    VDB_LAUNCH_PDL(is_short ? brief : wide, blocks(is_short ? n : n / len * ((len + 7) / 8)), 128, 0, st, in, (int)nx, (int)ny, (int)nz,
-                   (int)dmax, reach, out16, out32);
+    VDB_LAUNCH_PDL(is_short ? brief : wide, blocks(is_short ? n : n / len * ((len + 7) / 8)), 128, 0, st, in, (int)nx, (int)ny,
+                   (int)nz, (int)dmax, reach, out16, out32);
     return cudaGetLastError();
   };
   if (line(k_dense_win<1>, k_dense_short<1>, ny, g1, g2, nullptr) != cudaSuccess)

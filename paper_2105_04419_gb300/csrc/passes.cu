@@ -814,17 +814,23 @@ GridView pool_view(const GridView& g) {
 // launch): there a launch costs as much as the pass (160^3: 65.7 us a call with its export, 70.2 without).
 // A pass that fills the GPU is launched on its own: started early, its blocks take the places that the
 // previous pass's leave one by one, and y and z together took 0.82 ms where they take 0.65 (1024 x 1024 x 256
-// tunnel scene, dmax 32).
+// tunnel scene, dmax 32).  Nearer the line (transform alone, random cubes, dmax 16, chained / not): 8,000 bricks 37.8 / 44.6 us,
+// 15,625 49.1 / 56.0, 17,576 51.9 / 59.7, 32,768 72.5 / 80.5, 64,000 116 / 122 -- chaining gains 7 us on either side of it, and
+// loses only where the passes are long against that.  By capacity, which the host knows, not by the work: a map of 131,072
+// bricks that holds few gives up the same 7 us.
 constexpr int kChainBricks = 16384;
 
 // Runs of 8 bricks share their halo over twice as many outputs as runs of 4 and halve the work lists: for whole
 // transforms that fill the GPU, with halos of three bricks or more (1024 x 1024 x 256 tunnel scene: dmax 32
 // lists 22 us, x 115, y 313, z 336 with 4, 16, 107, 305, 317 with 8; dmax 24 249 and 278, 248 and 266; at dmax
-// 8 y takes 121 and 131).  Updates keep 4: their dirty runs are short.
+// 8 y takes 121 and 131).  Around the line both take the same (random cubes, dmax 32, 4 / 8: 15,625 bricks 57.5 / 58.3 us, 17,576
+// 65.5 / 67.3, 32,768 90.4 / 91.1, 64,000 146 / 144), and so do large maps that hold few bricks (48 us for 3,000 voxels).
+// Updates keep 4: their dirty runs are short.
+constexpr int kLongRunBricks = 16384;
 int effective_run(const GridView& g, const Tuning& t, int axis, bool whole) {
   if (!windowed_form(g)) return kEnvRun;
   if (t.run[axis]) return t.run[axis];
-  return whole && g.item_cap > kChainBricks && g.R >= 3 ? 8 : 4;
+  return whole && g.item_cap > kLongRunBricks && g.R >= 3 ? 8 : 4;
 }
 
 cudaError_t launch_pass(const GridView& g, const Tuning& t, int axis, const Items& it, bool chained, cudaStream_t st) {

@@ -188,7 +188,8 @@ __global__ void __launch_bounds__(128) k_query_nearest(GridView g, const int32_t
         if (near) {
           // the sphere's points in (z, y, x) order, all within one voxel on every axis
           for (int r = 0; r < 9 && !found; ++r) {
-            const int oz = z + r / 3 - 1, oy = y + r % 3 - 1, dx = D - (oz - z) * (oz - z) - (oy - y) * (oy - y);  // its own square
+            const int dz = r / 3 - 1, dy = r % 3 - 1, oz = z + dz, oy = y + dy;
+            const int dx = D - dz * dz - dy * dy;  // 0 or 1: its own square
             if ((unsigned)dx > 1u || (unsigned)oy >= (unsigned)g.ny || (unsigned)oz >= (unsigned)g.nz) continue;
             int ox = x - dx;
             found = ox >= 0 && occupied_at(g, ox, oy, oz, nc);

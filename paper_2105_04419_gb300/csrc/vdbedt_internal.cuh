@@ -436,7 +436,8 @@ cudaError_t launch_items_dirty_batch(const UpdArgs* d_args, int k, const Tuning&
 cudaError_t launch_count_run_bricks(const GridView* views, const GridView& one, const int32_t* items_ctr, int item_cap,
                                    const Tuning& t, const Items& it, cudaStream_t st);
 // Untruncated grids: store every brick (at creation), clear the occupancy (reset), take a dense
-// uint8 grid, and the transform proper (three whole-line passes; `scratch` holds 8 bytes per voxel).
+// uint8 grid, and the transform proper (three whole-line passes; `scratch`: ut_scratch_bytes, 0 and null unless ny or
+// nz exceeds the longest line that shared memory holds, then 8 bytes per voxel).
 cudaError_t launch_ut_init(const GridView& g, cudaStream_t st);
 cudaError_t launch_ut_reset(const GridView& g, cudaStream_t st);
 cudaError_t launch_ut_dense(const GridView& g, const uint8_t* grid, cudaStream_t st);
