@@ -143,3 +143,59 @@ def test_a_refused_stream_order_leaves_the_map_usable(captured):
     assert torch.equal(m.query(q).cpu(), want)
     assert np.array_equal(m.export_dense(), O.edt_factorised(occ, 8))
     m.close()
+
+
+def test_calls_inside_a_caller_s_own_capture():
+    """A caller's graph on a stream that is not the map's: the map's first kernel after each join follows a kernel, a copy
+    or nothing of the caller's, and a second stream joins between.  Replays answer as eager calls on another map."""
+    import torch
+    import paper_2105_04419_gb300 as V
+    rs = np.random.default_rng(11)
+    nx, ny, nz, n = 130, 90, 64, 400
+    occ = torch.from_numpy((rs.random((nz, ny, nx)) < 0.001).astype(np.uint8)).cuda()
+    maps = [V.Map(nx, ny, nz, 20) for _ in range(2)]
+    buf = torch.zeros((n, 3), dtype=torch.int32, device="cuda")
+    val = torch.zeros(n, dtype=torch.uint8, device="cuda")
+
+    def session(m):
+        cur, other = torch.cuda.current_stream(), torch.cuda.Stream()
+        out = [m.query(buf)]                            # nothing of the caller's before it
+        z = torch.empty_like(occ)
+        z.copy_(occ)                                    # a copy
+        m.set_occupancy_dense(z)
+        m.global_()
+        m.set_occupancy(buf + 0, val + 0)               # kernels
+        m.update()
+        out.append(m.query(buf + 0) * 2)
+        other.wait_stream(cur)
+        with torch.cuda.stream(other):
+            x = torch.clamp(buf + 1, max=nz - 1)
+            m.set_occupancy(x, 1 - val)
+            m.update()
+            near = m.query_nearest(x)
+        cur.wait_stream(other)
+        d, g = m.distance_at((x.float() * 0.1).contiguous())
+        return out + [near, d, g, m.export_dense(on_device=True)]
+
+    stream = torch.cuda.Stream()
+    for m in maps:
+        m.set_occupancy_dense(occ)
+        m.global_()
+        with torch.cuda.stream(stream):
+            session(m)
+        torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        got = session(maps[0])
+    for _ in range(8):
+        buf.copy_(torch.from_numpy(np.stack([rs.integers(0, k, n) for k in (nx, ny, nz)], 1).astype(np.int32)))
+        val.copy_(torch.from_numpy(rs.integers(0, 2, n).astype(np.uint8)))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        want = session(maps[1])
+        torch.cuda.synchronize()
+        assert [torch.equal(a, b) for a, b in zip(got, want)] == [True] * len(want)
+    del graph
+    for m in maps:
+        m.close()
